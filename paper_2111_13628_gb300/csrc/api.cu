@@ -656,11 +656,17 @@ void parallel_ranges(int64_t count, F f, int64_t per_thread = 8192) {
 // of its three literals that add the fewest distinct words to banks already used in this slot
 // (first found on ties; a lane with none left takes an inert entry). Simulated on the
 // 50,000-variable bench formula: 3.39 -> 1.98 passes per load on average (1.94 with every
-// remaining occurrence a candidate, at several times the host time). A lane's occurrences in
-// which its own literal is positive come first, those where it is negated next, so that the
-// kernel can count each kind with one bit-sliced counter outside the slots where lanes differ.
+// remaining occurrence a candidate, at several times the host time).
+//
+// Occurrences that hold a literal of the previous colour class go to the last slots of every lane
+// (from slot `pre` on), so that the kernel can count all others while that class is still being
+// updated. Of the slots before `pre`, a lane's occurrences in which its own literal is positive
+// come first, those where it is negated last, so that the kernel can count each kind with one
+// bit-sliced counter outside the slots where lanes differ; which of a lane's occurrences fill up
+// the last slots is free, and is chosen to bring the lanes' sign boundaries together.
 struct BankOrder {
-  std::vector<int32_t> pend[2][32];  // per lane: own-positive / own-negative occurrences to place
+  // per lane: own-positive / own-negative occurrences to place before `pre`, those to place after
+  std::vector<int32_t> pend[3][32];
   int32_t addr[3][32][32];           // per literal position and bank: distinct words this slot
   int32_t cnt[3][32];
 
@@ -676,23 +682,58 @@ struct BankOrder {
       if (addr[p][b][i] == w) return;
     addr[p][b][cnt[p][b]++] = w;
   }
-  // Writes the group's len x 32 entries (int4 each: sign bytes, three word byte offsets). A
-  // lane's own-positive occurrences fill its first npos slots, its own-negative ones the next.
-  void build(int32_t g0, int32_t cend, int32_t len, int32_t n, const HostVec &occ,
-             const std::vector<int32_t> &occ_ptr, const std::vector<int32_t> &orig,
-             const std::vector<int32_t> &deg, const std::vector<int32_t> &npos, int32_t *dst0) {
+  // Writes the group's len x 32 entries (int4 each: sign bytes, three word byte offsets); the
+  // previous colour class holds the new ids [prev0, prev1). Returns the slot regions (units of 4
+  // slots): own-positive in every lane below ra, own-negated in every lane from rb on, no literal
+  // of the previous class below pre, as ra | rb << 10 | pre << 20.
+  int32_t build(int32_t g0, int32_t cend, int32_t len, int32_t n, int32_t prev0, int32_t prev1,
+                const HostVec &occ, const std::vector<int32_t> &occ_ptr,
+                const std::vector<int32_t> &orig, const std::vector<int32_t> &deg, int32_t *dst0) {
     static const int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-    int32_t np[32];
+    const int32_t lit0 = 2 * prev0, lit1 = 2 * prev1;  // literals of the previous class
+    int32_t dep = 0;
     for (int32_t l = 0; l < 32; ++l) {
-      pend[0][l].clear();
-      pend[1][l].clear();
-      np[l] = 0;
+      for (int i = 0; i < 3; ++i) pend[i][l].clear();
       const int32_t v = g0 + l;
       if (v >= cend) continue;
-      np[l] = npos[orig[v]];
       for (int32_t j = 0; j < deg[orig[v]]; ++j) {
         const int32_t e = occ_ptr[v] + j;
-        pend[occ[static_cast<size_t>(e) * 4] != 0 ? 1 : 0][l].push_back(e);
+        const int32_t *q = &occ[static_cast<size_t>(e) * 4];
+        const bool d = (q[1] >= lit0 && q[1] < lit1) || (q[2] >= lit0 && q[2] < lit1) ||
+                       (q[3] >= lit0 && q[3] < lit1);
+        pend[d ? 2 : (q[0] != 0 ? 1 : 0)][l].push_back(e);
+      }
+      dep = std::max(dep, static_cast<int32_t>(pend[2][l].size()));
+    }
+    const int32_t pre = len - ((dep + 3) & ~3);
+    // a lane's sign boundary before `pre` can lie anywhere in [lo, hi]: with more occurrences than
+    // slots some move behind `pre`, with fewer there are inert entries between the two signs
+    int32_t lo[32], hi[32], top = 0, bot = pre;
+    for (int32_t l = 0; l < 32; ++l) {
+      const int32_t np = static_cast<int32_t>(pend[0][l].size()),
+                    nn = static_cast<int32_t>(pend[1][l].size());
+      lo[l] = np + nn > pre ? std::max(0, pre - nn) : np;
+      hi[l] = np + nn > pre ? std::min(np, pre) : pre - nn;
+      top = std::max(top, lo[l]);
+      bot = std::min(bot, hi[l]);
+    }
+    const int32_t aim = ((top + bot) / 2 + 2) & ~3;
+    int32_t bound[32], first_neg[32], ra = pre, rb = 0;
+    for (int32_t l = 0; l < 32; ++l) {
+      bound[l] = std::min(std::max(aim, lo[l]), hi[l]);
+      ra = std::min(ra, bound[l]);
+      rb = std::max(rb, bound[l]);
+      first_neg[l] = bound[l];
+      const int32_t np = static_cast<int32_t>(pend[0][l].size()),
+                    nn = static_cast<int32_t>(pend[1][l].size());
+      if (np + nn > pre) {  // the last of each sign move behind `pre`
+        for (int32_t k = bound[l]; k < np; ++k) pend[2][l].push_back(pend[0][l][k]);
+        for (int32_t k = pre - bound[l]; k < nn; ++k) pend[2][l].push_back(pend[1][l][k]);
+        pend[0][l].resize(bound[l]);
+        pend[1][l].resize(pre - bound[l]);
+      } else {
+        bound[l] = np;
+        first_neg[l] = pre - nn;
       }
     }
     for (int32_t j = 0; j < len; ++j) {
@@ -700,8 +741,8 @@ struct BankOrder {
         for (int b = 0; b < 32; ++b) cnt[p][b] = 0;
       for (int32_t l = 0; l < 32; ++l) {
         int32_t *dst = dst0 + (static_cast<size_t>(j) * 32 + l) * 4;
-        std::vector<int32_t> &pool = pend[j < np[l] ? 0 : 1][l];
-        if (pool.empty()) {  // inert: own sign 0, one always-true literal (word n)
+        std::vector<int32_t> &pool = pend[j >= pre ? 2 : (j < bound[l] ? 0 : 1)][l];
+        if (pool.empty() || (j < pre && j >= bound[l] && j < first_neg[l])) {  // inert: own sign 0, one always-true literal (word n)
           dst[0] = static_cast<int32_t>(1u << 15);
           dst[1] = dst[2] = dst[3] = n * 4;
           for (int p = 0; p < 3; ++p) add(p, n);
@@ -736,6 +777,7 @@ struct BankOrder {
         dst[0] = static_cast<int32_t>(signs);
       }
     }
+    return (ra / 4) | ((rb + 3) / 4) << 10 | (pre / 4) << 20;
   }
 };
 
@@ -1077,24 +1119,19 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
       grp_v0.push_back(g0);
     }
   }
-  // sign regions of every group (k <= 4): slots [0, a) hold own-positive occurrences in every
-  // lane, slots from b on none; stored as a | b << 16 after the G + 1 offsets
+  // slot regions of every group, stored after the G + 1 offsets (BankOrder::build; k > 4: only
+  // the first slot with a literal of the previous class)
   const int32_t n_groups = static_cast<int32_t>(grp_v0.size());
   grp_base.resize(static_cast<size_t>(2) * n_groups + 1, 0);
-  if (kq == 1)
-    for (int32_t c = 0; c < n_colours; ++c)
-      for (int32_t g = cgrp[c]; g < cgrp[c + 1]; ++g) {
-        int32_t lo = INT32_MAX, hi = 0;
-        for (int32_t v = grp_v0[g]; v < std::min(grp_v0[g] + 32, col_ptr[c + 1]); ++v) {
-          lo = std::min(lo, npos[orig[v]]);
-          hi = std::max(hi, npos[orig[v]]);
-        }
-        grp_base[n_groups + 1 + g] = (lo & ~3) | (((hi + 3) & ~3) << 16);
-      }
-  // the class end of every group's first variable
-  std::vector<int32_t> grp_end(grp_v0.size());
+  // of every group's class: its end, its first variable and the previous class's first variable
+  // (the first class has no previous one: a sweep starts with every word published)
+  std::vector<int32_t> grp_end(n_groups), grp_c0(n_groups), grp_prev(n_groups);
   for (int32_t c = 0; c < n_colours; ++c)
-    for (int32_t g = cgrp[c]; g < cgrp[c + 1]; ++g) grp_end[g] = col_ptr[c + 1];
+    for (int32_t g = cgrp[c]; g < cgrp[c + 1]; ++g) {
+      grp_end[g] = col_ptr[c + 1];
+      grp_c0[g] = col_ptr[c];
+      grp_prev[g] = c > 0 ? col_ptr[c - 1] : col_ptr[c];
+    }
   // every entry of every group is written below (lanes x occurrences x kq int4)
   const int64_t n_rows = grp_base[n_groups];
   HostVec occ_t(static_cast<size_t>(std::max<int64_t>(n_rows, 1)) * 4);
@@ -1105,21 +1142,39 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
       const int32_t g0 = grp_v0[g], cend = grp_end[g];
       const int32_t len = (grp_base[g + 1] - grp_base[g]) / (kq * 32);
       if (kq == 1) {
-        bo.build(g0, cend, len, n, occ, occ_ptr, orig, deg, npos,
-                 &occ_t[static_cast<size_t>(grp_base[g]) * 4]);
+        grp_base[n_groups + 1 + g] = bo.build(g0, cend, len, n, grp_prev[g], grp_c0[g], occ, occ_ptr,
+                                              orig, deg, &occ_t[static_cast<size_t>(grp_base[g]) * 4]);
         continue;
       }
       // k > 4: two int4 per occurrence (src: {own sign mask, lit1..lit7} in literal ids; inert:
       // own sign 0, literal 1 always true (word n negated), the rest always false (word n))
+      const int32_t lit0 = 2 * grp_prev[g], lit1 = 2 * grp_c0[g];
+      std::vector<int32_t> rest[32], late[32];  // occurrences without / with the previous class
+      int32_t dep = 0;
+      for (int32_t l = 0; l < 32 && g0 + l < cend; ++l) {
+        for (int32_t e = occ_ptr[g0 + l]; e < occ_ptr[g0 + l] + deg[orig[g0 + l]]; ++e) {
+          bool d = false;
+          for (int z = 1; z < slots; ++z) {
+            const int32_t u = occ[static_cast<size_t>(e) * slots + z];
+            d = d || (u >= lit0 && u < lit1);
+          }
+          (d ? late : rest)[l].push_back(e);
+        }
+        dep = std::max(dep, static_cast<int32_t>(late[l].size()));
+      }
+      const int32_t pre = len - ((dep + 3) & ~3);
+      grp_base[n_groups + 1 + g] = (pre / 4) << 20;
       for (int32_t l = 0; l < 32; ++l) {
-        const int32_t v = g0 + l;
+        size_t at = 0, lat = 0;
         for (int32_t j = 0; j < len; ++j) {
           int32_t *dst = &occ_t[(static_cast<size_t>(grp_base[g]) + j * kq * 32 + l) * 4];
           int32_t *dst2 = dst + 32 * 4;  // the occurrence's second int4, one warp row further
-          const bool real = v < cend && j < occ_ptr[v + 1] - occ_ptr[v];
-          const int32_t *src = real ? &occ[static_cast<size_t>(occ_ptr[v] + j) * slots] : nullptr;
-          auto lit = [&](int z) { return real ? src[z] : (z == 1 ? lit_true : lit_false); };
-          uint32_t signs = static_cast<uint32_t>(real && src[0] != 0) << 7;
+          int32_t e = -1;
+          if (j >= pre && lat < late[l].size()) e = late[l][lat++];
+          else if (at < rest[l].size()) e = rest[l][at++];
+          const int32_t *src = e >= 0 ? &occ[static_cast<size_t>(e) * slots] : nullptr;
+          auto lit = [&](int z) { return src ? src[z] : (z == 1 ? lit_true : lit_false); };
+          uint32_t signs = static_cast<uint32_t>(src && src[0] != 0) << 7;
           for (int z = 1; z < 4; ++z) signs |= static_cast<uint32_t>(lit(z) & 1) << (8 * z + 7);
           for (int z = 4; z < 8; ++z) signs |= static_cast<uint32_t>(lit(z) & 1) << (8 * (z - 4) + 6);
           dst[0] = static_cast<int32_t>(signs);
