@@ -129,13 +129,44 @@ __device__ __forceinline__ uint32_t sign_mask(uint32_t sg) {
   return r;
 }
 
-// Byte b (0..3) of x as a signed value: prmt replicates the byte's sign into the upper three
-// bytes (selector nibbles 8-15).
-__device__ __forceinline__ int sext_byte(uint32_t x, int b) {
-  uint32_t r;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(0u), "r"(0x8880u + 0x1111u * (uint32_t)b));
-  return (int)r;
+// Byte b (0..3) of x, zero-extended.
+__device__ __forceinline__ uint32_t byte_of(uint32_t x, int b) {
+  return __byte_perm(x, 0u, 0x4440u + (uint32_t)b);
 }
+
+// Table index of an uphill move: (b dE) >> 8 clamped to tab_len, whose entry is 0. With b at most
+// tab_len << 8 (a larger inverse temperature rejects every uphill move all the same) the product of
+// b and a byte stays below 2^32: one product, one shift, one minimum. For dE <= 0 (bytes 0 and
+// 128..255) the index is in range and meaningless: those replicas accept whatever the table says.
+__device__ __forceinline__ uint32_t table_index(uint32_t b, uint32_t de, int tab_len) {
+  return min((b * de) >> 8, (uint32_t)tab_len);
+}
+
+// Inverse temperature of a replica with multiplier m: min(2^32 - 1, (m bq) >> 16), clamped for
+// table_index.
+__device__ __forceinline__ uint32_t pt_beta(uint32_t m, uint32_t bq, int tab_len) {
+  const uint32_t lo = m * bq, hi = __umulhi(m, bq);
+  const uint32_t cap = (uint32_t)tab_len << 8;
+  return hi >> 16 ? cap : min(__funnelshift_r(lo, hi, 16), cap);
+}
+
+// The sweep's Philox rows (one per group of 4 replicas of the word), in shared memory.
+struct SweepRows {
+  uint2 vw[8];
+  uint32_t u[8];
+  __device__ __forceinline__ PhiloxRow at(int g) const {
+    const uint2 x = vw[g];
+    return PhiloxRow{u[g], x.x, x.y};
+  }
+  // written by threads 0..7 for sweep t; a barrier lies between this and the readers on both sides
+  __device__ __forceinline__ void fill(const BatchItem &B, int t) {
+    if (threadIdx.x < 8) {
+      const PhiloxRow r = philox_row((uint32_t)t, (uint32_t)(8 * B.w) + threadIdx.x, B.k0, B.k1);
+      vw[threadIdx.x] = make_uint2(r.v, r.w);
+      u[threadIdx.x] = r.u;
+    }
+  }
+};
 
 // OR over the clause's other literals of their truth values (32 replicas), from an occurrence's
 // entry: q = {sign bits, byte offsets of literals 1..3}; for k > 4 also q2 = {byte offsets of
@@ -318,13 +349,16 @@ __device__ __forceinline__ void count_slots(const uint32_t *xs, uint32_t x, Atte
   }
 }
 
-// Acceptance of variable v at sweep t for the 32 replicas of the word, from the counters of its
-// whole list; returns its new word. With PT, replica j of the word moves at min(2^32-1,
+// Acceptance of variable v at the sweep of `rows` for the 32 replicas of the word, from the counters of its
+// whole list; returns its new word. With the table index from one product, the eight-word
+// transpose and the Philox blocks from their third round on, 200 sweeps of the 50,000-variable
+// bench instance with 1,024 replicas take 41.90 ms (43.94 before), 24 uneven 3-/4-SAT sets 15.75
+// ms per 100 sweeps (16.96). With PT, replica j of the word moves at min(2^32-1,
 // (mult_s[j] * bq) >> 16) instead of bq.
 template <int KQ, bool PT>
 __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint32_t *tab_s,
-                                                 int tab_len, const uint32_t *mult_s, int v, int t,
-                                                 uint32_t x, uint32_t bqv, Counts &C,
+                                                 int tab_len, const uint32_t *mult_s,
+                                                 const SweepRows &rows, int v, uint32_t x, uint32_t bqv, Counts &C,
                                                  uint32_t (&acc)[kAccPlanes]) {
   constexpr int NB = kCountPlanes;
   uint32_t (&bc)[NB] = C.a;
@@ -349,41 +383,28 @@ __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint3
     }
     s8[NB] = br;
   }
-  const uint32_t vo = (uint32_t)__ldg(B.orig + v);
-  // (bq * dE) >> 8 in 32-bit pieces: bq = 256 hi + lo, so the index is hi dE + (lo dE) >> 8
-  // exactly (dE <= 127 keeps both terms below 2^31).
-  const uint32_t bq_hi = bqv >> 8, bq_lo = bqv & 255u;
+  const PhiloxCol col = philox_col((uint32_t)__ldg(B.orig + v), kTagKsatSweep, B.k1);
+  const uint32_t bqc = min(bqv, (uint32_t)tab_len << 8);
   // replicas whose dE <= 0 (sign plane set, or every plane zero) accept without a draw
   uint32_t flip = s8[7] | ~(s8[0] | s8[1] | s8[2] | s8[3] | s8[4] | s8[5] | s8[6]);
+  uint32_t de[8];  // byte q of de[j]: the dE of replica 8q + j
+#pragma unroll
+  for (int j = 0; j < 8; ++j) de[j] = s8[j];
+  transpose8x32(de);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     // replicas 8q .. 8q+7: Philox groups 2q and 2q+1, drawn together and always (a draw that
     // cannot change an acceptance changes nothing; a branch on whether any lane needs one rarely
     // skips the work for the whole warp and keeps the four pairs from overlapping: 236.5 -> 225.7
     // us per sweep on the 50,000-variable bench instance)
-    const unsigned long long xm = transpose8(gather_bytes(s8, q));
-    int de[8];
     uint32_t th[8];
-    const uint32_t xlo = (uint32_t)xm, xhi = (uint32_t)(xm >> 32);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      de[j] = sext_byte(j < 4 ? xlo : xhi, j & 3);
-      uint32_t hi = bq_hi, lo = bq_lo;
-      if (PT) {
-        const unsigned long long be = ((unsigned long long)mult_s[8 * q + j] * bqv) >> 16;
-        const uint32_t b = be > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)be;
-        hi = b >> 8;  // below 2^24, so hi dE stays below 2^31
-        lo = b & 255u;
-      }
-      // for dE <= 0 the index is meaningless but clamped into the table; those replicas
-      // accept whatever the comparison gives
-      const uint32_t idx = hi * (uint32_t)de[j] + ((lo * (uint32_t)de[j]) >> 8);
-      th[j] = tab_s[min(idx, (uint32_t)tab_len)];  // entry tab_len is 0
+      const uint32_t b = PT ? pt_beta(mult_s[8 * q + j], bqv, tab_len) : bqc;
+      th[j] = tab_s[table_index(b, byte_of(de[j], q), tab_len)];
     }
-    uint4 u0, u1;
-    philox4x32_10_x2(make_uint4(vo, (uint32_t)t, (uint32_t)(8 * B.w + 2 * q), kTagKsatSweep),
-                       make_uint4(vo, (uint32_t)t, (uint32_t)(8 * B.w + 2 * q + 1), kTagKsatSweep),
-                       B.k0, B.k1, u0, u1);
+    const uint4 u0 = philox4x32_meet(rows.at(2 * q), col, B.k0, B.k1);
+    const uint4 u1 = philox4x32_meet(rows.at(2 * q + 1), col, B.k0, B.k1);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const uint32_t u = j < 4 ? uint4_word(u0, j) : uint4_word(u1, j - 4);
@@ -416,8 +437,8 @@ __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint3
 template <int KQ, int TL, bool PT, bool PF = false>
 __device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint32_t *xs,
                                                  const uint32_t *tab_s, int tab_len,
-                                                 const uint32_t *mult_s, int cg, int c0, int v,
-                                                 bool active, int t, int tl,
+                                                 const uint32_t *mult_s, const SweepRows &rows,
+                                                 int cg, int c0, int v, bool active, int t, int tl,
                                                  int (&acc)[32 / TL]) {
   constexpr int NB = 7;
   const uint32_t x = active ? xs[v] : 0u;
@@ -521,8 +542,9 @@ __device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint3
     }
     d[NB] = br;
   }
-  const uint32_t vo = active ? (uint32_t)__ldg(B.orig + v) : 0u;
-  const uint32_t bq_hi = bqv >> 8, bq_lo = bqv & 255u;
+  const PhiloxCol col =
+      philox_col(active ? (uint32_t)__ldg(B.orig + v) : 0u, kTagKsatSweep, B.k1);
+  const uint32_t bqc = min(bqv, (uint32_t)tab_len << 8);
   constexpr int GPL = 8 / TL;             // Philox groups (4 replicas) per lane
   constexpr int NBK = GPL >= 2 ? GPL / 2 : 1;  // blocks of 8 replicas the lane's groups lie in
   // one 8x8 transpose of the 8 planes of D per block gives the replicas' signed bytes
@@ -530,7 +552,7 @@ __device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint3
 #pragma unroll
   for (int b = 0; b < NBK; ++b) xmb[b] = transpose8(gather_bytes(d, ((tl * GPL) >> 1) + b));
   uint32_t flip = 0u;
-  // the lane's Philox groups, drawn always and two at a time (as in attempt_batch)
+  // the lane's Philox groups, drawn always (as in accept_batch)
   int de[4 * GPL];
   uint32_t th[4 * GPL];
 #pragma unroll
@@ -541,40 +563,20 @@ __device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint3
       const int r = 4 * g + j;
       const int val = (int)(signed char)(unsigned char)(xmb[gi >> 1] >> (8 * (r & 7)));
       de[4 * gi + j] = val;
-      uint32_t hi = bq_hi, lo = bq_lo;
-      if (PT) {
-        const unsigned long long be = ((unsigned long long)mult_s[r] * bqv) >> 16;
-        const uint32_t b = be > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)be;
-        hi = b >> 8;
-        lo = b & 255u;
-      }
-      // for dE <= 0 the index is meaningless but clamped into the table; those replicas accept
-      const uint32_t idx = hi * (uint32_t)val + ((lo * (uint32_t)val) >> 8);
-      th[4 * gi + j] = tab_s[min(idx, (uint32_t)tab_len)];  // entry tab_len is 0
+      const uint32_t b = PT ? pt_beta(mult_s[r], bqv, tab_len) : bqc;
+      th[4 * gi + j] = tab_s[table_index(b, (uint32_t)val & 255u, tab_len)];
     }
   }
 #pragma unroll
-  for (int gi = 0; gi < GPL; gi += 2) {
+  for (int gi = 0; gi < GPL; ++gi) {
     const int g = tl * GPL + gi;
-    uint4 u[2];
-    if (gi + 1 < GPL) {
-      philox4x32_10_x2(make_uint4(vo, (uint32_t)t, (uint32_t)(8 * B.w + g), kTagKsatSweep),
-                       make_uint4(vo, (uint32_t)t, (uint32_t)(8 * B.w + g + 1), kTagKsatSweep),
-                       B.k0, B.k1, u[0], u[1]);
-    } else {
-      u[0] = philox4x32_10(make_uint4(vo, (uint32_t)t, (uint32_t)(8 * B.w + g), kTagKsatSweep),
-                           B.k0, B.k1);
-      u[1] = u[0];
-    }
+    const uint4 u = philox4x32_meet(rows.at(g), col, B.k0, B.k1);
 #pragma unroll
-    for (int k = 0; k < 2 && gi + k < GPL; ++k) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int i = 4 * (gi + k) + j;
-        const bool ok = de[i] <= 0 || uint4_word(u[k], j) < th[i];
-        flip |= (uint32_t)ok << (4 * (g + k) + j);
-        if (active) acc[i] += ok ? de[i] : 0;
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int i = 4 * gi + j;
+      const bool ok = de[i] <= 0 || uint4_word(u, j) < th[i];
+      flip |= (uint32_t)ok << (4 * g + j);
+      if (active) acc[i] += ok ? de[i] : 0;
     }
   }
   if (frozen) flip = 0u;  // zero counters read as dE = 0: cancel those flips
@@ -647,8 +649,9 @@ __device__ __forceinline__ T *rank_ptr(T *p, int r) {
 // replicas' energy changes to ep_s. Warps with no team in range skip the class.
 template <int KQ, int CS, int TT, bool PT>
 __device__ __forceinline__ void class_teams(const BatchItem &B, uint32_t *xs, const uint32_t *tab_s,
-                                            int tab_len, const uint32_t *mult_s, int cg, int c0,
-                                            int cnt, int rank, int t, int *ep_s) {
+                                            int tab_len, const uint32_t *mult_s,
+                                            const SweepRows &rows, int cg, int c0, int cnt,
+                                            int rank, int t, int *ep_s) {
   const int lane = threadIdx.x & 31;
   if ((int)(threadIdx.x & ~31u) / TT >= cnt) return;  // the whole warp
   const int team = threadIdx.x / TT, tl = lane % TT;
@@ -657,7 +660,8 @@ __device__ __forceinline__ void class_teams(const BatchItem &B, uint32_t *xs, co
   int tacc[32 / TT];
 #pragma unroll
   for (int i = 0; i < 32 / TT; ++i) tacc[i] = 0;
-  const uint32_t xn = attempt_team<KQ, TT, PT>(B, xs, tab_s, tab_len, mult_s, cg, c0, v, active, t, tl, tacc);
+  const uint32_t xn = attempt_team<KQ, TT, PT>(B, xs, tab_s, tab_len, mult_s, rows, cg, c0, v,
+                                                  active, t, tl, tacc);
   if (active && tl == 0) {
     if (CS == 1) {
       xs[v] = xn;
@@ -686,6 +690,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
   uint32_t *tab_s = smem + ((xs_words + 31) & ~31);  // then the acceptance table
   __shared__ int e_s[32], be_s[32], ep_s[32];
   __shared__ uint32_t mult_s[32];
+  __shared__ SweepRows rows_s;
   __shared__ uint32_t imp_s;
   __shared__ int item_s;
   __shared__ BatchItem item_b;  // the current item, read from shared memory where needed
@@ -720,6 +725,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
     // variable bench instance.
     uint32_t *best_t = B.best + (size_t)n * W + (size_t)w * n;
     uint32_t m_item = 0;  // replicas improved during this item
+    rows_s.fill(B, B.t0);
     group_sync<CS>();
     for (int t = B.t0; t < B.t1; ++t) {
       uint32_t acc[kAccPlanes];
@@ -760,11 +766,14 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
           // a smaller share (the later colour classes): teams of 8, 4 or 2 lanes per variable
           // shorten the class's critical path; their energy changes go to ep_s directly
           if (cnt <= kThreads / 8)
-            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, mult_s, cg, c0, cnt, rank, t, ep_s);
+            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt, rank, t,
+                                         ep_s);
           else if (cnt <= kThreads / 4)
-            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, mult_s, cg, c0, cnt, rank, t, ep_s);
+            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt, rank, t,
+                                         ep_s);
           else
-            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, mult_s, cg, c0, cnt, rank, t, ep_s);
+            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt, rank, t,
+                                         ep_s);
         } else {
           auto store = [&](int v, uint32_t xn) {
             if (CS == 1) {
@@ -796,7 +805,8 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
               }
               if (go) count_slots<KQ>(xs, x, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
             }
-            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, mult_s, v, t, x, P.bq, C, acc));
+            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, mult_s, rows_s, v, x, P.bq,
+                                                    C, acc));
             if (base + kThreads >= cnt) break;
           }
         }
@@ -816,19 +826,29 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         cg = cgn;
       }
       class_wait();
-      // per-replica sums of this sweep: planes -> 16-bit values (two byte transposes per block
-      // of 8 replicas), then a warp reduction per replica
+      // per-replica sums of this sweep: planes -> 16-bit values (one byte transpose for each
+      // half of the planes), then a warp reduction per replica
+      {
+        uint32_t lo[8], hi[8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const unsigned long long lo = transpose8(gather_bytes(acc, q));
-        const unsigned long long hi = transpose8(gather_bytes(acc + 8, q));
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int val = (int)(short)(unsigned short)(((lo >> (8 * i)) & 0xFFull) |
-                                                       (((hi >> (8 * i)) & 0xFFull) << 8));
-          const int s2 = __reduce_add_sync(0xFFFFFFFFu, val);
-          if (lane == 0 && s2 != 0) atomicAdd(&ep_s[8 * q + i], s2);
+        for (int j = 0; j < 8; ++j) {
+          lo[j] = acc[j];
+          hi[j] = acc[8 + j];
         }
+        transpose8x32(lo);
+        transpose8x32(hi);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            // bytes q of lo and hi as one signed 16-bit value, sign-extended
+            uint32_t val;
+            asm("prmt.b32 %0, %1, %2, %3;"
+                : "=r"(val)
+                : "r"(lo[j]), "r"(hi[j]), "r"(0xCC40u + 0x1111u * (uint32_t)q));
+            const int sum = __reduce_add_sync(0xFFFFFFFFu, (int)val);
+            if (lane == 0 && sum != 0) atomicAdd(&ep_s[8 * q + j], sum);
+          }
       }
       group_sync<CS>();
       if (rank == 0 && warp == 0) {
@@ -848,7 +868,8 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
       group_sync<CS>();
       const uint32_t m = *rank_ptr<CS>(&imp_s, 0);
       if (threadIdx.x < 32) ep_s[threadIdx.x] = 0;
-      __syncthreads();  // cleared before the next sweep's team-path adds
+      rows_s.fill(B, t + 1);
+      __syncthreads();  // cleared and filled before the next sweep's attempts
       if (m) {  // the improved replicas' states, into this word's staging row (coalesced)
         const int b0 = rank * share, b1 = min(n, b0 + share);
         for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x)
@@ -890,6 +911,7 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
   uint32_t *tab_s = smem + ((xs_words + 31) & ~31);  // then the acceptance table
   __shared__ int e_s[32], be_s[32], ep_s[32];
   __shared__ uint32_t mult_s[32];
+  __shared__ SweepRows rows_s;
   __shared__ uint32_t imp_s;
   __shared__ int item_s;
   __shared__ BatchItem item_b;
@@ -927,6 +949,7 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
     // variable bench instance.
     uint32_t *best_t = B.best + (size_t)n * W + (size_t)w * n;
     uint32_t m_item = 0;  // replicas improved during this item
+    rows_s.fill(B, B.t0);
     group_sync<CS>();
     for (int t = B.t0; t < B.t1; ++t) {
       int acc[32 / TL];
@@ -954,9 +977,8 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
           const int v = vw + (lane / TL);
           const bool active = v < v1;
           const uint32_t xn =
-              attempt_team<KQ, TL, PT, (sweep_threads<KQ, TL>() == kTeamThreads)>(B, xs, tab_s, tab_len,
-                                                                         mult_s, cg, c0, v, active,
-                                                                         t, tl, acc);
+              attempt_team<KQ, TL, PT, (sweep_threads<KQ, TL>() == kTeamThreads)>(
+                  B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, v, active, t, tl, acc);
           if (active && tl == 0) {
             if (CS == 1) {
               xs[v] = xn;
@@ -993,6 +1015,8 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
       group_sync<CS>();
       const uint32_t m = *rank_ptr<CS>(&imp_s, 0);
       if (threadIdx.x < 32) ep_s[threadIdx.x] = 0;
+      rows_s.fill(B, t + 1);
+      __syncthreads();
       if (m) {  // the improved replicas' states, into this word's staging row (coalesced)
         const int b0 = rank * share, b1 = min(n, b0 + share);
         for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x)

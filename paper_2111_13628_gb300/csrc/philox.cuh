@@ -24,25 +24,53 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
   return c;
 }
 
-// Two Philox4x32-10 blocks under one key, their rounds interleaved (the same definition as
-// philox4x32_10, twice: more independent work per thread than two calls in sequence).
-__device__ __forceinline__ void philox4x32_10_x2(uint4 a, uint4 b, uint32_t k0, uint32_t k1,
-                                                 uint4 &ua, uint4 &ub) {
+// The blocks of a sweep's attempts, counters (v, t, g, tag) for many v and few (t, g), from the
+// point where the two meet. Round 1 multiplies v and g apart and round 2 multiplies one word that
+// depends on (t, g) only and one that depends on v only, so a PhiloxRow per (t, g) and a PhiloxCol
+// per v hold everything up to there and a block starts at round 3: eight rounds instead of ten
+// and, for the eight blocks of an attempt, 40 of 320 products and 40 of 240 logic operations less.
+struct PhiloxRow {
+  uint32_t u, v, w;
+};
+struct PhiloxCol {
+  uint32_t a, y, w;
+};
+
+__device__ __forceinline__ PhiloxRow philox_row(uint32_t t, uint32_t g, uint32_t k0, uint32_t k1) {
+  const uint32_t x = __umulhi(0xCD9E8D57u, g) ^ t ^ k0;  // round 1, word 0
+  PhiloxRow r;
+  r.u = 0xCD9E8D57u * g ^ (k0 + 0x9E3779B9u);
+  r.v = __umulhi(0xD2511F53u, x) ^ (k1 + 0xBB67AE85u);
+  r.w = 0xD2511F53u * x;
+  return r;
+}
+
+__device__ __forceinline__ PhiloxCol philox_col(uint32_t v, uint32_t tag, uint32_t k1) {
+  const uint32_t z = __umulhi(0xD2511F53u, v) ^ tag ^ k1;  // round 1, word 2
+  PhiloxCol c;
+  c.a = __umulhi(0xCD9E8D57u, z);
+  c.y = 0xCD9E8D57u * z;
+  c.w = 0xD2511F53u * v;
+  return c;
+}
+
+// Rounds 3..10 of the block of (row, col): equal to philox4x32_10(make_uint4(v, t, g, tag), k0, k1).
+__device__ __forceinline__ uint4 philox4x32_meet(const PhiloxRow &r, const PhiloxCol &c, uint32_t k0,
+                                                 uint32_t k1) {
+  uint4 s = make_uint4(c.a ^ r.u, c.y, r.v ^ c.w, r.w);
+  k0 += 0x9E3779B9u;
+  k1 += 0xBB67AE85u;
 #pragma unroll
-  for (int round = 0; round < 10; ++round) {
-    if (round > 0) {
-      k0 += 0x9E3779B9u;
-      k1 += 0xBB67AE85u;
-    }
-    const uint32_t alo0 = 0xD2511F53u * a.x, ahi0 = __umulhi(0xD2511F53u, a.x);
-    const uint32_t alo1 = 0xCD9E8D57u * a.z, ahi1 = __umulhi(0xCD9E8D57u, a.z);
-    const uint32_t blo0 = 0xD2511F53u * b.x, bhi0 = __umulhi(0xD2511F53u, b.x);
-    const uint32_t blo1 = 0xCD9E8D57u * b.z, bhi1 = __umulhi(0xCD9E8D57u, b.z);
-    a = make_uint4(ahi1 ^ a.y ^ k0, alo1, ahi0 ^ a.w ^ k1, alo0);
-    b = make_uint4(bhi1 ^ b.y ^ k0, blo1, bhi0 ^ b.w ^ k1, blo0);
+  for (int round = 2; round < 10; ++round) {
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+    const uint32_t lo0 = 0xD2511F53u * s.x;
+    const uint32_t hi0 = __umulhi(0xD2511F53u, s.x);
+    const uint32_t lo1 = 0xCD9E8D57u * s.z;
+    const uint32_t hi1 = __umulhi(0xCD9E8D57u, s.z);
+    s = make_uint4(hi1 ^ s.y ^ k0, lo1, hi0 ^ s.w ^ k1, lo0);
   }
-  ua = a;
-  ub = b;
+  return s;
 }
 
 __device__ __forceinline__ uint32_t uint4_word(const uint4 &u, int j) {
