@@ -32,6 +32,7 @@ struct Instance {
   int32_t n_steps = 0;
   int users = 0;  // live replica sets
   int32_t *lbp_vptr = nullptr;   // k-SAT: variable -> clause-slot CSR for LBP (built on first use)
+  int32_t lbp_deg = 0;           // largest number of clauses of a variable (with lbp_vptr)
   int32_t *lbp_vedge = nullptr;
 };
 
@@ -96,6 +97,9 @@ struct nmc_ctx {
   // launches share the SMs (the second fills those the first's tail leaves idle)
   cudaStream_t kaux = nullptr;
   cudaEvent_t kfork = nullptr, kjoin = nullptr;
+  // LBP: pinned read-back of the running seeds and its events (created on first use)
+  int32_t *lbp_seen = nullptr;
+  cudaEvent_t lbp_ev[2] = {};
   // tuned batched-sweep shapes: (occurrence width, largest n, work items) -> (cs, lanes)
   std::map<std::tuple<int, int, int>, std::pair<int, int>> tune;
 };
@@ -556,6 +560,9 @@ void nmc_destroy(nmc_ctx *ctx) {
   }
   if (ctx->kfork) cudaEventDestroy(ctx->kfork);
   if (ctx->kjoin) cudaEventDestroy(ctx->kjoin);
+  if (ctx->lbp_seen) cudaFreeHost(ctx->lbp_seen);
+  for (cudaEvent_t ev : ctx->lbp_ev)
+    if (ev) cudaEventDestroy(ev);
   for (auto &kv : ctx->sets) free_set(kv.second);
   for (auto &kv : ctx->insts) free_instance(kv.second);
   dev_free(ctx->tab);
@@ -2001,7 +2008,10 @@ int ensure_lbp_graph(nmc_ctx *ctx, Instance &I) {
   std::vector<int32_t> vptr(static_cast<size_t>(n) + 1, 0), vedge;
   for (size_t e = 0; e < slots; ++e)
     if (cl[e] < 2 * n) vptr[(cl[e] >> 1) + 1]++;
-  for (int32_t v = 0; v < n; ++v) vptr[v + 1] += vptr[v];
+  for (int32_t v = 0; v < n; ++v) {
+    I.lbp_deg = std::max(I.lbp_deg, vptr[v + 1]);
+    vptr[v + 1] += vptr[v];
+  }
   vedge.resize(static_cast<size_t>(vptr[n]) + 1);
   std::vector<int32_t> fill(vptr.begin(), vptr.end() - 1);
   for (size_t e = 0; e < slots; ++e)
@@ -2282,6 +2292,22 @@ int nmc_cnf_lbp(nmc_ctx *ctx, int32_t inst, int32_t n_seeds, const uint8_t *x_st
   A.lambdas = lambdas;
   A.beta = beta;
   A.tol = tol;
+  double lam_max = 0.0, eps_max = I->lbp_deg;  // without eps: the number of clauses
+  for (int32_t k = 0; k < n_lambda; ++k) lam_max = std::max(lam_max, std::fabs(lambdas[k]));
+  if (eps) {
+    eps_max = 0.0;
+    for (int32_t i = 0; i < n; ++i) eps_max = std::max(eps_max, std::fabs(eps[i]));
+  }
+  A.max_deg = I->lbp_deg;
+  A.max_bias = lam_max * eps_max;
+  if (!ctx->lbp_seen)
+    NMC_CUDA(cudaMallocHost(reinterpret_cast<void **>(&ctx->lbp_seen), 2 * sizeof(int32_t)),
+             "allocate LBP read-back");
+  for (cudaEvent_t &ev : ctx->lbp_ev)
+    if (!ev) NMC_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "create LBP event");
+  A.seen = ctx->lbp_seen;
+  A.ev[0] = ctx->lbp_ev[0];
+  A.ev[1] = ctx->lbp_ev[1];
   A.scratch = scratch;
   A.marg = marg;
   A.corr = corr;

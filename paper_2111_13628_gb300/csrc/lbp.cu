@@ -12,6 +12,14 @@
 // Frames: spin r = 2x - 1; literal i of clause a is satisfied by sigma_ai (+1 positive, -1
 // negated). h_{i->a} = sigma_ai (lambda eps_i s*_i + sum_{b != a} sigma_bi u_{b->i});
 // u_{a->i} = -1/2 ln[1 - (1 - e^{-2 beta}) prod_{j != i} (1 - tanh h_{j->a}) / 2].
+//
+// Two forms of the same iteration. The product form keeps w = e^{-2u} and E = e^{2h} instead of u
+// and h: sums of u become products of w, (1 - tanh h) / 2 is 1 / (1 + E), and an iteration needs
+// neither exponentials nor logarithms (9 double-precision instructions per message instead of 82;
+// the log form was bound by them, 85% of the pipe). It is used whenever no e^{2 field} can leave
+// the range of a double and the tolerance is above the resolution of w; the log form runs otherwise.
+// 4-SAT, 5,000 variables, 64 seeds: clause pass 1,924 -> 140 us, a call with its backbones 120 -> 34
+// ms; 500 variables, 5 seeds: 5.9 -> 2.8 ms.
 #include <math.h>
 
 #include "nmc_internal.h"
@@ -110,6 +118,252 @@ __global__ void lbp_var_kernel(const int32_t *__restrict__ vptr, const int32_t *
       h[e * S + s] = sg * (field - sg * u[e * S + s]);
     }
   }
+}
+
+// ---- product form -----------------------------------------------------------------------------
+
+// Largest 1 + E a clause product takes: with it the K factors of a clause stay below 2^1000. A
+// larger one (a literal false with probability below 2^-125) changes no w.
+template <int K>
+__device__ __forceinline__ double cut_factor(double d) {
+  constexpr int kHi = (1023 + 1000 / K) << 20;  // high word of 2^(1000 / K)
+  return __double2hiint(d) >= kHi ? __hiloint2double(kHi, 0) : d;
+}
+
+// |x| to 20 bits as a float, for |x| < 2^128 (0 below 2^-126), with integer operations only.
+__device__ __forceinline__ float approx_abs(double x) {
+  const int h = (__double2hiint(x) & 0x7FFFFFFF) - (896 << 20);
+  return h <= 0 ? 0.0f : __int_as_float(h << 3);
+}
+
+// E of every edge at the first lambda (G = e^{2 lambda eps s*} per variable and seed).
+__global__ void lbp_init_prod_kernel(const int32_t *__restrict__ clits, long long n_edges, int32_t n,
+                                     int32_t S, const double *__restrict__ G, double *E) {
+  const long long total = n_edges * S;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int l = clits[i / S];
+    if (l >= 2 * n) continue;
+    const double g = G[(size_t)(l >> 1) * S + i % S];
+    E[i] = (l & 1) ? 1.0 / g : g;
+  }
+}
+
+// G[v][s] = e^{2 lambda eps_v s*_{v,s}}.
+__global__ void lbp_gain_kernel(const double *__restrict__ eps, const uint8_t *__restrict__ xs,
+                                int32_t n, int32_t S, double lambda, double *G) {
+  const long long total = (long long)n * S;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x)
+    G[i] = exp(2.0 * lambda * eps[i / S] * (2.0 * (double)xs[i] - 1.0));
+}
+
+// |ln(w / old)| with chg = w - old: the series where it is short enough, else log1p.
+__device__ __forceinline__ double log_change(double chg, double old) {
+  const double r = chg / old;
+  if (fabs(r) < 1e-4) return fabs(r * fma(r, fma(r, fma(r, -0.25, 1.0 / 3.0), -0.5), 1.0));
+  return fabs(log1p(r));
+}
+
+// Clause pass: w = 1 - c prod_{j != i} 1 / (1 + E_j) of every literal, from one division by the
+// product of all K factors. The largest change of u per seed, |ln(w / w_old)| / 2, is found in two steps:
+// single precision picks the edges that can hold the maximum (relative error below 2e-5, margin
+// twice that), and only those are evaluated in double precision, usually one per thread. The
+// recorded maximum does not depend on which thread comes first: an edge is passed over only when
+// a larger value is already recorded.
+// Bound by the double-precision pipe (2 lanes per cycle and SM): 27 instructions a clause and seed.
+template <int K>
+__global__ void lbp_clause_prod_kernel(const int32_t *__restrict__ clits, int32_t m, int32_t n,
+                                       int32_t S, const double *__restrict__ E, double *w, double c,
+                                       const int32_t *__restrict__ status, unsigned long long *dmax,
+                                       int track) {
+  const long long total = (long long)m * S;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long a = i / S;
+    const int s = (int)(i - a * S);
+    if (status && status[s] != kRunning) continue;
+    const size_t e0 = (size_t)(a * K) * S + s;
+    double d[K], old[K];
+    bool used[K];
+    double all = 1.0;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      used[q] = clits[a * K + q] < 2 * n;
+      d[q] = used[q] ? cut_factor<K>(1.0 + E[e0 + (size_t)q * S]) : 1.0;
+      old[q] = used[q] && track ? w[e0 + (size_t)q * S] : 1.0;
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q) all *= d[q];
+    const double r = 1.0 / all;
+    double chg[K], chg_top = 0.0, old_top = 1.0;
+    float est[K], top = 0.0f;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      const double wn = fma(-c, d[q] * r, 1.0);
+      if (used[q]) w[e0 + (size_t)q * S] = wn;
+      chg[q] = used[q] ? wn - old[q] : 0.0;
+      est[q] = 0.0f;
+      if (track) {
+        const float x = __fdividef(approx_abs(chg[q]), approx_abs(old[q]));
+        est[q] = fabsf(log1pf(__double2hiint(chg[q]) < 0 ? -x : x));
+        if (est[q] > top) {
+          top = est[q];
+          chg_top = chg[q];
+          old_top = old[q];
+        }
+      }
+    }
+    if (!track || top == 0.0f) continue;
+    const float seen = approx_abs(__longlong_as_double((long long)*(volatile unsigned long long *)&dmax[s]));
+    if (0.5f * top * (1.0f + 4e-5f) < seen) continue;
+    double dm = log_change(chg_top, old_top);
+    const float tie = top * (1.0f - 4e-5f);
+    int ties = 0;
+#pragma unroll
+    for (int q = 0; q < K; ++q) ties += est[q] >= tie;
+    if (ties > 1) {  // another edge may hold the larger change
+#pragma unroll
+      for (int q = 0; q < K; ++q)
+        if (est[q] >= tie) dm = fmax(dm, log_change(chg[q], old[q]));
+    }
+    if (dm > 0.0) atomicMax(&dmax[s], (unsigned long long)__double_as_longlong(0.5 * dm));
+  }
+}
+
+// Products of w over the positive and the negated edges p0, p0 + step, ... of a variable for seed s.
+__device__ __forceinline__ void edge_products(const int32_t *vedge, const int32_t *clits, int p0,
+                                              int p1, int step, int S, int s, const double *w,
+                                              double &pp, double &pn) {
+  pp = pn = 1.0;
+#pragma unroll 4
+  for (int p = p0; p < p1; p += step) {
+    const long long e = vedge[p];
+    const double x = w[e * S + s];
+    if (clits[e] & 1) pn *= x;
+    else pp *= x;
+  }
+}
+
+// Variable pass: e^{2 field} = G prod_neg w / prod_pos w, and E = e^{+-2 field} w of each edge
+// (the cavity takes the edge's own message out again). LANES consecutive lanes share a variable
+// and seed and split its edges: one where there are enough of them to fill the GPU (coalesced over
+// seeds), eight where a single lane's chain of loads and products would be the time (5 seeds of a
+// 500-variable formula).
+template <int LANES>
+__global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int32_t *__restrict__ vedge,
+                                    const int32_t *__restrict__ clits, int32_t n, int32_t S,
+                                    const double *__restrict__ G, const double *__restrict__ w,
+                                    double *E, const int32_t *__restrict__ status) {
+  const long long total = (long long)n * S;
+  const int sub = threadIdx.x % LANES;
+  // whole teams run the same iterations (blockDim is a multiple of LANES)
+  for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / LANES; i < total;
+       i += (long long)gridDim.x * blockDim.x / LANES) {
+    const int v = (int)(i / S), s = (int)(i - (long long)v * S);
+    if (status[s] != kRunning) continue;
+    const int p0 = vptr[v], p1 = vptr[v + 1];
+    double pp, pn;
+    edge_products(vedge, clits, p0 + sub, p1, LANES, S, s, w, pp, pn);
+    if (LANES > 1) {
+      const unsigned team = ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) - sub);
+#pragma unroll
+      for (int o = LANES / 2; o > 0; o >>= 1) {
+        pp *= __shfl_xor_sync(team, pp, o);
+        pn *= __shfl_xor_sync(team, pn, o);
+      }
+    }
+    pn *= G[i];
+    const double x = pn / pp, xi = pp / pn;
+#pragma unroll 4
+    for (int p = p0 + sub; p < p1; p += LANES) {
+      const long long e = vedge[p];
+      E[e * S + s] = ((clits[e] & 1) ? xi : x) * w[e * S + s];
+    }
+  }
+}
+
+// Marginals <r_v> = tanh field = (a - b) / (a + b), a / b = e^{2 field}, each seed at its own
+// lambda. Written as 1 - 2 b / (a + b) or its mirror image, whichever term is the small one.
+__global__ void lbp_marg_prod_kernel(const int32_t *__restrict__ vptr, const int32_t *__restrict__ vedge,
+                                     const int32_t *__restrict__ clits,
+                                     const int32_t *__restrict__ orig, int32_t n, int32_t S,
+                                     const double *__restrict__ eps, const uint8_t *__restrict__ xs,
+                                     const double *__restrict__ lambdas,
+                                     const int32_t *__restrict__ lam_idx,
+                                     const double *__restrict__ w, double *marg) {
+  const long long total = (long long)n * S;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int v = (int)(i / S), s = (int)(i - (long long)v * S);
+    double pp, pn;
+    edge_products(vedge, clits, vptr[v], vptr[v + 1], 1, S, s, w, pp, pn);
+    pn *= exp(2.0 * lambdas[lam_idx[s]] * eps[v] * (2.0 * (double)xs[i] - 1.0));
+    marg[(size_t)s * n + orig[v]] =
+        pn >= pp ? fma(-2.0, pp / (pn + pp), 1.0) : fma(2.0, pn / (pn + pp), -1.0);
+  }
+}
+
+// (p, q1) of one seed per block, in a fixed summation order.
+__global__ void lbp_overlap_kernel(const int32_t *__restrict__ orig, int32_t n, int32_t S,
+                                   const uint8_t *__restrict__ xs, const double *__restrict__ marg,
+                                   double *overlap) {
+  const int s = blockIdx.x;
+  __shared__ double sp[kLbpBlock], sq[kLbpBlock];
+  double p = 0.0, q = 0.0;
+  for (int v = threadIdx.x; v < n; v += blockDim.x) {
+    const double mv = marg[(size_t)s * n + orig[v]];
+    p += (2.0 * (double)xs[(size_t)v * S + s] - 1.0) * mv;
+    q += mv * mv;
+  }
+  sp[threadIdx.x] = p;
+  sq[threadIdx.x] = q;
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      sp[threadIdx.x] += sp[threadIdx.x + o];
+      sq[threadIdx.x] += sq[threadIdx.x + o];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    overlap[2 * s] = sp[0] / n;
+    overlap[2 * s + 1] = sq[0] / n;
+  }
+}
+
+// Clause correlations as lbp_corr_kernel, from f = 1 / (1 + E) = (1 - t) / 2; t = 1 - 2 f or
+// 2 E f - 1, whichever has the small product.
+__global__ void lbp_corr_prod_kernel(const int32_t *__restrict__ clits, int32_t m, int32_t kmax,
+                                     int32_t n, int32_t S, const double *__restrict__ E, double c,
+                                     double *corr) {
+  const long long total = (long long)m * S;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long a = i / S;
+    const int s = (int)(i - a * S);
+    double free_prod = 1.0, viol_prod = 1.0, sign = 1.0;
+    int k = 0;
+    for (int q = 0; q < kmax; ++q) {
+      const long long e = a * kmax + q;
+      const int l = clits[e];
+      if (l >= 2 * n) continue;
+      const double sg = lit_sigma(l), x = E[e * S + s], f = 1.0 / (1.0 + x);
+      free_prod *= sg * (x >= 1.0 ? fma(-2.0, f, 1.0) : fma(2.0 * x, f, -1.0));
+      viol_prod *= f;
+      sign *= -sg;
+      ++k;
+    }
+    const double z = 1.0 - c * viol_prod;
+    corr[(size_t)s * m + a] = k > 0 ? (free_prod - c * sign * viol_prod) / z : 0.0;
+  }
+}
+
+template <int K>
+void clause_prod(const int32_t *clits, int32_t m, int32_t n, int32_t S, const double *E, double *w,
+                 double c, const int32_t *status, unsigned long long *dmax, int track,
+                 unsigned grid, cudaStream_t st) {
+  lbp_clause_prod_kernel<K><<<grid, kLbpBlock, 0, st>>>(clits, m, n, S, E, w, c, status, dmax, track);
 }
 
 // Per seed after an iteration at lambda index k: count, convergence, failure, bookkeeping.
@@ -302,40 +556,83 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
   LBP_CHECK(cudaMemsetAsync(u, 0, sizeof(double) * E * S, st));
   LBP_CHECK(cudaMemcpyAsync(lam_dev, A.lambdas, sizeof(double) * L, cudaMemcpyHostToDevice, st));
   const unsigned gS = (unsigned)((S + kLbpBlock - 1) / kLbpBlock);
+  const unsigned gVS = blocks_for((long long)n * S), gMS = blocks_for((long long)m * S),
+                 gES = blocks_for(E * S);
+  // the product form needs every product of w and every e^{2 field} inside the range of a double:
+  // u lies in [0, beta], so |field| <= beta deg + |lambda eps|. w is resolved to about 1e-16, a
+  // change of u to 1e-16 e^{2 beta} / 2: smaller tolerances take the log form, whose resolution is
+  // the same for large u but finer for small ones
+  const bool prod = A.beta <= 4.0 && A.beta * A.max_deg + A.max_bias < 340.0 &&
+                    A.tol >= 2e-15 * exp(2.0 * A.beta);
+  const bool split = (long long)n * S < 152 * 256;  // fewer than eight warps an SM otherwise
+  const auto clause = [&](const int32_t *seeds, int track) {
+    if (!prod) {
+      lbp_clause_kernel<<<gMS, kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, u, c, seeds, dmax, track);
+      return;
+    }
+    switch (kmax) {
+#define LBP_CASE(k) \
+  case k: clause_prod<k>(A.clits, m, n, S, h, u, c, seeds, dmax, track, gMS, st); break;
+      LBP_CASE(1) LBP_CASE(2) LBP_CASE(3) LBP_CASE(4)
+      LBP_CASE(5) LBP_CASE(6) LBP_CASE(7) LBP_CASE(8)
+#undef LBP_CASE
+    }
+  };
+  const auto bias_at = [&](double lambda) {
+    if (prod) lbp_gain_kernel<<<gVS, kLbpBlock, 0, st>>>(A.eps, A.xs, n, S, lambda, bias);
+    else lbp_bias_kernel<<<gVS, kLbpBlock, 0, st>>>(A.eps, A.xs, n, S, lambda, bias);
+  };
   // initial messages at lambda_0: h from the bias, u from those h
-  lbp_bias_kernel<<<blocks_for((long long)n * S), kLbpBlock, 0, st>>>(A.eps, A.xs, n, S, A.lambdas[0], bias);
-  lbp_init_h_kernel<<<blocks_for(E * S), kLbpBlock, 0, st>>>(A.clits, E, n, S, bias, h);
-  lbp_clause_kernel<<<blocks_for((long long)m * S), kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, u, c,
-                                                                     nullptr, dmax, 0);
+  bias_at(A.lambdas[0]);
+  if (prod) lbp_init_prod_kernel<<<gES, kLbpBlock, 0, st>>>(A.clits, E, n, S, bias, h);
+  else lbp_init_h_kernel<<<gES, kLbpBlock, 0, st>>>(A.clits, E, n, S, bias, h);
+  clause(nullptr, 0);
   LBP_CHECK(cudaGetLastError());
   for (int32_t k = 0; k < L; ++k) {
     if (k > 0) {
       lbp_advance_kernel<<<gS, kLbpBlock, 0, st>>>(S, k, L, status);
-      lbp_bias_kernel<<<blocks_for((long long)n * S), kLbpBlock, 0, st>>>(A.eps, A.xs, n, S, A.lambdas[k], bias);
+      bias_at(A.lambdas[k]);
     }
+    // One iteration is always queued behind the one whose outcome the host reads: once no seed is
+    // running the queued one changes nothing (every kernel leaves seeds that are not running
+    // alone), and the GPU does not wait for the host in between.
     for (int32_t it = 0; it < A.max_iter; ++it) {
-      lbp_var_kernel<<<blocks_for((long long)n * S), kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, n, S,
-                                                                       bias, u, h, status);
-      lbp_clause_kernel<<<blocks_for((long long)m * S), kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, u,
-                                                                         c, status, dmax, 1);
+      if (prod && split)
+        lbp_var_prod_kernel<8><<<blocks_for(8LL * n * S), kLbpBlock, 0, st>>>(
+            A.vptr, A.vedge, A.clits, n, S, bias, u, h, status);
+      else if (prod)
+        lbp_var_prod_kernel<1><<<gVS, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, n, S, bias, u, h,
+                                                          status);
+      else
+        lbp_var_kernel<<<gVS, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, n, S, bias, u, h, status);
+      clause(status, 1);
       LBP_CHECK(cudaMemsetAsync(running, 0, sizeof(int32_t), st));
       lbp_control_kernel<<<gS, kLbpBlock, 0, st>>>(S, k, L, A.tol, A.max_iter, status, A.iters,
                                                    A.deltas, A.n_done, lam_idx, copy_flag, dmax,
                                                    running);
-      lbp_copy_kernel<<<blocks_for(E * S), kLbpBlock, 0, st>>>(E, S, copy_flag, h, u, hg, ug);
-      lbp_clear_flags_kernel<<<gS, kLbpBlock, 0, st>>>(S, copy_flag);
       LBP_CHECK(cudaGetLastError());
-      int32_t run_h = 0;
-      LBP_CHECK(cudaMemcpyAsync(&run_h, running, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      LBP_CHECK(cudaStreamSynchronize(st));
-      if (run_h == 0) break;
+      LBP_CHECK(cudaMemcpyAsync(A.seen + (it & 1), running, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+      LBP_CHECK(cudaEventRecord(A.ev[it & 1], st));
+      if (it == 0) continue;
+      LBP_CHECK(cudaEventSynchronize(A.ev[(it - 1) & 1]));
+      if (A.seen[(it - 1) & 1] == 0) break;
     }
+    // seeds that converged or gave up at this lambda stopped changing: snapshots once, at its end
+    lbp_copy_kernel<<<gES, kLbpBlock, 0, st>>>(E, S, copy_flag, h, u, hg, ug);
+    lbp_clear_flags_kernel<<<gS, kLbpBlock, 0, st>>>(S, copy_flag);
+    LBP_CHECK(cudaGetLastError());
   }
   lbp_advance_kernel<<<gS, kLbpBlock, 0, st>>>(S, L, L, status);
-  lbp_marg_kernel<<<S, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, A.orig, n, S, A.eps, A.xs,
-                                          lam_dev, lam_idx, u, A.marg, A.overlap);
-  lbp_corr_kernel<<<blocks_for((long long)m * S), kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, c,
-                                                                   A.corr);
+  if (prod) {
+    lbp_marg_prod_kernel<<<gVS, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, A.orig, n, S, A.eps,
+                                                    A.xs, lam_dev, lam_idx, u, A.marg);
+    lbp_overlap_kernel<<<S, kLbpBlock, 0, st>>>(A.orig, n, S, A.xs, A.marg, A.overlap);
+    lbp_corr_prod_kernel<<<gMS, kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, c, A.corr);
+  } else {
+    lbp_marg_kernel<<<S, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, A.orig, n, S, A.eps, A.xs,
+                                            lam_dev, lam_idx, u, A.marg, A.overlap);
+    lbp_corr_kernel<<<gMS, kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, c, A.corr);
+  }
   LBP_CHECK(cudaGetLastError());
 #undef LBP_CHECK
   return 0;

@@ -250,6 +250,10 @@ struct LbpArgs {
   const uint8_t *xs;      // device [n][S] seeds (0/1), new order, seed fastest
   const double *lambdas;  // host [n_lambda]
   double beta, tol;
+  double max_deg;         // largest number of clauses of a variable
+  double max_bias;        // largest |lambda eps|
+  int32_t *seen;          // pinned host [2]: seeds still running after the last two iterations
+  cudaEvent_t ev[2];      // recorded after each of those two read-backs
   void *scratch;          // lbp_scratch_bytes
   double *marg;           // device out [S][n], original order
   double *corr;           // device out [S][m]
@@ -262,8 +266,8 @@ size_t lbp_scratch_bytes(int32_t n, int32_t m, int32_t kmax, int32_t S, int32_t 
 cudaError_t lbp_prepare(const uint8_t *x_in, const double *eps_in, const int32_t *orig,
                         const int32_t *vptr, int32_t n, int32_t S, uint8_t *xs, double *eps,
                         cudaStream_t st);
-// Runs the continuation; returns 0 or a cudaError_t value. Synchronises the stream once per
-// iteration (to see whether any seed is still iterating).
+// Runs the continuation; returns 0 or a cudaError_t value. Reads back once per iteration, one
+// iteration behind, whether any seed is still iterating.
 int lbp_run(const LbpArgs &A, cudaStream_t st);
 
 struct BackboneArgs {
