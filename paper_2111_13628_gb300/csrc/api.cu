@@ -1399,6 +1399,7 @@ int nmc_load_qap(nmc_ctx *ctx, int32_t n, const int32_t *F, const int32_t *D, in
   I.kind = NMC_KIND_QAP;
   I.n_units = n;
   I.qp.n = n;
+  I.qp.narrow = *std::max_element(f.begin(), f.end()) <= 127 && *std::max_element(d.begin(), d.end()) <= 127;
   cudaError_t e = cudaSuccess;
   if ((e = dev_alloc(&I.qp.F, f.size())) != cudaSuccess ||
       (e = dev_alloc(&I.qp.D, d.size())) != cudaSuccess ||

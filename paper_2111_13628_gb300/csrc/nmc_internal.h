@@ -74,6 +74,7 @@ struct KsatReplicas {
 struct QapDevice {
   int32_t n;
   uint8_t *F, *D;  // n*n, entries 0..255
+  bool narrow;     // every entry is at most 127
 };
 
 struct QapReplicas {
@@ -310,6 +311,7 @@ struct QapArgs {
   const uint32_t *mult;  // replica exchange: Q16 temperature multiplier of each replica, or null
   double *stats;         // energy statistics [2][R] (running sums of E and E^2), or null
   int32_t stats_t0;      // first step whose end-of-step cost enters stats
+  int32_t narrow;        // entries of F and D at most 127
 };
 
 QapArgs qap_block_args(const QapDevice &I, QapReplicas &Rp, const uint32_t *bq, const uint32_t *tab,

@@ -11,9 +11,13 @@
 // chunks of CHB = 4, 8 or 16 bytes (a lane's facilities, zero padded), so a lane reads its part
 // of a row with one aligned load. The swap change
 //   dC(r,s) = 2 sum_{k != r,s} (F_rk - F_sk)(D_{p(s)p(k)} - D_{p(r)p(k)})
-// is an O(n) dot product split over the replica's lanes: the gathered D bytes are packed four
-// to a word and the byte products F_r D_s + F_s D_r - F_r D_r - F_s D_s are summed with dp4a,
-// then over the lanes. The Philox blocks of LPR consecutive attempts of each replica are drawn
+// is an O(n) dot product split over the replica's lanes. Entries up to 127 (the narrow form): the
+// lanes first write the row difference D_{p(s).} - D_{p(r).} as signed bytes to a row of the
+// replica's own, then each gathers its facilities' bytes from it, packs them four to a word and
+// sums their products with F_r - F_s by dp4a. Larger entries (their differences need nine bits):
+// both D rows are gathered and the four byte products F_r D_s + F_s D_r - F_r D_r - F_s D_s are
+// summed. The narrow form has half the random byte loads, which the shared-memory pipe was 75 %
+// busy with, half the packing and a quarter of the dp4a. Then the sums over the lanes. The Philox blocks of LPR consecutive attempts of each replica are drawn
 // in parallel, one per lane, and broadcast in turn.
 #include "nmc_internal.h"
 #include "philox.cuh"
@@ -34,15 +38,6 @@ __device__ __forceinline__ void put(int (&p)[NPL], int i, int v) {
     if (q == i) p[q] = v;
 }
 
-template <int NPL>
-__device__ __forceinline__ int pick(const int (&p)[NPL], int i) {
-  int v = p[0];
-#pragma unroll
-  for (int q = 1; q < NPL; ++q)
-    if (q == i) v = p[q];
-  return v;
-}
-
 // Shared-memory layout of F: row r at r * LDF, as LPR lane chunks of CHB bytes; facility k
 // sits in chunk k / NPL at byte k % NPL (padding bytes zero).
 template <int NPL, int LPR>
@@ -57,13 +52,32 @@ __device__ __forceinline__ uint32_t pack4(uint32_t b0, uint32_t b1, uint32_t b2,
   return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
 }
 
+// Differences a - b of four bytes, each at most 127, as signed bytes.
+__device__ __forceinline__ uint32_t sub4(uint32_t a, uint32_t b) {
+  return ((a | 0x80808080u) - b) ^ 0x80808080u;
+}
+
+// N words from a 4 N-byte aligned address of shared memory.
+template <int N>
+__device__ __forceinline__ void load_words(const uint8_t *p, uint32_t (&w)[N]) {
+  if constexpr (N == 4) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(p);
+    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+  } else if constexpr (N == 2) {
+    const uint2 v = *reinterpret_cast<const uint2 *>(p);
+    w[0] = v.x; w[1] = v.y;
+  } else {
+    w[0] = *reinterpret_cast<const uint32_t *>(p);
+  }
+}
+
 // Cost of the permutation ps with the whole warp: sum_i sum_j F_ij D_{p(i)p(j)}. The warp's
 // 32 / LPR lane groups take rows i in turn; lane l of a group reads its chunk of F row i and the
 // bytes D_{p(i)p(k)} of its facilities k = NPL l + q, four to a word, and sums the products with
 // dp4a (a row's partial sum stays below 2^22).
 template <int NPL, int LPR>
-__device__ long long warp_cost(const uint8_t *Fs, const uint8_t *Ds, const uint8_t *ps, int n,
-                               int lane) {
+__device__ long long warp_cost(const uint8_t *Fs, const uint8_t *Ds, int ldd, const uint8_t *ps,
+                               int n, int lane) {
   constexpr int CHB = FLayout<NPL, LPR>::CHB, LDF = FLayout<NPL, LPR>::LDF, RPW = 32 / LPR;
   const int hl = lane % LPR;
   int pk[NPL];
@@ -74,7 +88,7 @@ __device__ long long warp_cost(const uint8_t *Fs, const uint8_t *Ds, const uint8
   }
   long long acc = 0;
   for (int i = lane / LPR; i < n; i += RPW) {
-    const uint8_t *Drow = Ds + ps[i] * n;
+    const uint8_t *Drow = Ds + ps[i] * ldd;
     const uint32_t *Fw = reinterpret_cast<const uint32_t *>(Fs + i * LDF + CHB * hl);
     uint32_t row = 0u;
 #pragma unroll
@@ -98,8 +112,8 @@ __device__ long long warp_cost(const uint8_t *Fs, const uint8_t *Ds, const uint8
 // identity, position q = n-1..1 exchanged with (u (q+1)) >> 32, or a copy of the given state),
 // then its cost and the global copies. Whole warp.
 template <int NPL, int LPR>
-__device__ void qap_init_one(const QapArgs &a, const uint8_t *Fs, const uint8_t *Ds, uint8_t *ps,
-                             int r, int lane) {
+__device__ void qap_init_one(const QapArgs &a, const uint8_t *Fs, const uint8_t *Ds, int ldd,
+                             uint8_t *ps, int r, int lane) {
   const int n = a.n;
   int16_t *gp = a.perm + (size_t)r * n;
   if (a.init_mode == 1) {
@@ -127,7 +141,7 @@ __device__ void qap_init_one(const QapArgs &a, const uint8_t *Fs, const uint8_t 
     for (int k = lane; k < n; k += 32) ps[k] = (uint8_t)gp[k];
     __syncwarp();
   }
-  const long long c = warp_cost<NPL, LPR>(Fs, Ds, ps, n, lane);
+  const long long c = warp_cost<NPL, LPR>(Fs, Ds, ldd, ps, n, lane);
   const bool set_best = a.init_mode != 3;
   for (int k = lane; k < n; k += 32) {
     gp[k] = (int16_t)ps[k];
@@ -142,7 +156,7 @@ __device__ void qap_init_one(const QapArgs &a, const uint8_t *Fs, const uint8_t 
 
 // A CTA runs the 32 replicas of one block: lane group h = lane / LPR of warp w runs replica
 // 32 block + RPW w + h, its lane l = lane % LPR owning facilities NPL l + i.
-template <int NPL, int LPR>
+template <int NPL, int LPR, bool NARROW>
 __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
   constexpr int RPW = 32 / LPR;  // replicas per warp
   extern __shared__ __align__(16) uint32_t smem[];
@@ -151,27 +165,37 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
   uint32_t *tab_s = smem;
   uint8_t *Fs = (uint8_t *)(smem + ((a.tab_len + 31) & ~31));
   uint8_t *Ds = Fs + ((n * LDF + 15) & ~15);
-  uint8_t *pw_all = Ds + ((n * n + 15) & ~15);  // one n-byte row per replica (permutation copy)
+  const int ldd = NARROW ? LDF : n;  // the narrow form reads D rows in lane chunks
+  uint8_t *pw_all = Ds + ((n * ldd + 15) & ~15);  // one n-byte row per replica (permutation copy)
   const int pstride = (n + 15) & ~15;
+  uint8_t *diff_all = pw_all + 32 * pstride;  // NARROW: one LDF-byte row per replica
   for (int i = threadIdx.x; i < a.tab_len; i += blockDim.x) tab_s[i] = a.tab[i];
   for (int i = threadIdx.x; i < n * LDF; i += blockDim.x) {
     const int row = i / LDF, col = i % LDF, j = col % CHB, k = NPL * (col / CHB) + j;
     Fs[i] = (j < NPL && k < n) ? a.F[row * n + k] : (uint8_t)0;
   }
-  for (int i = threadIdx.x; i < n * n; i += blockDim.x) Ds[i] = a.D[i];
+  if (NARROW) {
+    for (int i = threadIdx.x; i < n * LDF; i += blockDim.x) {
+      const int row = i / LDF, col = i % LDF;
+      Ds[i] = col < n ? a.D[row * n + col] : (uint8_t)0;
+    }
+  } else {
+    for (int i = threadIdx.x; i < n * n; i += blockDim.x) Ds[i] = a.D[i];
+  }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r0 = block * 32 + RPW * warp;  // the warp's first replica
   if (r0 >= a.R) return;                   // the whole warp
   if (a.init_mode != 0) {
     for (int h = 0; h < RPW && r0 + h < a.R; ++h)
-      qap_init_one<NPL, LPR>(a, Fs, Ds, pw_all + (RPW * warp + h) * pstride, r0 + h, lane);
+      qap_init_one<NPL, LPR>(a, Fs, Ds, ldd, pw_all + (RPW * warp + h) * pstride, r0 + h, lane);
     return;
   }
   const int half = lane / LPR, hl = lane % LPR;
   const int r = r0 + half;
   const bool live = r < a.R;  // the second half of the last warp may have no replica
   uint8_t *pw = pw_all + (RPW * warp + half) * pstride;
+  uint8_t *diff = diff_all + (RPW * warp + half) * LDF;
   const int16_t *gp = a.perm + (size_t)(live ? r : r0) * n;
   for (int k = hl; k < n; k += LPR) pw[k] = live ? (uint8_t)gp[k] : (uint8_t)0;
   __syncwarp();
@@ -220,57 +244,66 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
           const bool held = (pj >> 18) != 0;
           if (__all_sync(0xFFFFFFFFu, held)) continue;  // every replica of the warp held
           const int rr = pj & 511, ss = (pj >> 9) & 511;
-          int pr, ps;
-          if constexpr (LPR == 32) {  // from the owning lanes' registers
-            pr = __shfl_sync(0xFFFFFFFFu, pick<NPL>(p, rr % NPL), rr / NPL);
-            ps = __shfl_sync(0xFFFFFFFFu, pick<NPL>(p, ss % NPL), ss / NPL);
-          } else {  // from the shared-memory copy
-            pr = pw[rr];
-            ps = pw[ss];
-          }
-          const uint8_t *Dr = Ds + pr * n, *Dsr = Ds + ps * n;
+          const int pr = pw[rr], ps = pw[ss];
+          const uint8_t *Dr = Ds + pr * ldd, *Dsr = Ds + ps * ldd;
           // this lane's chunks of rows r and s of F
           uint32_t fr4[CHB / 4], fs4[CHB / 4];
-          if constexpr (CHB == 16) {
-            const uint4 a4 = *reinterpret_cast<const uint4 *>(Fs + rr * LDF + 16 * hl);
-            const uint4 b4 = *reinterpret_cast<const uint4 *>(Fs + ss * LDF + 16 * hl);
-            fr4[0] = a4.x; fr4[1] = a4.y; fr4[2] = a4.z; fr4[3] = a4.w;
-            fs4[0] = b4.x; fs4[1] = b4.y; fs4[2] = b4.z; fs4[3] = b4.w;
-          } else if constexpr (CHB == 8) {
-            const uint2 a2 = *reinterpret_cast<const uint2 *>(Fs + rr * LDF + 8 * hl);
-            const uint2 b2 = *reinterpret_cast<const uint2 *>(Fs + ss * LDF + 8 * hl);
-            fr4[0] = a2.x; fr4[1] = a2.y;
-            fs4[0] = b2.x; fs4[1] = b2.y;
-          } else {
-            fr4[0] = *reinterpret_cast<const uint32_t *>(Fs + rr * LDF + 4 * hl);
-            fs4[0] = *reinterpret_cast<const uint32_t *>(Fs + ss * LDF + 4 * hl);
-          }
+          load_words<CHB / 4>(Fs + rr * LDF + CHB * hl, fr4);
+          load_words<CHB / 4>(Fs + ss * LDF + CHB * hl, fs4);
           // sum over every k (padding bytes of F are zero); the k = r and k = s terms sum to
-          // -2 F_rs D_{p(r)p(s)} by symmetry and are added back below. Positive and negative
-          // products are summed apart (unsigned, below 2^22) and subtracted at the end.
-          uint32_t accp = 0u, accn = 0u;
+          // -2 F_rs D_{p(r)p(s)} by symmetry and are added back below
+          int acc = 0;
+          if constexpr (NARROW) {
+            uint32_t dr4[CHB / 4], ds4[CHB / 4];
+            load_words<CHB / 4>(Dr + CHB * hl, dr4);
+            load_words<CHB / 4>(Dsr + CHB * hl, ds4);
 #pragma unroll
-          for (int w4 = 0; w4 < CHB / 4; ++w4) {
-            uint32_t dr[4], dsb[4];
+            for (int w4 = 0; w4 < CHB / 4; ++w4) dr4[w4] = sub4(ds4[w4], dr4[w4]);
+            if constexpr (CHB == 16)
+              *reinterpret_cast<uint4 *>(diff + 16 * hl) = make_uint4(dr4[0], dr4[1], dr4[2], dr4[3]);
+            else if constexpr (CHB == 8)
+              *reinterpret_cast<uint2 *>(diff + 8 * hl) = make_uint2(dr4[0], dr4[1]);
+            else
+              *reinterpret_cast<uint32_t *>(diff + 4 * hl) = dr4[0];
+            __syncwarp();  // the row is complete; the end of the attempt orders its next writes
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int i = 4 * w4 + q;
-              dr[q] = i < NPL ? (uint32_t)Dr[p[i < NPL ? i : 0]] : 0u;
-              dsb[q] = i < NPL ? (uint32_t)Dsr[p[i < NPL ? i : 0]] : 0u;
+            for (int w4 = 0; w4 < CHB / 4; ++w4) {
+              uint32_t g[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int i = 4 * w4 + q;
+                g[q] = i < NPL ? (uint32_t)diff[p[i < NPL ? i : 0]] : 0u;
+              }
+              acc = __dp4a((int)sub4(fr4[w4], fs4[w4]), (int)pack4(g[0], g[1], g[2], g[3]), acc);
             }
-            const uint32_t wr = pack4(dr[0], dr[1], dr[2], dr[3]);
-            const uint32_t wsv = pack4(dsb[0], dsb[1], dsb[2], dsb[3]);
-            accp = __dp4a(fr4[w4], wsv, accp);
-            accp = __dp4a(fs4[w4], wr, accp);
-            accn = __dp4a(fr4[w4], wr, accn);
-            accn = __dp4a(fs4[w4], wsv, accn);
+          } else {
+            // positive and negative products are summed apart (unsigned, below 2^22)
+            uint32_t accp = 0u, accn = 0u;
+#pragma unroll
+            for (int w4 = 0; w4 < CHB / 4; ++w4) {
+              uint32_t dr[4], dsb[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int i = 4 * w4 + q;
+                dr[q] = i < NPL ? (uint32_t)Dr[p[i < NPL ? i : 0]] : 0u;
+                dsb[q] = i < NPL ? (uint32_t)Dsr[p[i < NPL ? i : 0]] : 0u;
+              }
+              const uint32_t wr = pack4(dr[0], dr[1], dr[2], dr[3]);
+              const uint32_t wsv = pack4(dsb[0], dsb[1], dsb[2], dsb[3]);
+              accp = __dp4a(fr4[w4], wsv, accp);
+              accp = __dp4a(fs4[w4], wr, accp);
+              accn = __dp4a(fr4[w4], wr, accn);
+              accn = __dp4a(fs4[w4], wsv, accn);
+            }
+            acc = (int)(accp - accn);
           }
-          int acc = (int)(accp - accn);
           if constexpr (LPR == 32) {
             acc = __reduce_add_sync(0xFFFFFFFFu, acc);
           } else {
-#pragma unroll
-            for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+            // the two replicas' sums as two whole-warp reductions side by side
+            const int lo = __reduce_add_sync(0xFFFFFFFFu, half == 0 ? acc : 0);
+            const int hi = __reduce_add_sync(0xFFFFFFFFu, half == 0 ? 0 : acc);
+            acc = half == 0 ? lo : hi;
           }
           acc += 2 * (int)Fs[FLayout<NPL, LPR>::at(rr, ss)] * (int)Dr[ps];  // |sum| < 2^24: exact
           const long long d = 2LL * acc;
@@ -297,13 +330,13 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
           if (ok) {
             if (hl == rr / NPL) put<NPL>(p, rr % NPL, ps);
             if (hl == ss / NPL) put<NPL>(p, ss % NPL, pr);
-            if (LPR < 32 && hl == 0) {
+            if (hl == 0) {
               pw[rr] = (uint8_t)ps;
               pw[ss] = (uint8_t)pr;
             }
             e += d;
           }
-          if (LPR < 32) __syncwarp();  // the row update is seen by the next attempt
+          __syncwarp();  // the row updates are seen by the next attempt
         }
       }
     }
@@ -338,16 +371,24 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
   }
 }
 
+// Facilities per lane from which the narrow form is used: its row exchange costs more than it
+// saves for one or two gathers a lane (4 sets of 4,096 replicas, wide -> narrow: n = 16 677 -> 736
+// us per 40 steps, n = 64 1,460 -> 1,467 per 20, n = 96 2,705 -> 2,445, n = 128 4,129 -> 3,300,
+// n = 192 4,979 -> 4,331 per 10, n = 256 7,435 -> 6,033).
+constexpr int kNarrowNpl = 3;
+
 template <int NPL, int LPR>
-__global__ void __launch_bounds__(qap_threads<LPR>()) qap_kernel(QapArgs a) {
-  qap_body<NPL, LPR>(a, blockIdx.x);
+__global__ void __launch_bounds__(qap_threads<LPR>(), LPR == 16 ? 2 : 1) qap_kernel(QapArgs a) {
+  if (NPL >= kNarrowNpl && a.narrow) qap_body<NPL, LPR, NPL >= kNarrowNpl>(a, blockIdx.x);
+  else qap_body<NPL, LPR, false>(a, blockIdx.x);
 }
 
 // Batched QAP: CTA b runs replica block items[b].block of the replica set items[b] describes.
 template <int NPL, int LPR>
-__global__ void __launch_bounds__(qap_threads<LPR>()) qap_batch_kernel(const QapArgs *items) {
+__global__ void __launch_bounds__(qap_threads<LPR>(), LPR == 16 ? 2 : 1) qap_batch_kernel(const QapArgs *items) {
   const QapArgs a = items[blockIdx.x];
-  qap_body<NPL, LPR>(a, a.block);
+  if (NPL >= kNarrowNpl && a.narrow) qap_body<NPL, LPR, NPL >= kNarrowNpl>(a, a.block);
+  else qap_body<NPL, LPR, false>(a, a.block);
 }
 
 // Shape parameters: NPL and LPR of shape q.
@@ -357,8 +398,9 @@ __host__ __device__ constexpr int shape_lpr(int q) { return q < 8 ? 16 : 32; }
 size_t qap_smem_shape(int n, int q, int tab_len) {
   const int npl = shape_npl(q);
   const int ldf = shape_lpr(q) * (npl <= 4 ? 4 : (npl <= 8 ? 8 : 16));  // FLayout::LDF
-  return sizeof(uint32_t) * ((tab_len + 31) & ~31) + (size_t)((n * ldf + 15) & ~15) +
-         (size_t)((n * n + 15) & ~15) + (size_t)32 * ((n + 15) & ~15);
+  // the narrow form's layout, the larger one (ldf >= n, and its difference rows)
+  return sizeof(uint32_t) * ((tab_len + 31) & ~31) + 2 * (size_t)((n * ldf + 15) & ~15) +
+         (size_t)32 * ((n + 15) & ~15) + (size_t)32 * ldf;
 }
 
 template <int Q>
@@ -419,6 +461,7 @@ QapArgs make_args(const QapDevice &I, QapReplicas &Rp, uint64_t seed) {
   a.k1 = (uint32_t)(seed >> 32);
   a.init_mode = 0;
   a.block = -1;
+  a.narrow = I.narrow ? 1 : 0;
   a.mult = nullptr;
   a.stats = nullptr;
   a.stats_t0 = 0;
