@@ -1304,6 +1304,15 @@ int qap_batch_enqueue(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int
   std::vector<QapArgs> by_npl[kQapShapes];
   int max_n[kQapShapes] = {0};
   std::map<int32_t, int> seen;
+  double load = 0.0;  // of the sets that run
+  for (int32_t i = 0; i < n_sets; ++i) {
+    ReplicaSet *S = find_set(ctx, rs[i]);
+    const Instance *I = S ? find_inst(ctx, S->inst) : nullptr;
+    if (I && I->kind == NMC_KIND_QAP && t1[i] > t0[i]) load += qap_load(I->qp.n, S->R);
+  }
+  int rpb[kQapShapes];
+  for (int q = 0; q < kQapShapes; ++q)
+    rpb[q] = qap_replicas_per_block(load, qap_lanes(q), ctx->device);
   for (int32_t i = 0; i < n_sets; ++i) {
     ReplicaSet *S = find_set(ctx, rs[i]);
     if (!S) return fail(ctx, NMC_EINVAL, "unknown replica set in batch");
@@ -1316,9 +1325,9 @@ int qap_batch_enqueue(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int
     if (t1[i] == t0[i]) continue;
     const int n = I->qp.n;
     const int q = qap_shape(n);
-    for (int b = 0; b < (S->R + 31) / 32; ++b)
+    for (int b = 0; b < (S->R + rpb[q] - 1) / rpb[q]; ++b)
       by_npl[q].push_back(qap_block_args(I->qp, S->qp, I->bq, ctx->tab, ctx->tab_len, t0[i], t1[i],
-                                         S->seed, b));
+                                         S->seed, rpb[q], b));
     max_n[q] = std::max(max_n[q], n);
   }
   size_t total = 0;
@@ -1355,7 +1364,7 @@ int qap_batch_enqueue(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int
   for (int q = 0; q < kQapShapes && err == cudaSuccess; ++q) {
     if (by_npl[q].empty()) continue;
     if ((err = cudaStreamWaitEvent(ctx->qaux[q], ctx->qfork, 0)) != cudaSuccess) break;
-    err = qap_batch(ctx->qitems + off[q], static_cast<int>(by_npl[q].size()), q, max_n[q],
+    err = qap_batch(ctx->qitems + off[q], static_cast<int>(by_npl[q].size()), q, rpb[q], max_n[q],
                     ctx->tab_len, ctx->qaux[q]);
     const cudaError_t e2 = cudaEventRecord(ctx->qjoin[q], ctx->qaux[q]);
     if (e2 == cudaSuccess) *joins |= 1u << q;  // launched (or failed): joined all the same
@@ -1850,7 +1859,9 @@ int nmc_replicas_run_pt(nmc_ctx *ctx, int32_t rs, int32_t t0, int32_t t1,
     // QAP: per segment one batched launch of the set's 32-replica blocks (with the
     // multipliers), then the exchange round on the 64-bit costs
     const int32_t Lq = S->pt_L, Gq = S->R / Lq, perq = sweeps_per_round;
-    const int32_t nblk = (S->R + 31) / 32, n = I->qp.n, shape = qap_shape(n);
+    const int32_t n = I->qp.n, shape = qap_shape(n);
+    const int rpb = qap_replicas_per_block(qap_load(n, S->R), qap_lanes(shape), ctx->device);
+    const int32_t nblk = (S->R + rpb - 1) / rpb;
     int32_t t = t0;
     std::vector<QapArgs> qitems;
     std::vector<int32_t> ends;
@@ -1862,7 +1873,7 @@ int nmc_replicas_run_pt(nmc_ctx *ctx, int32_t rs, int32_t t0, int32_t t1,
         const int64_t te = std::min<int64_t>(t1, (static_cast<int64_t>(t) / perq + 1) * perq);
         for (int32_t b = 0; b < nblk; ++b) {
           QapArgs a = qap_block_args(I->qp, S->qp, I->bq, ctx->tab, ctx->tab_len, t,
-                                     static_cast<int32_t>(te), S->seed, b);
+                                     static_cast<int32_t>(te), S->seed, rpb, b);
           a.mult = S->pt_mult;
           qitems.push_back(a);
         }
@@ -1880,7 +1891,7 @@ int nmc_replicas_run_pt(nmc_ctx *ctx, int32_t rs, int32_t t0, int32_t t1,
                                cudaMemcpyHostToDevice, ctx->stream),
                "upload QAP work list");
       for (size_t i = 0; i < ends.size(); ++i) {
-        NMC_CUDA(qap_batch(ctx->qitems + i * nblk, nblk, shape, n, ctx->tab_len, ctx->stream),
+        NMC_CUDA(qap_batch(ctx->qitems + i * nblk, nblk, shape, rpb, n, ctx->tab_len, ctx->stream),
                  "launch QAP steps");
         if (ends[i] % perq == 0)
           NMC_CUDA(pt_exchange64(S->pt_lq, Lq, Gq, reinterpret_cast<const long long *>(S->qp.energy),
@@ -2049,13 +2060,15 @@ struct DevScratch {
 };
 
 // The adaptive ladder on a QAP replica set S (fresh, Philox initial states): level i runs steps
-// [i T, (i+1) T) of every 32-replica block in one batched launch at the constant schedule beta_i,
+// [i T, (i+1) T) of every replica block in one batched launch at the constant schedule beta_i,
 // with per-replica double sums of the costs of the last sweeps_meas steps, then the one-thread
 // ladder step.
 int qap_ladder(nmc_ctx *ctx, const Instance &I, ReplicaSet &S, double beta0, double alpha,
                       double sigma_min, int32_t max_temps, int32_t sweeps_eq, int32_t sweeps_meas,
                       double *betas_out, double *sigmas_out, int32_t *n_temps_out) {
-  const int32_t n = I.qp.n, R = S.R, nblk = (R + 31) / 32, shape = qap_shape(n);
+  const int32_t n = I.qp.n, R = S.R, shape = qap_shape(n);
+  const int rpb = qap_replicas_per_block(qap_load(n, R), qap_lanes(shape), ctx->device);
+  const int32_t nblk = (R + rpb - 1) / rpb;
   const int64_t T = static_cast<int64_t>(sweeps_eq) + sweeps_meas;
   uint32_t *bq = nullptr;
   double *stats = nullptr, *out_dev = nullptr;
@@ -2091,7 +2104,7 @@ int qap_ladder(nmc_ctx *ctx, const Instance &I, ReplicaSet &S, double beta0, dou
     const uint32_t *base = reinterpret_cast<const uint32_t *>(
         reinterpret_cast<uintptr_t>(bq) - sizeof(uint32_t) * static_cast<size_t>(ts) * n);
     for (int32_t b = 0; b < nblk; ++b) {
-      items[b] = qap_block_args(I.qp, S.qp, base, ctx->tab, ctx->tab_len, ts, te, S.seed, b);
+      items[b] = qap_block_args(I.qp, S.qp, base, ctx->tab, ctx->tab_len, ts, te, S.seed, rpb, b);
       items[b].stats = stats;
       items[b].stats_t0 = ts + sweeps_eq;
     }
@@ -2100,7 +2113,7 @@ int qap_ladder(nmc_ctx *ctx, const Instance &I, ReplicaSet &S, double beta0, dou
         (e = cudaMemsetAsync(stats, 0, sizeof(double) * 2 * R, ctx->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(ctx->qitems, items.data(), sizeof(QapArgs) * nblk, cudaMemcpyHostToDevice,
                              ctx->stream)) != cudaSuccess ||
-        (e = qap_batch(ctx->qitems, nblk, shape, n, ctx->tab_len, ctx->stream)) != cudaSuccess ||
+        (e = qap_batch(ctx->qitems, nblk, shape, rpb, n, ctx->tab_len, ctx->stream)) != cudaSuccess ||
         (e = ladder_step_f64(stats, R, static_cast<long long>(R) * sweeps_meas, beta, alpha, out_dev,
                              ctx->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(out, out_dev, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream)) != cudaSuccess ||

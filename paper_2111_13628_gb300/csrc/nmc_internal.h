@@ -307,19 +307,26 @@ struct QapArgs {
   int32_t tab_len, n, R, t0, t1;
   uint32_t k0, k1;
   int init_mode;  // 0: run steps; 1: draw initial states (Fisher-Yates); 2: states given
-  int block;      // batched launches: replica block (32 replicas) this CTA runs; else -1
+  int block;      // batched launches: replica block (rpb replicas) this CTA runs; else -1
   const uint32_t *mult;  // replica exchange: Q16 temperature multiplier of each replica, or null
   double *stats;         // energy statistics [2][R] (running sums of E and E^2), or null
   int32_t stats_t0;      // first step whose end-of-step cost enters stats
   int32_t narrow;        // entries of F and D at most 127
+  int32_t rpb;           // replicas per block, at most 32 (a whole number of warps)
 };
 
 QapArgs qap_block_args(const QapDevice &I, QapReplicas &Rp, const uint32_t *bq, const uint32_t *tab,
-                       int32_t tab_len, int32_t t0, int32_t t1, uint64_t seed, int block);
+                       int32_t tab_len, int32_t t0, int32_t t1, uint64_t seed, int rpb,
+                       int block);
 // Launch shape of the QAP kernels for an instance of n facilities: 0..kQapShapes-1 (lanes per
 // replica and facilities per lane); a batched launch takes items of one shape.
 constexpr int kQapShapes = 12;
 int qap_shape(int n);
+int qap_lanes(int shape);  // lanes per replica
+// Replicas per block for a launch (or launches side by side) of `load` SMs' worth of full blocks, the
+// sum of qap_load over its replica sets; lanes: qap_lanes of the launch's shape.
+double qap_load(int32_t n, int32_t R);
+int qap_replicas_per_block(double load, int lanes, int device);
 // The batched QAP launches of these sets (as nmc_qap_batch_run does them), each launch shape on
 // an auxiliary stream forked from the context's stream after the work-list upload; *joins gets
 // the streams to join. qap_batch_join makes the context's stream wait for them; call it also
@@ -328,8 +335,8 @@ int qap_batch_enqueue(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int
                       const int32_t *t1, uint32_t *joins);
 int qap_batch_join(nmc_ctx *ctx, uint32_t joins);
 // Runs n_blocks QAP replica blocks (items_dev[b] for CTA b) in one launch; every item has
-// qap_shape(n) == shape, and max_n (the largest n) sizes the shared memory.
-cudaError_t qap_batch(const QapArgs *items_dev, int n_blocks, int shape, int max_n, int tab_len,
+// qap_shape(n) == shape and the given rpb, and max_n (the largest n) sizes the shared memory.
+cudaError_t qap_batch(const QapArgs *items_dev, int n_blocks, int shape, int rpb, int max_n, int tab_len,
                       cudaStream_t st);
 // (older single-set launchers below) ------------------------------------------------------------
 // Initial permutations (Fisher-Yates from Philox, or init_dev [R][n]) with their costs; with

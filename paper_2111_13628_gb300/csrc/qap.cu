@@ -19,6 +19,9 @@
 // summed. The narrow form has half the random byte loads, which the shared-memory pipe was 75 %
 // busy with, half the packing and a quarter of the dp4a. Then the sums over the lanes. The Philox blocks of LPR consecutive attempts of each replica are drawn
 // in parallel, one per lane, and broadcast in turn.
+#include <algorithm>
+#include <cmath>
+
 #include "nmc_internal.h"
 #include "philox.cuh"
 
@@ -29,7 +32,7 @@ namespace {
 // Launch shapes: shape q < 8 runs n <= 16 (q + 1) with LPR = 16; shape 8 + q runs
 // n <= 32 (q + 5) with LPR = 32.
 template <int LPR>
-constexpr int qap_threads() { return 32 * 32 / (32 / LPR); }  // 32 replicas per CTA
+constexpr int qap_threads() { return 32 * LPR; }  // at most 32 replicas per CTA
 
 template <int NPL>
 __device__ __forceinline__ void put(int (&p)[NPL], int i, int v) {
@@ -154,8 +157,13 @@ __device__ void qap_init_one(const QapArgs &a, const uint8_t *Fs, const uint8_t 
   __syncwarp();
 }
 
-// A CTA runs the 32 replicas of one block: lane group h = lane / LPR of warp w runs replica
-// 32 block + RPW w + h, its lane l = lane % LPR owning facilities NPL l + i.
+// A byte of shared memory by its 32-bit address.
+__device__ __forceinline__ uint32_t shared_byte(uint32_t addr) {
+  return *static_cast<const uint8_t *>(__cvta_shared_to_generic(addr));
+}
+
+// A CTA runs the a.rpb (at most 32) replicas of one block: lane group h = lane / LPR of warp w runs
+// replica rpb block + RPW w + h, its lane l = lane % LPR owning facilities NPL l + i.
 template <int NPL, int LPR, bool NARROW>
 __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
   constexpr int RPW = 32 / LPR;  // replicas per warp
@@ -184,8 +192,8 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r0 = block * 32 + RPW * warp;  // the warp's first replica
-  if (r0 >= a.R) return;                   // the whole warp
+  const int r0 = block * a.rpb + RPW * warp;  // the warp's first replica
+  if (r0 >= a.R) return;                      // the whole warp
   if (a.init_mode != 0) {
     for (int h = 0; h < RPW && r0 + h < a.R; ++h)
       qap_init_one<NPL, LPR>(a, Fs, Ds, ldd, pw_all + (RPW * warp + h) * pstride, r0 + h, lane);
@@ -199,11 +207,14 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
   const int16_t *gp = a.perm + (size_t)(live ? r : r0) * n;
   for (int k = hl; k < n; k += LPR) pw[k] = live ? (uint8_t)gp[k] : (uint8_t)0;
   __syncwarp();
-  int p[NPL];  // padding facilities (k >= n) sit at location 0; their F entries are zero
+  // Locations of the lane's facilities; padding facilities (k >= n) sit at location 0, their F
+  // entries are zero. NARROW: as shared addresses of their bytes in the difference row.
+  const int off = NARROW ? (int)(uint32_t)__cvta_generic_to_shared(diff) : 0;
+  int p[NPL];
 #pragma unroll
   for (int i = 0; i < NPL; ++i) {
     const int k = NPL * hl + i;
-    p[i] = k < n ? pw[k] : 0;
+    p[i] = off + (k < n ? pw[k] : 0);
   }
   long long e = live ? a.energy[r] : 0;
   long long be = live ? a.best_energy[r] : 0;
@@ -222,7 +233,7 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
       for (int a0 = 0; a0 < n; a0 += LPR) {
         // lane l of each replica draws its attempt a0 + l
         const int at = a0 + hl;
-        int fr = 0, fs = 0, frz = live ? 0 : 1;  // no replica: every attempt rejected
+        int fr = 0, fs = 0, frs = 0, frz = live ? 0 : 1;  // no replica: every attempt rejected
         uint32_t u2 = 0u, bqs = 0u;
         if (at < n && live) {
           const uint4 u =
@@ -234,16 +245,18 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
           const uint32_t br = __ldg(bqt + fr), bs = __ldg(bqt + fs);
           frz = (br == kFrozenQ16 || bs == kFrozenQ16) ? 1 : 0;  // a held facility: reject
           bqs = (uint32_t)(((unsigned long long)br + bs) >> 1);
+          frs = Fs[FLayout<NPL, LPR>::at(fr, fs)];
         }
         const int cnt = (n - a0) < LPR ? (n - a0) : LPR;
-        // r, s (< 256 each) and the held flag of every lane's attempt in one word: one
+        // r, s and F_rs (a byte each) and the held flag of every lane's attempt in one word: one
         // broadcast per attempt within each replica's lanes
-        const int packed = fr | (fs << 9) | (frz << 18);
+        const int packed = fr | (fs << 8) | (frs << 16) | (frz << 24);
+        const bool any_held = __any_sync(0xFFFFFFFFu, frz);
         for (int j = 0; j < cnt; ++j) {
           const int pj = __shfl_sync(0xFFFFFFFFu, packed, j, LPR);
-          const bool held = (pj >> 18) != 0;
-          if (__all_sync(0xFFFFFFFFu, held)) continue;  // every replica of the warp held
-          const int rr = pj & 511, ss = (pj >> 9) & 511;
+          const bool held = (pj >> 24) != 0;
+          if (any_held && __all_sync(0xFFFFFFFFu, held)) continue;  // every replica of the warp held
+          const int rr = pj & 255, ss = (pj >> 8) & 255;
           const int pr = pw[rr], ps = pw[ss];
           const uint8_t *Dr = Ds + pr * ldd, *Dsr = Ds + ps * ldd;
           // this lane's chunks of rows r and s of F
@@ -272,7 +285,7 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
                 const int i = 4 * w4 + q;
-                g[q] = i < NPL ? (uint32_t)diff[p[i < NPL ? i : 0]] : 0u;
+                g[q] = i < NPL ? shared_byte((uint32_t)p[i < NPL ? i : 0]) : 0u;
               }
               acc = __dp4a((int)sub4(fr4[w4], fs4[w4]), (int)pack4(g[0], g[1], g[2], g[3]), acc);
             }
@@ -305,8 +318,8 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
             const int hi = __reduce_add_sync(0xFFFFFFFFu, half == 0 ? 0 : acc);
             acc = half == 0 ? lo : hi;
           }
-          acc += 2 * (int)Fs[FLayout<NPL, LPR>::at(rr, ss)] * (int)Dr[ps];  // |sum| < 2^24: exact
-          const long long d = 2LL * acc;
+          acc += 2 * ((pj >> 16) & 255) * (int)Dr[ps];
+          const int d = 2 * acc;  // |acc| < 2^25
           // the draw and pair temperature of the attempt: with two replicas per warp fetched
           // always (the uphill test below may diverge between them)
           uint32_t bj = 0u, uj = 0u;
@@ -324,12 +337,12 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
               const unsigned long long be2 = (mr * bj) >> 16;
               bj = be2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)be2;
             }
-            const unsigned long long idx = ((unsigned long long)bj * (unsigned long long)d) >> 8;
+            const unsigned long long idx = ((unsigned long long)bj * (uint32_t)d) >> 8;
             ok = idx < (unsigned long long)a.tab_len && uj < tab_s[idx];
           }
           if (ok) {
-            if (hl == rr / NPL) put<NPL>(p, rr % NPL, ps);
-            if (hl == ss / NPL) put<NPL>(p, ss % NPL, pr);
+            if (hl == rr / NPL) put<NPL>(p, rr % NPL, off + ps);
+            if (hl == ss / NPL) put<NPL>(p, ss % NPL, off + pr);
             if (hl == 0) {
               pw[rr] = (uint8_t)ps;
               pw[ss] = (uint8_t)pr;
@@ -345,7 +358,7 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
 #pragma unroll
       for (int i = 0; i < NPL; ++i) {
         const int k = NPL * hl + i;
-        if (k < n) a.best_perm[(size_t)r * n + k] = (int16_t)p[i];
+        if (k < n) a.best_perm[(size_t)r * n + k] = (int16_t)(p[i] - off);
       }
     }
     if (a.stats && live && t >= a.stats_t0) {
@@ -359,7 +372,7 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
 #pragma unroll
   for (int i = 0; i < NPL; ++i) {
     const int k = NPL * hl + i;
-    if (k < n) gq[k] = (int16_t)p[i];
+    if (k < n) gq[k] = (int16_t)(p[i] - off);
   }
   if (hl == 0) {
     a.energy[r] = e;
@@ -410,15 +423,19 @@ cudaError_t launch_qap(const QapArgs &a, cudaStream_t st) {
   auto kern = qap_kernel<NPL, LPR>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  const int blocks = (a.R + 31) / 32;
-  kern<<<blocks, qap_threads<LPR>(), smem, st>>>(a);
+  const int blocks = (a.R + a.rpb - 1) / a.rpb;
+  kern<<<blocks, a.rpb * LPR, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 #define NMC_QAP_CASES(CALL) \
   CALL(0) CALL(1) CALL(2) CALL(3) CALL(4) CALL(5) CALL(6) CALL(7) CALL(8) CALL(9) CALL(10) CALL(11)
 
-cudaError_t dispatch_qap(const QapArgs &a, cudaStream_t st) {
+cudaError_t dispatch_qap(QapArgs a, cudaStream_t st) {
+  int device = 0;
+  const cudaError_t err = cudaGetDevice(&device);
+  if (err != cudaSuccess) return err;
+  a.rpb = qap_replicas_per_block(qap_load(a.n, a.R), qap_lanes(qap_shape(a.n)), device);
   switch (qap_shape(a.n)) {
 #define NMC_CASE(k) case k: return launch_qap<k>(a, st);
     NMC_QAP_CASES(NMC_CASE)
@@ -462,6 +479,7 @@ QapArgs make_args(const QapDevice &I, QapReplicas &Rp, uint64_t seed) {
   a.init_mode = 0;
   a.block = -1;
   a.narrow = I.narrow ? 1 : 0;
+  a.rpb = 32;
   a.mult = nullptr;
   a.stats = nullptr;
   a.stats_t0 = 0;
@@ -469,22 +487,24 @@ QapArgs make_args(const QapDevice &I, QapReplicas &Rp, uint64_t seed) {
 }
 
 template <int Q>
-cudaError_t launch_qap_batch(const QapArgs *items_dev, int n_blocks, int max_n, int tab_len,
+cudaError_t launch_qap_batch(const QapArgs *items_dev, int n_blocks, int rpb, int max_n, int tab_len,
                              cudaStream_t st) {
   constexpr int NPL = shape_npl(Q), LPR = shape_lpr(Q);
   const size_t smem = qap_smem_shape(max_n, Q, tab_len);
   auto kern = qap_batch_kernel<NPL, LPR>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kern<<<n_blocks, qap_threads<LPR>(), smem, st>>>(items_dev);
+  kern<<<n_blocks, rpb * LPR, smem, st>>>(items_dev);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 QapArgs qap_block_args(const QapDevice &I, QapReplicas &Rp, const uint32_t *bq, const uint32_t *tab,
-                       int32_t tab_len, int32_t t0, int32_t t1, uint64_t seed, int block) {
+                       int32_t tab_len, int32_t t0, int32_t t1, uint64_t seed, int rpb,
+                       int block) {
   QapArgs a = make_args(I, Rp, seed);
+  a.rpb = rpb;
   a.bq = bq;
   a.tab = tab;
   a.tab_len = tab_len;
@@ -494,13 +514,35 @@ QapArgs qap_block_args(const QapDevice &I, QapReplicas &Rp, const uint32_t *bq, 
   return a;
 }
 
+int qap_lanes(int shape) { return shape_lpr(shape); }
+
 int qap_shape(int n) { return n <= 128 ? (n + 15) / 16 - 1 : 8 + (n + 31) / 32 - 5; }
 
-cudaError_t qap_batch(const QapArgs *items_dev, int n_blocks, int shape, int max_n, int tab_len,
+// A CTA of 32 replicas with 32 lanes each fills an SM, one with 16 lanes each half of one. The blocks
+// of a call take as many rounds of the SMs as full CTAs would, in equal parts: of 27 replicas where
+// 4 x 128 full CTAs would leave the last of four rounds two fifths empty (4 sets of 4,096 replicas,
+// n = 256), of few where full CTAs would leave SMs without any (256 replicas, n = 33: 8 CTAs of 32,
+// 60 % of their issue slots busy: 1.18 -> 0.95 ms per 100 steps). At least four warps, which also load the CTA's copies of F, D and
+// the table.
+int qap_replicas_per_block(double load, int lanes, int device) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms < 1) {
+    cudaGetLastError();
+    return 32;
+  }
+  const double share = load / (sms * std::max(1.0, std::ceil(load / sms)));
+  const int rpw = 32 / lanes;  // whole warps
+  const int rpb = (static_cast<int>(std::ceil(32.0 * share)) + rpw - 1) / rpw * rpw;
+  return std::min(32, std::max(rpb, 4 * rpw));
+}
+
+double qap_load(int32_t n, int32_t R) { return ((R + 31) / 32) * (n <= 128 ? 0.5 : 1.0); }
+
+cudaError_t qap_batch(const QapArgs *items_dev, int n_blocks, int shape, int rpb, int max_n, int tab_len,
                       cudaStream_t st) {
   if (n_blocks <= 0) return cudaSuccess;
   switch (shape) {
-#define NMC_CASE(k) case k: return launch_qap_batch<k>(items_dev, n_blocks, max_n, tab_len, st);
+#define NMC_CASE(k) case k: return launch_qap_batch<k>(items_dev, n_blocks, rpb, max_n, tab_len, st);
     NMC_QAP_CASES(NMC_CASE)
 #undef NMC_CASE
     default: return cudaErrorInvalidValue;
