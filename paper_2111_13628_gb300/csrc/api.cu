@@ -743,6 +743,14 @@ struct BankOrder {
         first_neg[l] = pre - nn;
       }
     }
+    ra &= ~3;
+    rb = (rb + 3) & ~3;
+    // inert entries among the slots counted as negated in every lane are marked negated; a lane's
+    // number of marked entries goes into the low 7 bits of its first sign byte (the kernel's
+    // counter starts at minus that; lists it takes have at most 128 slots, and with all 128 none is
+    // counted as negated only, so that the counter stays below 128)
+    if (len >= 128) rb = len;
+    int32_t marked[32] = {};
     for (int32_t j = 0; j < len; ++j) {
       for (int p = 0; p < 3; ++p)
         for (int b = 0; b < 32; ++b) cnt[p][b] = 0;
@@ -750,7 +758,9 @@ struct BankOrder {
         int32_t *dst = dst0 + (static_cast<size_t>(j) * 32 + l) * 4;
         std::vector<int32_t> &pool = pend[j >= pre ? 2 : (j < bound[l] ? 0 : 1)][l];
         if (pool.empty() || (j < pre && j >= bound[l] && j < first_neg[l])) {  // inert: own sign 0, one always-true literal (word n)
-          dst[0] = static_cast<int32_t>(1u << 15);
+          const bool neg = j >= rb && j < pre;
+          marked[l] += neg;
+          dst[0] = static_cast<int32_t>(1u << 15 | (neg ? 1u << 7 : 0u));
           dst[1] = dst[2] = dst[3] = n * 4;
           for (int p = 0; p < 3; ++p) add(p, n);
           continue;
@@ -775,6 +785,7 @@ struct BankOrder {
         const int32_t *src = &occ[static_cast<size_t>(pool[best_i]) * 4];
         pool.erase(pool.begin() + best_i);
         uint32_t signs = static_cast<uint32_t>(src[0] != 0) << 7;
+        marked[l] += src[0] != 0;
         for (int p = 0; p < 3; ++p) {
           const int32_t lit = src[1 + kPerm[best_pm][p]];
           signs |= static_cast<uint32_t>(lit & 1) << (8 * (p + 1) + 7);
@@ -784,7 +795,8 @@ struct BankOrder {
         dst[0] = static_cast<int32_t>(signs);
       }
     }
-    return (ra / 4) | ((rb + 3) / 4) << 10 | (pre / 4) << 20;
+    for (int32_t l = 0; l < 32 && len > 0; ++l) dst0[4 * l] |= marked[l] & 0x7F;
+    return (ra / 4) | (rb / 4) << 10 | (pre / 4) << 20;
   }
 };
 

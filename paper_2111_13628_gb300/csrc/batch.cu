@@ -234,123 +234,149 @@ __device__ __forceinline__ void prep_attempt(const BatchItem &B, int cg, int c0,
   }
 }
 
-// Bit-sliced counters of one attempt. k <= 4: a counts Zp, b counts Zn, the own-positive and
-// own-negated occurrences whose other literals are all false. k > 4: a counts the clauses a flip
-// would break, b those it would make.
+// Bit-sliced counters of one attempt.
+// k <= 4: one counter. With z = "every other literal of the clause false", a replica's energy change
+// is x ? Zp - Zn : Zn - Zp, Zp / Zn counting z over the occurrences whose own literal is positive /
+// negated. Counting z over the first and not z over the second gives Zp - Zn + K, K the lane's
+// number of slots counted as negated, so a counter that starts at -K ends at Zp - Zn (8 planes, two's
+// complement). K sits in the low 7 bits of the lane's first sign byte.
+// k > 4: a counts the clauses a flip would break, b those it would make.
 constexpr int kCountPlanes = 7;
-struct Counts {
-  uint32_t a[kCountPlanes], b[kCountPlanes];
+template <int KQ>
+struct Counts;
+template <>
+struct Counts<1> {
+  uint32_t c[8];
+  __device__ __forceinline__ void start(const AttemptPrep<1> &P) {
+    const uint32_t k = P.len > 0 ? 0u - ((uint32_t)P.q[0].x & 0x7Fu) : 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) c[j] = (uint32_t)((int)(k << (31 - j)) >> 31);
+  }
+  // planes of dE for the variable's word x
+  __device__ __forceinline__ void change(uint32_t x, uint32_t (&d)[8]) const {
+    uint32_t carry = ~x;  // negated where x = 0
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      d[j] = (c[j] ^ ~x) ^ carry;
+      carry = (c[j] ^ ~x) & carry;
+    }
+  }
 };
+template <>
+struct Counts<2> {
+  uint32_t a[kCountPlanes], b[kCountPlanes];
+  __device__ __forceinline__ void start(const AttemptPrep<2> &) {
+#pragma unroll
+    for (int j = 0; j < kCountPlanes; ++j) a[j] = b[j] = 0u;
+  }
+  __device__ __forceinline__ void change(uint32_t, uint32_t (&d)[8]) const {
+    uint32_t br = 0u;
+#pragma unroll
+    for (int j = 0; j < kCountPlanes; ++j) {
+      d[j] = a[j] ^ b[j] ^ br;
+      br = maj3b(~a[j], b[j], br);
+    }
+    d[kCountPlanes] = br;
+  }
+};
+
+// Requests the entries of slots e .. e + 3 of the list.
+template <int KQ>
+__device__ __forceinline__ void load_slots(const int4 *ent, int e, int4 (&q)[4 * KQ]) {
+#pragma unroll
+  for (int j = 0; j < 4 * KQ; ++j) q[j] = __ldg(ent + (size_t)(e * KQ + j) * 32);
+}
+
+// What 4 slots add to the k <= 4 counter: z where they count as positive in every lane, its
+// complement where as negated, and the one or the other by the own sign where lanes differ.
+__device__ __forceinline__ uint32_t count4(const uint32_t *xs, const int4 (&q)[4], bool pos, bool neg,
+                                           uint32_t (&c)[8]) {
+  uint32_t o[4], z[4], m[4];  // z = ~(o | m)
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t sg = (uint32_t)q[j].x;
+    o[j] = (xs_at(xs, q[j].y) ^ sign_mask<1>(sg)) | (xs_at(xs, q[j].z) ^ sign_mask<2>(sg));
+    m[j] = xs_at(xs, q[j].w) ^ sign_mask<3>(sg);
+  }
+  if (pos) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]);
+  } else if (neg) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) z[j] = o[j] | m[j];
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]) ^ sign_mask<0>((uint32_t)q[j].x);
+  }
+  return csa4_low<8>(c, z[0], z[1], z[2], z[3]);
+}
 
 // Adds slots [e0, e1) (multiples of 4) of the variable's list to the counters; P.q holds the
 // entries of slot e0's group on entry and those of slot e1's on return (while there are any).
+// Two groups of 4 a trip: each group's weight-4 carry is kept aside and the pair's carries enter
+// the planes from weight 4 up together, and the entries of a group are requested into the other of
+// two buffers while the group before it is evaluated, so the L2 latency of the list overlaps the
+// shared-memory gathers and counting and no entry is copied. With one counter instead of two and
+// no copies an attempt of 32 variables takes 2,025 warp instructions instead of 2,370 (4-SAT, 50,000
+// variables, 1,024 replicas, 200 sweeps: 41.90 -> 40.56 ms; 24 uneven 3-/4-SAT sets: 15.75 -> 12.91).
 template <int KQ>
 __device__ __forceinline__ void count_slots(const uint32_t *xs, uint32_t x, AttemptPrep<KQ> &P,
-                                            int e0, int e1, bool mixed, Counts &C) {
-  constexpr int NB = kCountPlanes;
-  uint32_t (&bc)[NB] = C.a;
-  uint32_t (&mc)[NB] = C.b;
+                                            int e0, int e1, bool mixed, Counts<KQ> &C) {
   const int len = P.len;
   const int4 *ent = P.ent;
-  // The entries of the next group of 4 occurrences are requested before the current group is
-  // evaluated, so the L2 latency of the list overlaps the shared-memory gathers and counting.
-  int4 (&qn)[4 * KQ] = P.q;
-  // break / make masks of the 4 occurrences whose entries are in qc
-  auto masks4 = [&](const int4 (&qc)[4 * KQ], uint32_t (&bb)[4], uint32_t (&mm)[4]) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int4 q = qc[j * KQ];
-      const uint32_t o = others_or<KQ>(xs, q, qc[j * KQ + KQ - 1]);
-      const uint32_t own = x ^ sign_mask<0>((uint32_t)q.x);
-      bb[j] = own & ~o;
-      mm[j] = ~(own | o);
-    }
-  };
+  int4 qb[4 * KQ];
   if constexpr (KQ == 1) {
-    // Own-sign split (k <= 4): in a lane's list the occurrences where its own literal is positive
-    // come first. With z = "every other literal of the clause false", a replica's energy change
-    // is x ? Zp - Zn : Zn - Zp, Zp / Zn counting z over the positive / negated occurrences; slots
-    // [0, ra) are positive in every lane of the group and slots from rb on negated (or inert), so
-    // only [ra, rb) needs both counters, split by the own sign. Each counter keeps one weight-4
-    // carry pending so that the carries of two groups enter it together.
-    const int ra = mixed ? 0 : region_ra(P.regions), rb = mixed ? e1 : region_rb(P.regions);
-    uint32_t fp = 0u, fn = 0u;
-    bool pp = false, pn = false;
-    auto add4 = [&](uint32_t (&c)[NB], uint32_t &f, bool &pend, const uint32_t (&z)[4]) {
-      const uint32_t g = csa4_low(c, z[0], z[1], z[2], z[3]);
-      if (pend) add_carry_pair<NB>(c, f, g);
-      else f = g;
-      pend = !pend;
-    };
-    for (int e = e0; e < e1; e += 4) {
-      int4 qc[4];
+    const int ra = mixed ? 0 : region_ra(P.regions), rb = mixed ? len : region_rb(P.regions);
+#pragma unroll 1
+    for (int e = e0; e < e1; e += 8) {
+      if (e + 4 < len) load_slots<KQ>(ent, e + 4, qb);
+      const uint32_t f = count4(xs, P.q, e + 4 <= ra, e >= rb, C.c);
+      if (e + 4 < e1) {
+        if (e + 8 < len) load_slots<KQ>(ent, e + 8, P.q);
+        add_carry_pair<8>(C.c, f, count4(xs, qb, e + 8 <= ra, e + 4 >= rb, C.c));
+      } else {
+        add_carry<8>(C.c, f);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) qc[j] = qn[j];
-      if (e + 4 < len) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) qn[j] = __ldg(ent + (size_t)(e + 4 + j) * 32);
+        for (int j = 0; j < 4 * KQ; ++j) P.q[j] = qb[j];
       }
-      uint32_t z[4];
+    }
+  } else {
+    constexpr int NB = kCountPlanes;
+    // break / make masks of the 4 occurrences whose entries are in qc
+    auto masks4 = [&](const int4 (&qc)[4 * KQ], uint32_t (&bb)[4], uint32_t (&mm)[4]) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const uint32_t sg = (uint32_t)qc[j].x;
-        z[j] = ~((xs_at(xs, qc[j].y) ^ sign_mask<1>(sg)) | (xs_at(xs, qc[j].z) ^ sign_mask<2>(sg)) |
-                 (xs_at(xs, qc[j].w) ^ sign_mask<3>(sg)));
+        const int4 q = qc[j * KQ];
+        const uint32_t o = others_or<KQ>(xs, q, qc[j * KQ + KQ - 1]);
+        const uint32_t own = x ^ sign_mask<0>((uint32_t)q.x);
+        bb[j] = own & ~o;
+        mm[j] = ~(own | o);
       }
-      if (e + 4 <= ra) {
-        add4(bc, fp, pp, z);
-      } else if (e >= rb) {
-        add4(mc, fn, pn, z);
-      } else {
-        uint32_t zp[4], zn[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t neg = sign_mask<0>((uint32_t)qc[j].x);
-          zp[j] = z[j] & ~neg;
-          zn[j] = z[j] & neg;
-        }
-        add4(bc, fp, pp, zp);
-        add4(mc, fn, pn, zn);
-      }
-    }
-    if (pp) add_carry<NB>(bc, fp);
-    if (pn) add_carry<NB>(mc, fn);
-  } else {
-    // Two groups of 4 per trip: each group's weight-4 carry is kept aside and the pair's carries
-    // enter the planes from weight 4 up once (one ripple per 8 occurrences instead of per 4).
-    // Every group's entries are still requested one group before they are evaluated.
+    };
+#pragma unroll 1
     for (int e = e0; e < e1; e += 8) {
-      int4 qc[4 * KQ];
       uint32_t bb[4], mm[4];
-#pragma unroll
-      for (int j = 0; j < 4 * KQ; ++j) qc[j] = qn[j];
-      if (e + 4 < len) {
-#pragma unroll
-        for (int j = 0; j < 4 * KQ; ++j) qn[j] = __ldg(ent + (size_t)((e + 4) * KQ + j) * 32);
-      }
-      masks4(qc, bb, mm);
-      uint32_t fb = csa4_low(bc, bb[0], bb[1], bb[2], bb[3]);
-      uint32_t fm = csa4_low(mc, mm[0], mm[1], mm[2], mm[3]);
+      if (e + 4 < len) load_slots<KQ>(ent, e + 4, qb);
+      masks4(P.q, bb, mm);
+      const uint32_t fb = csa4_low(C.a, bb[0], bb[1], bb[2], bb[3]);
+      const uint32_t fm = csa4_low(C.b, mm[0], mm[1], mm[2], mm[3]);
       if (e + 4 < e1) {
-#pragma unroll
-        for (int j = 0; j < 4 * KQ; ++j) qc[j] = qn[j];
-        if (e + 8 < len) {
-#pragma unroll
-          for (int j = 0; j < 4 * KQ; ++j) qn[j] = __ldg(ent + (size_t)((e + 8) * KQ + j) * 32);
-        }
-        masks4(qc, bb, mm);
-        add_carry_pair<NB>(bc, fb, csa4_low(bc, bb[0], bb[1], bb[2], bb[3]));
-        add_carry_pair<NB>(mc, fm, csa4_low(mc, mm[0], mm[1], mm[2], mm[3]));
+        if (e + 8 < len) load_slots<KQ>(ent, e + 8, P.q);
+        masks4(qb, bb, mm);
+        add_carry_pair<NB>(C.a, fb, csa4_low(C.a, bb[0], bb[1], bb[2], bb[3]));
+        add_carry_pair<NB>(C.b, fm, csa4_low(C.b, mm[0], mm[1], mm[2], mm[3]));
       } else {
-        add_carry<NB>(bc, fb);
-        add_carry<NB>(mc, fm);
+        add_carry<NB>(C.a, fb);
+        add_carry<NB>(C.b, fm);
+#pragma unroll
+        for (int j = 0; j < 4 * KQ; ++j) P.q[j] = qb[j];
       }
     }
   }
 }
 
-// Acceptance of variable v at the sweep of `rows` for the 32 replicas of the word, from the counters of its
-// whole list; returns its new word. With the table index from one product, the eight-word
+// Acceptance of variable v at the sweep of `rows` for the 32 replicas of the word, from the counters
+// of its whole list; returns its new word. With the table index from one product, the eight-word
 // transpose and the Philox blocks from their third round on, 200 sweeps of the 50,000-variable
 // bench instance with 1,024 replicas take 41.90 ms (43.94 before), 24 uneven 3-/4-SAT sets 15.75
 // ms per 100 sweeps (16.96). With PT, replica j of the word moves at min(2^32-1,
@@ -358,31 +384,10 @@ __device__ __forceinline__ void count_slots(const uint32_t *xs, uint32_t x, Atte
 template <int KQ, bool PT>
 __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint32_t *tab_s,
                                                  int tab_len, const uint32_t *mult_s,
-                                                 const SweepRows &rows, int v, uint32_t x, uint32_t bqv, Counts &C,
+                                                 const SweepRows &rows, int v, uint32_t x, uint32_t bqv, const Counts<KQ> &C,
                                                  uint32_t (&acc)[kAccPlanes]) {
-  constexpr int NB = kCountPlanes;
-  uint32_t (&bc)[NB] = C.a;
-  uint32_t (&mc)[NB] = C.b;
-  if (KQ == 1) {
-    // (bc, mc) <- (Zp, Zn) where x = 1, (Zn, Zp) where x = 0: the subtraction below is the dE
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const uint32_t a = (bc[j] & x) | (mc[j] & ~x), c = (mc[j] & x) | (bc[j] & ~x);
-      bc[j] = a;
-      mc[j] = c;
-    }
-  }
-  // D = B - U, 8 bit planes (two's complement), then per-replica bytes by 8x8 transposes
   uint32_t s8[8];
-  {
-    uint32_t br = 0u;
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      s8[j] = bc[j] ^ mc[j] ^ br;
-      br = maj3b(~bc[j], mc[j], br);
-    }
-    s8[NB] = br;
-  }
+  C.change(x, s8);
   const PhiloxCol col = philox_col((uint32_t)__ldg(B.orig + v), kTagKsatSweep, B.k1);
   const uint32_t bqc = min(bqv, (uint32_t)tab_len << 8);
   // replicas whose dE <= 0 (sign plane set, or every plane zero) accept without a draw
@@ -650,8 +655,7 @@ __device__ __forceinline__ T *rank_ptr(T *p, int r) {
 template <int KQ, int CS, int TT, bool PT>
 __device__ __forceinline__ void class_teams(const BatchItem &B, uint32_t *xs, const uint32_t *tab_s,
                                             int tab_len, const uint32_t *mult_s,
-                                            const SweepRows &rows, int cg, int c0, int cnt,
-                                            int rank, int t, int *ep_s) {
+                                            const SweepRows &rows, int cg, int c0, int cnt, int rank, int t, int *ep_s) {
   const int lane = threadIdx.x & 31;
   if ((int)(threadIdx.x & ~31u) / TT >= cnt) return;  // the whole warp
   const int team = threadIdx.x / TT, tl = lane % TT;
@@ -766,14 +770,14 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
           // a smaller share (the later colour classes): teams of 8, 4 or 2 lanes per variable
           // shorten the class's critical path; their energy changes go to ep_s directly
           if (cnt <= kThreads / 8)
-            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt, rank, t,
-                                         ep_s);
+            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt,
+                                         rank, t, ep_s);
           else if (cnt <= kThreads / 4)
-            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt, rank, t,
-                                         ep_s);
+            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt,
+                                         rank, t, ep_s);
           else
-            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt, rank, t,
-                                         ep_s);
+            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt,
+                                         rank, t, ep_s);
         } else {
           auto store = [&](int v, uint32_t xn) {
             if (CS == 1) {
@@ -795,7 +799,8 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
             if (!first) prep_attempt<KQ>(B, cg, c0, v, t, P);
             const bool go = li < cnt && P.bq != kFrozenQ16;  // a held variable takes no attempt
             const uint32_t x = xs[v];
-            Counts C = {};
+            Counts<KQ> C;
+            C.start(P);
 #pragma unroll 1
             for (int part = 0; part < 2; ++part) {
               const int pre = region_pre(P.regions);
@@ -805,8 +810,8 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
               }
               if (go) count_slots<KQ>(xs, x, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
             }
-            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, mult_s, rows_s, v, x, P.bq,
-                                                    C, acc));
+            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, mult_s, rows_s, v, x,
+                                                    P.bq, C, acc));
             if (base + kThreads >= cnt) break;
           }
         }
