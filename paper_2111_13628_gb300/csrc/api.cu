@@ -1138,8 +1138,7 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
       grp_v0.push_back(g0);
     }
   }
-  // slot regions of every group, stored after the G + 1 offsets (BankOrder::build; k > 4: only
-  // the first slot with a literal of the previous class)
+  // slot regions of every group, stored after the G + 1 offsets (BankOrder::build)
   const int32_t n_groups = static_cast<int32_t>(grp_v0.size());
   grp_base.resize(static_cast<size_t>(2) * n_groups + 1, 0);
   // of every group's class: its end, its first variable and the previous class's first variable
@@ -1182,9 +1181,10 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
         dep = std::max(dep, static_cast<int32_t>(late[l].size()));
       }
       const int32_t pre = len - ((dep + 3) & ~3);
-      grp_base[n_groups + 1 + g] = (pre / 4) << 20;
+      grp_base[n_groups + 1 + g] = (len / 4) << 10 | (pre / 4) << 20;  // no slot of one sign only
       for (int32_t l = 0; l < 32; ++l) {
         size_t at = 0, lat = 0;
+        uint32_t marked = 0;  // own-negated occurrences: into free bits of the first sign word
         for (int32_t j = 0; j < len; ++j) {
           int32_t *dst = &occ_t[(static_cast<size_t>(grp_base[g]) + j * kq * 32 + l) * 4];
           int32_t *dst2 = dst + 32 * 4;  // the occurrence's second int4, one warp row further
@@ -1194,12 +1194,16 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
           const int32_t *src = e >= 0 ? &occ[static_cast<size_t>(e) * slots] : nullptr;
           auto lit = [&](int z) { return src ? src[z] : (z == 1 ? lit_true : lit_false); };
           uint32_t signs = static_cast<uint32_t>(src && src[0] != 0) << 7;
+          marked += signs >> 7;
           for (int z = 1; z < 4; ++z) signs |= static_cast<uint32_t>(lit(z) & 1) << (8 * z + 7);
           for (int z = 4; z < 8; ++z) signs |= static_cast<uint32_t>(lit(z) & 1) << (8 * (z - 4) + 6);
           dst[0] = static_cast<int32_t>(signs);
           for (int z = 1; z < 4; ++z) dst[z] = (lit(z) >> 1) * 4;
           for (int z = 0; z < 4; ++z) dst2[z] = (lit(4 + z) >> 1) * 4;
         }
+        if (len > 0)
+          occ_t[(static_cast<size_t>(grp_base[g]) + l) * 4] |=
+              static_cast<int32_t>((marked & 0x3Fu) << 8 | (marked & 0x40u) << 10);
       }
     }
   }, 32);  // a group is 32 variables' lists

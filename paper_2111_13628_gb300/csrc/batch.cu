@@ -14,6 +14,7 @@
 // per-replica sums once per sweep.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -39,17 +40,16 @@ template <int KQ>
 __host__ __device__ constexpr int one_thread_threads() {
   return KQ == 1 ? 512 : 384;
 }
-constexpr int kTeamThreads = 384;   // team kernel with teams of 2 or 4: 12 warps, up to 168 registers
-constexpr int kTeam8Threads = 512;  // team kernel with teams of 8: up to 128 registers
+constexpr int kTeamThreads = 384;   // team kernel with teams of 4: 12 warps, up to 168 registers
+constexpr int kTeam8Threads = 512;  // team kernel with teams of 8, k <= 4: up to 128 registers
 
-// Threads of the sweep kernel with TL lanes per variable: 384 for teams of 2 or 4, which then
-// prefetch their occurrence entries a group ahead (measured at N = 5,000: 107 -> 102 us per
-// sweep); 512 for teams of 8 (the tiny classes of small instances, where 384 threads measured
-// slower: N = 200, 37.3 -> 45.3 us; 640 spilled with the replica-exchange multipliers); single
-// threads as one_thread_threads.
+// Threads of the sweep kernel with TL lanes per variable: 384 for teams of 4, which hold four to
+// eight of their list entries per lane, and for teams of 8 with two int4 per occurrence (512 threads
+// spilled 400 bytes); 512 for teams of 8 with k <= 4; single threads as one_thread_threads.
 template <int KQ, int TL>
 __host__ __device__ constexpr int sweep_threads() {
-  return (TL == 2 || TL == 4) ? kTeamThreads : (TL == 8 ? kTeam8Threads : one_thread_threads<KQ>());
+  return (TL == 4 || (TL == 8 && KQ == 2)) ? kTeamThreads
+                                           : (TL == 8 ? kTeam8Threads : one_thread_threads<KQ>());
 }
 
 template <int NB>
@@ -235,20 +235,21 @@ __device__ __forceinline__ void prep_attempt(const BatchItem &B, int cg, int c0,
 }
 
 // Bit-sliced counters of one attempt.
-// k <= 4: one counter. With z = "every other literal of the clause false", a replica's energy change
+// One counter. With z = "every other literal of the clause false", a replica's energy change
 // is x ? Zp - Zn : Zn - Zp, Zp / Zn counting z over the occurrences whose own literal is positive /
 // negated. Counting z over the first and not z over the second gives Zp - Zn + K, K the lane's
 // number of slots counted as negated, so a counter that starts at -K ends at Zp - Zn (8 planes, two's
-// complement). K sits in the low 7 bits of the lane's first sign byte.
-// k > 4: a counts the clauses a flip would break, b those it would make.
-constexpr int kCountPlanes = 7;
+// complement). K sits in free bits of the lane's first sign word: the low 7 bits (k <= 4), or the low
+// 6 bits of byte 1 and bit 16 (k > 4).
 template <int KQ>
-struct Counts;
-template <>
-struct Counts<1> {
+__device__ __forceinline__ uint32_t marked_slots(uint32_t sg) {  // K, from the first sign word
+  return KQ == 1 ? sg & 0x7Fu : ((sg >> 8) & 0x3Fu) | ((sg >> 10) & 0x40u);
+}
+template <int KQ>
+struct Counts {
   uint32_t c[8];
-  __device__ __forceinline__ void start(const AttemptPrep<1> &P) {
-    const uint32_t k = P.len > 0 ? 0u - ((uint32_t)P.q[0].x & 0x7Fu) : 0u;
+  __device__ __forceinline__ void start(const AttemptPrep<KQ> &P) {
+    const uint32_t k = P.len > 0 ? 0u - marked_slots<KQ>((uint32_t)P.q[0].x) : 0u;
 #pragma unroll
     for (int j = 0; j < 8; ++j) c[j] = (uint32_t)((int)(k << (31 - j)) >> 31);
   }
@@ -262,23 +263,6 @@ struct Counts<1> {
     }
   }
 };
-template <>
-struct Counts<2> {
-  uint32_t a[kCountPlanes], b[kCountPlanes];
-  __device__ __forceinline__ void start(const AttemptPrep<2> &) {
-#pragma unroll
-    for (int j = 0; j < kCountPlanes; ++j) a[j] = b[j] = 0u;
-  }
-  __device__ __forceinline__ void change(uint32_t, uint32_t (&d)[8]) const {
-    uint32_t br = 0u;
-#pragma unroll
-    for (int j = 0; j < kCountPlanes; ++j) {
-      d[j] = a[j] ^ b[j] ^ br;
-      br = maj3b(~a[j], b[j], br);
-    }
-    d[kCountPlanes] = br;
-  }
-};
 
 // Requests the entries of slots e .. e + 3 of the list.
 template <int KQ>
@@ -287,26 +271,34 @@ __device__ __forceinline__ void load_slots(const int4 *ent, int e, int4 (&q)[4 *
   for (int j = 0; j < 4 * KQ; ++j) q[j] = __ldg(ent + (size_t)(e * KQ + j) * 32);
 }
 
-// What 4 slots add to the k <= 4 counter: z where they count as positive in every lane, its
-// complement where as negated, and the one or the other by the own sign where lanes differ.
-__device__ __forceinline__ uint32_t count4(const uint32_t *xs, const int4 (&q)[4], bool pos, bool neg,
-                                           uint32_t (&c)[8]) {
-  uint32_t o[4], z[4], m[4];  // z = ~(o | m)
+// What 4 slots add to the counter: z where they count as positive in every lane, its complement
+// where as negated, and the one or the other by the own sign where lanes differ (k > 4: always).
+template <int KQ>
+__device__ __forceinline__ uint32_t count4(const uint32_t *xs, const int4 (&q)[4 * KQ], bool pos,
+                                           bool neg, uint32_t (&c)[8]) {
+  uint32_t z[4];
+  if constexpr (KQ == 2) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t sg = (uint32_t)q[j].x;
-    o[j] = (xs_at(xs, q[j].y) ^ sign_mask<1>(sg)) | (xs_at(xs, q[j].z) ^ sign_mask<2>(sg));
-    m[j] = xs_at(xs, q[j].w) ^ sign_mask<3>(sg);
-  }
-  if (pos) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]);
-  } else if (neg) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) z[j] = o[j] | m[j];
+    for (int j = 0; j < 4; ++j)
+      z[j] = ~others_or<2>(xs, q[2 * j], q[2 * j + 1]) ^ sign_mask<0>((uint32_t)q[2 * j].x);
   } else {
+    uint32_t o[4], m[4];  // z = ~(o | m)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]) ^ sign_mask<0>((uint32_t)q[j].x);
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t sg = (uint32_t)q[j].x;
+      o[j] = (xs_at(xs, q[j].y) ^ sign_mask<1>(sg)) | (xs_at(xs, q[j].z) ^ sign_mask<2>(sg));
+      m[j] = xs_at(xs, q[j].w) ^ sign_mask<3>(sg);
+    }
+    if (pos) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]);
+    } else if (neg) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) z[j] = o[j] | m[j];
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]) ^ sign_mask<0>((uint32_t)q[j].x);
+    }
   }
   return csa4_low<8>(c, z[0], z[1], z[2], z[3]);
 }
@@ -320,57 +312,23 @@ __device__ __forceinline__ uint32_t count4(const uint32_t *xs, const int4 (&q)[4
 // no copies an attempt of 32 variables takes 2,025 warp instructions instead of 2,370 (4-SAT, 50,000
 // variables, 1,024 replicas, 200 sweeps: 41.90 -> 40.56 ms; 24 uneven 3-/4-SAT sets: 15.75 -> 12.91).
 template <int KQ>
-__device__ __forceinline__ void count_slots(const uint32_t *xs, uint32_t x, AttemptPrep<KQ> &P,
-                                            int e0, int e1, bool mixed, Counts<KQ> &C) {
+__device__ __forceinline__ void count_slots(const uint32_t *xs, AttemptPrep<KQ> &P, int e0, int e1,
+                                            bool mixed, Counts<KQ> &C) {
   const int len = P.len;
   const int4 *ent = P.ent;
   int4 qb[4 * KQ];
-  if constexpr (KQ == 1) {
-    const int ra = mixed ? 0 : region_ra(P.regions), rb = mixed ? len : region_rb(P.regions);
+  const int ra = mixed ? 0 : region_ra(P.regions), rb = mixed ? len : region_rb(P.regions);
 #pragma unroll 1
-    for (int e = e0; e < e1; e += 8) {
-      if (e + 4 < len) load_slots<KQ>(ent, e + 4, qb);
-      const uint32_t f = count4(xs, P.q, e + 4 <= ra, e >= rb, C.c);
-      if (e + 4 < e1) {
-        if (e + 8 < len) load_slots<KQ>(ent, e + 8, P.q);
-        add_carry_pair<8>(C.c, f, count4(xs, qb, e + 8 <= ra, e + 4 >= rb, C.c));
-      } else {
-        add_carry<8>(C.c, f);
+  for (int e = e0; e < e1; e += 8) {
+    if (e + 4 < len) load_slots<KQ>(ent, e + 4, qb);
+    const uint32_t f = count4<KQ>(xs, P.q, e + 4 <= ra, e >= rb, C.c);
+    if (e + 4 < e1) {
+      if (e + 8 < len) load_slots<KQ>(ent, e + 8, P.q);
+      add_carry_pair<8>(C.c, f, count4<KQ>(xs, qb, e + 8 <= ra, e + 4 >= rb, C.c));
+    } else {
+      add_carry<8>(C.c, f);
 #pragma unroll
-        for (int j = 0; j < 4 * KQ; ++j) P.q[j] = qb[j];
-      }
-    }
-  } else {
-    constexpr int NB = kCountPlanes;
-    // break / make masks of the 4 occurrences whose entries are in qc
-    auto masks4 = [&](const int4 (&qc)[4 * KQ], uint32_t (&bb)[4], uint32_t (&mm)[4]) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int4 q = qc[j * KQ];
-        const uint32_t o = others_or<KQ>(xs, q, qc[j * KQ + KQ - 1]);
-        const uint32_t own = x ^ sign_mask<0>((uint32_t)q.x);
-        bb[j] = own & ~o;
-        mm[j] = ~(own | o);
-      }
-    };
-#pragma unroll 1
-    for (int e = e0; e < e1; e += 8) {
-      uint32_t bb[4], mm[4];
-      if (e + 4 < len) load_slots<KQ>(ent, e + 4, qb);
-      masks4(P.q, bb, mm);
-      const uint32_t fb = csa4_low(C.a, bb[0], bb[1], bb[2], bb[3]);
-      const uint32_t fm = csa4_low(C.b, mm[0], mm[1], mm[2], mm[3]);
-      if (e + 4 < e1) {
-        if (e + 8 < len) load_slots<KQ>(ent, e + 8, P.q);
-        masks4(qb, bb, mm);
-        add_carry_pair<NB>(C.a, fb, csa4_low(C.a, bb[0], bb[1], bb[2], bb[3]));
-        add_carry_pair<NB>(C.b, fm, csa4_low(C.b, mm[0], mm[1], mm[2], mm[3]));
-      } else {
-        add_carry<NB>(C.a, fb);
-        add_carry<NB>(C.b, fm);
-#pragma unroll
-        for (int j = 0; j < 4 * KQ; ++j) P.q[j] = qb[j];
-      }
+      for (int j = 0; j < 4 * KQ; ++j) P.q[j] = qb[j];
     }
   }
 }
@@ -430,7 +388,7 @@ __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint3
   return x ^ flip;
 }
 
-// ---- team variant: TL lanes per variable --------------------------------------------------------
+// ---- small classes of the one-thread kernel: TL lanes per variable -------------------------------
 //
 // Same dynamics, shorter critical path: a team of TL consecutive lanes evaluates one variable.
 // Lane t of the team takes occurrences t, t+TL, ... of the variable's list, counts its break /
@@ -439,7 +397,7 @@ __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint3
 // acceptance of replica groups [t*8/TL, (t+1)*8/TL) (one Philox block per group of 4 replicas)
 // and the team ORs the flip bits. A colour class of a few hundred variables then costs the
 // latency of a TL-th of one attempt instead of a whole one.
-template <int KQ, int TL, bool PT, bool PF = false>
+template <int KQ, int TL, bool PT>
 __device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint32_t *xs,
                                                  const uint32_t *tab_s, int tab_len,
                                                  const uint32_t *mult_s, const SweepRows &rows,
@@ -465,46 +423,7 @@ __device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint3
     len = (__ldg(B.grp_base + g + 1) - gb) / (32 * KQ);
     ent = B.occ_t + gb + ln;
   }
-  // occurrences j0 + i TL (i < 4) of the lane: break / make masks into the counters
-  auto eval4 = [&](const int4 (&qc)[4 * KQ], int j0) {
-    uint32_t bb[4], mm[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = j0 + i * TL;
-      bb[i] = 0u;
-      mm[i] = 0u;
-      if (j < len) {
-        const int4 q = qc[i * KQ];
-        const uint32_t o = others_or<KQ>(xs, q, qc[i * KQ + KQ - 1]);
-        const uint32_t own = x ^ sign_mask<0>((uint32_t)q.x);
-        bb[i] = own & ~o;
-        mm[i] = ~(own | o);
-      }
-    }
-    csa4<NB>(bc, bb[0], bb[1], bb[2], bb[3]);
-    csa4<NB>(mc, mm[0], mm[1], mm[2], mm[3]);
-  };
-  auto load4 = [&](int4 (&q)[4 * KQ], int j0) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = j0 + i * TL;
-#pragma unroll
-      for (int k = 0; k < KQ; ++k)
-        q[i * KQ + k] = j < len ? __ldg(ent + (size_t)(j * KQ + k) * 32) : make_int4(0, 0, 0, 0);
-    }
-  };
-  if constexpr (PF) {
-    // the next group of the lane's entries is requested before the current one is evaluated
-    int4 qn[4 * KQ];
-    if (tl < len) load4(qn, tl);
-    for (int j0 = tl; j0 < len; j0 += 4 * TL) {
-      int4 qc[4 * KQ];
-#pragma unroll
-      for (int i = 0; i < 4 * KQ; ++i) qc[i] = qn[i];
-      if (j0 + 4 * TL < len) load4(qn, j0 + 4 * TL);
-      eval4(qc, j0);
-    }
-  } else {
+  {
     // each group's entries loaded where they are evaluated
     for (int j0 = tl; j0 < len; j0 += 4 * TL) {
       uint32_t bb[4], mm[4];
@@ -691,6 +610,120 @@ __device__ __forceinline__ void class_teams(const BatchItem &B, uint32_t *xs, co
     if (tacc[i] != 0) atomicAdd(&ep_s[4 * (tl * (8 / TT) + i / 4) + (i & 3)], tacc[i]);
 }
 
+// ---- what both sweep kernels share --------------------------------------------------------------
+
+// Static shared memory of a sweep kernel.
+struct SweepShared {
+  BatchItem item;   // the current item, read from here where needed
+  int ep[2][32];    // energy changes of the even and odd sweeps, per replica
+  uint32_t mult[32];  // temperature multipliers (replica exchange)
+  SweepRows rows;
+  uint32_t improved;  // replicas that improved in the last sweep
+  int next;           // index of the current item
+};
+
+// Energies of the word's replicas, kept by warp 0 of every CTA (its lane's replica), and the
+// replicas that improved during the item.
+struct EnergyTrack {
+  int e, best;
+  long long s1, s2;  // sums of E and E^2 of the sampled sweeps
+  uint32_t m_item;
+};
+
+// Takes the next item from the counter into sh.item; false when there is none left.
+template <int CS>
+__device__ __forceinline__ bool next_batch_item(const BatchItem *items, int n_items, int *next_item,
+                                                int rank, SweepShared &sh) {
+  if (rank == 0 && threadIdx.x == 0) sh.next = atomicAdd(next_item, 1);
+  group_sync<CS>();
+  const int it = *rank_ptr<CS>(&sh.next, 0);
+  if (it < n_items && threadIdx.x == 0) sh.item = items[it];
+  group_sync<CS>();  // every rank has read the item id before any rank moves on or exits
+  return it < n_items;
+}
+
+// The item's word vector, energies and multipliers into shared memory and registers, and the Philox
+// rows of its first sweep. A barrier of the CTAs must follow.
+template <int CS, bool PT>
+__device__ __forceinline__ void load_item(const BatchItem &B, int rank, uint32_t *xs, SweepShared &sh,
+                                          EnergyTrack &k) {
+  const int n = B.n, W = B.W, w = B.w;
+  for (int v = threadIdx.x; v < n; v += blockDim.x) xs[v] = B.S[(size_t)(2 * v) * W + w];
+  if (threadIdx.x == 0) xs[n] = 0u;
+  k = EnergyTrack{};
+  if (threadIdx.x < 32) {
+    sh.ep[0][threadIdx.x] = sh.ep[1][threadIdx.x] = 0;
+    if (PT) sh.mult[threadIdx.x] = B.mult[32 * w + threadIdx.x];
+    k.e = B.energy[32 * w + threadIdx.x];
+    k.best = B.best_energy[32 * w + threadIdx.x];
+  }
+  sh.rows.fill(B, B.t0);
+}
+
+// After the last class of sweep t is published (and with it every CTA's energy changes): energies,
+// best energies and, where a replica improved, its state. Every CTA sums the changes itself, so the
+// CTAs only meet again when there is a state to copy.
+// Best states go to a word-major staging row (the second half of the best buffer) at each improving
+// sweep end, and into the [var][word] layout once, at the end of the item: a merge into that layout
+// touches one 32-byte sector per variable, which at every improving sweep cost about 30 us per sweep
+// on the 50,000-variable bench instance.
+template <int CS, bool PT>
+__device__ __forceinline__ void end_sweep(const BatchItem &B, int rank, int t, uint32_t *xs,
+                                          SweepShared &sh, EnergyTrack &k) {
+  const int n = B.n;
+  if (threadIdx.x < 32) {
+    int sum = k.e;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) sum += rank_ptr<CS>(&sh.ep[t & 1][0], r)[threadIdx.x];
+    k.e = sum;
+    if (PT && B.stats && t >= B.stats_t0) {
+      k.s1 += sum;
+      k.s2 += (long long)sum * sum;
+    }
+    const bool better = sum < k.best;
+    if (better) k.best = sum;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, better);
+    if (threadIdx.x == 0) sh.improved = m;
+    sh.ep[~t & 1][threadIdx.x] = 0;  // last read before this sweep's class barriers
+  }
+  sh.rows.fill(B, t + 1);
+  __syncthreads();
+  const uint32_t m = sh.improved;
+  if (m) {
+    uint32_t *best_t = B.best + (size_t)n * B.W + (size_t)B.w * n;
+    const int share = (n + CS - 1) / CS, b0 = rank * share, b1 = min(n, b0 + share);
+    for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x)
+      best_t[v] = (best_t[v] & ~m) | (xs[v] & m);
+    k.m_item |= m;
+    group_sync<CS>();
+  }
+}
+
+// States, best states and energies of the item back to memory.
+template <int CS, bool PT>
+__device__ __forceinline__ void store_item(const BatchItem &B, int rank, const uint32_t *xs,
+                                           const EnergyTrack &k) {
+  const int n = B.n, W = B.W, w = B.w;
+  const uint32_t *best_t = B.best + (size_t)n * W + (size_t)w * n;
+  const int share = (n + CS - 1) / CS, b0 = rank * share, b1 = min(n, b0 + share);
+  for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x) {
+    B.S[(size_t)(2 * v) * W + w] = xs[v];
+    B.S[(size_t)(2 * v + 1) * W + w] = ~xs[v];
+    if (k.m_item) {  // replicas improved during the item: their last best state from staging
+      const size_t bi = (size_t)v * W + w;
+      B.best[bi] = (B.best[bi] & ~k.m_item) | (best_t[v] & k.m_item);
+    }
+  }
+  if (rank == 0 && threadIdx.x < 32) {
+    B.energy[32 * w + threadIdx.x] = k.e;
+    B.best_energy[32 * w + threadIdx.x] = k.best;
+    if (PT && B.stats) {  // one item per word in a launch: plain read-modify-write
+      B.stats[32 * w + threadIdx.x] += k.s1;
+      B.stats[32 * (B.W + w) + threadIdx.x] += k.s2;
+    }
+  }
+}
+
 // CS = CTAs per item. With CS > 1 every CTA of the cluster keeps a full copy of the item's
 // word vector; each CTA updates its share of every colour class and stores the new words
 // into all CS copies (distributed shared memory), then the cluster barrier publishes them.
@@ -703,44 +736,15 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
   extern __shared__ __align__(16) uint32_t smem[];
   uint32_t *xs = smem;                               // word vector first (byte offsets in lists)
   uint32_t *tab_s = smem + ((xs_words + 31) & ~31);  // then the acceptance table
-  __shared__ int e_s[32], be_s[32], ep_s[32];
-  __shared__ uint32_t mult_s[32];
-  __shared__ SweepRows rows_s;
-  __shared__ uint32_t imp_s;
-  __shared__ int item_s;
-  __shared__ BatchItem item_b;  // the current item, read from shared memory where needed
+  __shared__ SweepShared sh;
   const int rank = CS == 1 ? 0 : (int)cg::this_cluster().block_rank();
   for (int i = threadIdx.x; i <= tab_len; i += blockDim.x) tab_s[i] = i < tab_len ? tab[i] : 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   while (true) {
-    if (rank == 0 && threadIdx.x == 0) item_s = atomicAdd(next_item, 1);
-    group_sync<CS>();
-    const int it = *rank_ptr<CS>(&item_s, 0);
-    if (it < n_items && threadIdx.x == 0) item_b = items[it];
-    group_sync<CS>();  // every rank has read the item id before any rank moves on or exits
-    if (it >= n_items) break;
-    const BatchItem &B = item_b;
-    const int n = B.n, W = B.W, w = B.w;
-    const int share = (n + CS - 1) / CS;
-    for (int v = threadIdx.x; v < n; v += blockDim.x) xs[v] = B.S[(size_t)(2 * v) * W + w];
-    if (threadIdx.x == 0) xs[n] = 0u;
-    if (threadIdx.x < 32) {
-      ep_s[threadIdx.x] = 0;
-      if (PT) mult_s[threadIdx.x] = B.mult[32 * w + threadIdx.x];
-      if (rank == 0) {
-        e_s[threadIdx.x] = B.energy[32 * w + threadIdx.x];
-        be_s[threadIdx.x] = B.best_energy[32 * w + threadIdx.x];
-      }
-    }
-    long long s1 = 0, s2 = 0;  // energy statistics of this lane's replica (rank 0, warp 0)
-    // Best states of the replicas that improve during this item go to a word-major staging row
-    // (the second half of the best buffer) at each improving sweep end, and into the [var][word]
-    // layout once, at the end of the item: a merge into that layout touches one 32-byte sector
-    // per variable, which at every improving sweep cost about 30 us per sweep on the 50,000-
-    // variable bench instance.
-    uint32_t *best_t = B.best + (size_t)n * W + (size_t)w * n;
-    uint32_t m_item = 0;  // replicas improved during this item
-    rows_s.fill(B, B.t0);
+    if (!next_batch_item<CS>(items, n_items, next_item, rank, sh)) break;
+    const BatchItem &B = sh.item;
+    EnergyTrack track;
+    load_item<CS, PT>(B, rank, xs, sh, track);
     group_sync<CS>();
     for (int t = B.t0; t < B.t1; ++t) {
       uint32_t acc[kAccPlanes];
@@ -781,14 +785,14 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
           // a smaller share (the later colour classes): teams of 8, 4 or 2 lanes per variable
           // shorten the class's critical path; their energy changes go to ep_s directly
           if (cnt <= kThreads / 8)
-            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt,
-                                         rank, t, ep_s);
+            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, sh.mult, sh.rows, cg, c0, cnt,
+                                         rank, t, sh.ep[t & 1]);
           else if (cnt <= kThreads / 4)
-            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt,
-                                         rank, t, ep_s);
+            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, sh.mult, sh.rows, cg, c0, cnt,
+                                         rank, t, sh.ep[t & 1]);
           else
-            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, cnt,
-                                         rank, t, ep_s);
+            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, sh.mult, sh.rows, cg, c0, cnt,
+                                         rank, t, sh.ep[t & 1]);
         } else {
           auto store = [&](int v, uint32_t xn) {
             if (CS == 1) {
@@ -819,12 +823,36 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
                 __syncwarp();
                 class_wait();
               }
-              if (go) count_slots<KQ>(xs, x, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
+              if (go) count_slots<KQ>(xs, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
             }
-            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, mult_s, rows_s, v, x,
+            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, sh.mult, sh.rows, v, x,
                                                     P.bq, C, acc));
             if (base + kThreads >= cnt) break;
           }
+        }
+        if (c + 1 == B.n_colours) {
+          // the sweep's energy changes, published with its last class: planes -> 16-bit values (one
+          // byte transpose for each half of the planes), then a warp reduction per replica
+          uint32_t lo[8], hi[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            lo[j] = acc[j];
+            hi[j] = acc[8 + j];
+          }
+          transpose8x32(lo);
+          transpose8x32(hi);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              // bytes q of lo and hi as one signed 16-bit value, sign-extended
+              uint32_t val;
+              asm("prmt.b32 %0, %1, %2, %3;"
+                  : "=r"(val)
+                  : "r"(lo[j]), "r"(hi[j]), "r"(0xCC40u + 0x1111u * (uint32_t)q));
+              const int sum = __reduce_add_sync(0xFFFFFFFFu, (int)val);
+              if (lane == 0 && sum != 0) atomicAdd(&sh.ep[t & 1][8 * q + j], sum);
+            }
         }
         // this CTA's words of the class are published; the next class's loads are requested and
         // its slots before `pre` counted (none holds a literal of this class) before the wait
@@ -842,228 +870,379 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         cg = cgn;
       }
       class_wait();
-      // per-replica sums of this sweep: planes -> 16-bit values (one byte transpose for each
-      // half of the planes), then a warp reduction per replica
-      {
-        uint32_t lo[8], hi[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          lo[j] = acc[j];
-          hi[j] = acc[8 + j];
-        }
-        transpose8x32(lo);
-        transpose8x32(hi);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            // bytes q of lo and hi as one signed 16-bit value, sign-extended
-            uint32_t val;
-            asm("prmt.b32 %0, %1, %2, %3;"
-                : "=r"(val)
-                : "r"(lo[j]), "r"(hi[j]), "r"(0xCC40u + 0x1111u * (uint32_t)q));
-            const int sum = __reduce_add_sync(0xFFFFFFFFu, (int)val);
-            if (lane == 0 && sum != 0) atomicAdd(&ep_s[8 * q + j], sum);
-          }
-      }
-      group_sync<CS>();
-      if (rank == 0 && warp == 0) {
-        int sum = e_s[lane];
-#pragma unroll
-        for (int r = 0; r < CS; ++r) sum += rank_ptr<CS>(ep_s, r)[lane];
-        e_s[lane] = sum;
-        if (PT && B.stats && t >= B.stats_t0) {
-          s1 += sum;
-          s2 += (long long)sum * sum;
-        }
-        const bool better = sum < be_s[lane];
-        if (better) be_s[lane] = sum;
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, better);
-        if (lane == 0) imp_s = m;
-      }
-      group_sync<CS>();
-      const uint32_t m = *rank_ptr<CS>(&imp_s, 0);
-      if (threadIdx.x < 32) ep_s[threadIdx.x] = 0;
-      rows_s.fill(B, t + 1);
-      __syncthreads();  // cleared and filled before the next sweep's attempts
-      if (m) {  // the improved replicas' states, into this word's staging row (coalesced)
-        const int b0 = rank * share, b1 = min(n, b0 + share);
-        for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x)
-          best_t[v] = (best_t[v] & ~m) | (xs[v] & m);
-        m_item |= m;
-        group_sync<CS>();
-      }
+      end_sweep<CS, PT>(B, rank, t, xs, sh, track);
     }
-    {
-      const int b0 = rank * share, b1 = min(n, b0 + share);
-      for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x) {
-        B.S[(size_t)(2 * v) * W + w] = xs[v];
-        B.S[(size_t)(2 * v + 1) * W + w] = ~xs[v];
-        if (m_item) {  // replicas improved during the item: their last best state from staging
-          const size_t bi = (size_t)v * W + w;
-          B.best[bi] = (B.best[bi] & ~m_item) | (best_t[v] & m_item);
-        }
-      }
-    }
-    if (rank == 0 && threadIdx.x < 32) {
-      B.energy[32 * w + threadIdx.x] = e_s[threadIdx.x];
-      B.best_energy[32 * w + threadIdx.x] = be_s[threadIdx.x];
-      if (PT && B.stats) {  // one item per word in a launch: plain read-modify-write
-        B.stats[32 * w + threadIdx.x] += s1;
-        B.stats[32 * (B.W + w) + threadIdx.x] += s2;
-      }
-    }
+    store_item<CS, PT>(B, rank, xs, track);
     group_sync<CS>();
   }
 }
 
+// ---- team kernel: every class with TL lanes per variable ---------------------------------------
+//
+// For instances whose classes put few variables on a CTA the sweep is a chain of class latencies,
+// so whatever does not depend on the previous class is taken off that chain. A warp handles 32 / TL
+// variables, and the warps of a CTA are dealt out over consecutive classes. A warp looks up to two
+// classes ahead for its next unit and requests that unit's list entries at once (class bounds and
+// list positions come from shared memory, so nothing waits); between its arrival at the class before
+// and its wait it draws the Philox words of its replicas and counts the slots that hold no literal
+// of the class still being updated, summed over the team. After the wait remain the last slots of
+// each lane, their sum over the team, the table lookups and the new word.
+//
+// Lane tl of a team resolves the replicas r = tl + TL k: their dE come out of the bit planes by one
+// shift and one masked merge per plane, and one ballot per k gives TL bits of each team's flips.
+// The Philox block of replicas 4g .. 4g + 3 is drawn by lane g TL / 8, its words handed round the
+// team by shuffles ahead of the wait.
+
+// What it measured (the kernel before it, with every load and draw after the barrier, in brackets):
+// N = 200, 64 replicas, one CTA a word, 8 lanes: 24.0 us a sweep (34.5); N = 5,000, 1,024 replicas,
+// 4 CTAs, 4 lanes: 61.4 (95.9); 6-SAT N = 8,678, 226 replicas, 8 CTAs, 4 lanes: 185 (334). Clock
+// reads at N = 5,000 put 1,000 - 1,700 of a class's 4,400 cycles in the release of the cluster
+// barrier, 350 - 500 in the late slots and 350 - 900 in the acceptance.
+
+// Slots per lane behind `pre` that are loaded ahead of the wait; lists with more (few classes) take
+// all their slots after it.
+template <int TL>
+__host__ __device__ constexpr int post_slots() { return 16 / TL; }
+
+// Words of shared memory for the class bounds and list positions of an instance (read from global
+// memory where an instance has more).
+constexpr int kMetaWords = 4096;
+
+constexpr int kLookAhead = 2;  // classes a warp looks ahead for its next unit
+
+// A warp's next unit and its state-independent loads.
+template <int KQ, int TL>
+struct TeamPrep {
+  int c, t;                   // class and sweep of the unit, or of the class to look on from
+  bool work;                  // a unit
+  int v0, c0, c1, cg, units;  // the CTA's share of that class
+  const int4 *ent;  // the lane's column of its group's interleaved list
+  int len, pre, regions;
+  bool late;
+  uint32_t bq, vo, first;  // first: the first slot's sign word
+  // k <= 4: the lane's first slots before and behind `pre` (two entries per slot would not fit)
+  int4 q[KQ == 1 ? 4 : 1], qp[KQ == 1 ? post_slots<TL>() : 1];
+};
+
+// What one slot adds to the counter: z, complemented where the own literal is negated.
+template <int KQ>
+__device__ __forceinline__ uint32_t slot_mask(const uint32_t *xs, const int4 &q, const int4 &q2) {
+  return ~others_or<KQ>(xs, q, q2) ^ sign_mask<0>((uint32_t)q.x);
+}
+
+// Adds the other lanes' counters of the team (A planes) in a butterfly: one plane more per stage,
+// at most 8 (two's complement).
+template <int TL, int A, int S = 1>
+__device__ __forceinline__ void team_sum(uint32_t (&c)[8]) {
+  if constexpr (S < TL) {
+    constexpr int N = A < 8 ? A + 1 : 8;
+    uint32_t p[A];
+#pragma unroll
+    for (int j = 0; j < A; ++j) p[j] = __shfl_xor_sync(0xFFFFFFFFu, c[j], S);
+    uint32_t carry = 0u;
+#pragma unroll
+    for (int j = 0; j < A; ++j) {
+      const uint32_t a = c[j];
+      c[j] = a ^ p[j] ^ carry;
+      carry = maj3b(a, p[j], carry);
+    }
+    if constexpr (A < 8) c[A] = carry;
+    team_sum<TL, N, 2 * S>(c);
+  }
+}
 
 template <int KQ, int CS, int TL, bool PT>
 __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
     ksat_team_kernel(const BatchItem *__restrict__ items, int n_items, int *next_item,
-                     const uint32_t *tab, int tab_len, int xs_words, int small_teams) {
+                     const uint32_t *tab, int tab_len, int xs_words, int meta_words) {
+  constexpr int kThreads = sweep_threads<KQ, TL>(), kWarps = kThreads / 32;
+  constexpr int VPW = 32 / TL;        // variables of a warp
+  constexpr int RPL = 32 / TL;        // replicas of a lane
+  constexpr int POST = post_slots<TL>();
   extern __shared__ __align__(16) uint32_t smem[];
   uint32_t *xs = smem;                               // word vector first (byte offsets in lists)
   uint32_t *tab_s = smem + ((xs_words + 31) & ~31);  // then the acceptance table
-  __shared__ int e_s[32], be_s[32], ep_s[32];
-  __shared__ uint32_t mult_s[32];
-  __shared__ SweepRows rows_s;
-  __shared__ uint32_t imp_s;
-  __shared__ int item_s;
-  __shared__ BatchItem item_b;
+  int *meta = reinterpret_cast<int *>(tab_s + tab_len + 1);  // then class bounds, list positions
+  __shared__ SweepShared sh;
   const int rank = CS == 1 ? 0 : (int)cg::this_cluster().block_rank();
   for (int i = threadIdx.x; i <= tab_len; i += blockDim.x) tab_s[i] = i < tab_len ? tab[i] : 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int tl = lane % TL;                       // lane inside the team
-  const int team = threadIdx.x / TL;              // team inside the CTA
-  const int nteams = blockDim.x / TL;
+  const int tl = lane % TL, team = lane / TL;
   while (true) {
-    if (rank == 0 && threadIdx.x == 0) item_s = atomicAdd(next_item, 1);
-    group_sync<CS>();
-    const int it = *rank_ptr<CS>(&item_s, 0);
-    if (it < n_items && threadIdx.x == 0) item_b = items[it];
-    group_sync<CS>();
-    if (it >= n_items) break;
-    const BatchItem &B = item_b;
+    if (!next_batch_item<CS>(items, n_items, next_item, rank, sh)) break;
+    const BatchItem &B = sh.item;
     const int n = B.n, W = B.W, w = B.w;
-    const int share = (n + CS - 1) / CS;
-    for (int v = threadIdx.x; v < n; v += blockDim.x) xs[v] = B.S[(size_t)(2 * v) * W + w];
-    if (threadIdx.x == 0) xs[n] = 0u;
-    if (threadIdx.x < 32) {
-      ep_s[threadIdx.x] = 0;
-      if (PT) mult_s[threadIdx.x] = B.mult[32 * w + threadIdx.x];
-      if (rank == 0) {
-        e_s[threadIdx.x] = B.energy[32 * w + threadIdx.x];
-        be_s[threadIdx.x] = B.best_energy[32 * w + threadIdx.x];
-      }
+    const int32_t inert_off = n * 4;
+    EnergyTrack track;
+    load_item<CS, PT>(B, rank, xs, sh, track);
+    uint32_t pm[PT ? RPL : 1];  // the lane's replicas' temperature multipliers
+    if (PT) {
+#pragma unroll
+      for (int k = 0; k < RPL; ++k) pm[k] = B.mult[32 * w + tl + TL * k];
     }
-    long long s1 = 0, s2 = 0;  // energy statistics of this lane's replica (rank 0, warp 0)
-    // Best states of the replicas that improve during this item go to a word-major staging row
-    // (the second half of the best buffer) at each improving sweep end, and into the [var][word]
-    // layout once, at the end of the item: a merge into that layout touches one 32-byte sector
-    // per variable, which at every improving sweep cost about 30 us per sweep on the 50,000-
-    // variable bench instance.
-    uint32_t *best_t = B.best + (size_t)n * W + (size_t)w * n;
-    uint32_t m_item = 0;  // replicas improved during this item
-    rows_s.fill(B, B.t0);
+    // [v0, v0 + n_units * VPW) of class [c0, c1): the CTA's contiguous share, in warp-sized units
+    auto share_of = [&](int c0, int c1, int &v0) {
+      const int part = ((c1 - c0 + CS - 1) / CS + VPW - 1) / VPW * VPW;
+      v0 = c0 + rank * part;
+      return max(0, (min(c1, v0 + part) - v0 + VPW - 1) / VPW);
+    };
+    const int nc = B.n_colours, G = B.n_groups;
+    const int32_t *col_ptr = B.col_ptr, *cgrp = B.cgrp, *grp = B.grp_base;
+    const bool staged = 2 * (nc + 1) + 2 * G + 1 <= meta_words;
+    if (staged) {
+      for (int i = threadIdx.x; i <= nc; i += blockDim.x) {
+        meta[i] = col_ptr[i];
+        meta[nc + 1 + i] = cgrp[i];
+      }
+      for (int i = threadIdx.x; i <= 2 * G; i += blockDim.x) meta[2 * (nc + 1) + i] = grp[i];
+      col_ptr = meta;
+      cgrp = meta + nc + 1;
+      grp = meta + 2 * (nc + 1);
+    }
+    __syncthreads();
+    TeamPrep<KQ, TL> P{};
+    auto load_slot = [&](int j, int end, int4 &q, int4 &q2) {
+      if (j < end) {
+        q = __ldg(P.ent + (size_t)(j * KQ) * 32);
+        if (KQ == 2) q2 = __ldg(P.ent + (size_t)(j * KQ + 1) * 32);
+      } else {  // inert: literal 1 always true
+        q = make_int4(1 << 15, inert_off, inert_off, inert_off);
+        if (KQ == 2) q2 = make_int4(inert_off, inert_off, inert_off, inert_off);
+      }
+    };
+    // requests the loads of unit `unit` of P's class
+    auto request = [&](int unit) {
+      const int v = P.v0 + unit * VPW + team;
+      P.len = 0;
+      P.bq = kFrozenQ16;
+      if (v < P.c1) {
+        const int off = v - P.c0, g = P.cg + (off >> 5);
+        const int gb = grp[g], ge = grp[g + 1];
+        P.bq = __ldg(B.bq + (size_t)P.t * n + v);
+        P.vo = (uint32_t)__ldg(B.orig + v);
+        P.regions = grp[G + 1 + g];
+        P.ent = B.occ_t + gb + (off & 31);
+        P.len = (ge - gb) / (32 * KQ);
+        if (P.len > 0) P.first = (uint32_t)__ldg(&P.ent->x);
+      }
+      // lists with more late slots than are kept in registers: everything after the wait
+      P.late = P.len - region_pre(P.regions) > POST * TL;
+      P.pre = P.len > 0 ? (P.late ? P.len : region_pre(P.regions)) : 0;
+      if (KQ == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) load_slot(tl + i * TL, P.pre, P.q[i], P.q[i]);
+#pragma unroll
+        for (int i = 0; i < POST; ++i) load_slot(P.pre + tl + i * TL, P.len, P.qp[i], P.qp[i]);
+      }
+    };
+    // finds the warp's next unit from class c of sweep t on: `mine` counts down over the units of
+    // the classes passed, and is the unit's number in the class found
+    int mine = warp;
+    auto seek = [&](int c, int t) {
+#pragma unroll 1
+      for (int left = kLookAhead;; --left) {
+        if (c == nc) {
+          c = 0;
+          ++t;
+        }
+        P.c = c;
+        P.t = t;
+        P.work = false;
+        if (t >= B.t1 || left == 0) return;
+        P.c0 = col_ptr[c];
+        P.c1 = col_ptr[c + 1];
+        P.cg = cgrp[c];
+        P.units = share_of(P.c0, P.c1, P.v0);
+        if (mine < P.units) break;
+        mine -= P.units;
+        ++c;
+      }
+      P.work = true;
+      request(mine);
+    };
+    seek(0, B.t0);
     group_sync<CS>();
     for (int t = B.t0; t < B.t1; ++t) {
-      int acc[32 / TL];
+      int acc[RPL];  // energy change of the lane's replicas
 #pragma unroll
-      for (int i = 0; i < 32 / TL; ++i) acc[i] = 0;
-      // class bounds and first group: for teams of 2 or 4 those of class c + 1 are requested
-      // during class c (the tiny classes of teams of 8 measured faster loading their own)
-      constexpr bool ahead = sweep_threads<KQ, TL>() == kTeamThreads;
-      int c0 = __ldg(B.col_ptr), c1 = __ldg(B.col_ptr + 1), cg = __ldg(B.cgrp);
-      for (int c = 0; c < B.n_colours; ++c) {
-        int c2 = 0, cgn = 0;
-        if (!ahead) {
-          c0 = __ldg(B.col_ptr + c);
-          c1 = __ldg(B.col_ptr + c + 1);
-          cg = __ldg(B.cgrp + c);
-        } else if (c + 1 < B.n_colours) {
-          c2 = __ldg(B.col_ptr + c + 2);
-          cgn = __ldg(B.cgrp + c + 1);
-        }
-        // contiguous shares here (measured: round-robin groups are slower for the teams)
-        const int part = ((c1 - c0 + CS - 1) / CS + 31) & ~31;
-        const int v0 = c0 + rank * part, v1 = min(c1, v0 + part);
-        // warp-uniform trip count: the warp's teams take consecutive variables each round
-        for (int vw = v0 + warp * (32 / TL); vw < v1; vw += nteams) {
-          const int v = vw + (lane / TL);
-          const bool active = v < v1;
-          const uint32_t xn =
-              attempt_team<KQ, TL, PT, (sweep_threads<KQ, TL>() == kTeamThreads)>(
-                  B, xs, tab_s, tab_len, mult_s, rows_s, cg, c0, v, active, t, tl, acc);
-          if (active && tl == 0) {
-            if (CS == 1) {
-              xs[v] = xn;
+      for (int k = 0; k < RPL; ++k) acc[k] = 0;
+      for (int c = 0; c < nc; ++c) {
+        bool waited = c == 0;  // a sweep starts with every word published
+        auto wait = [&]() {
+          if (!waited) {
+            __syncwarp();
+            class_wait();
+          }
+          waited = true;
+        };
+        if (P.c == c && P.t == t && !P.work) seek(c, t);
+        const bool here = P.c == c && P.t == t;
+        for (int unit = mine; here && unit < P.units; unit += kWarps) {
+          if (unit != mine) request(unit);
+          const int v = P.v0 + unit * VPW + team;
+          const bool go = v < P.c1;
+          const int len = P.len, pre = P.pre;
+          if (__any_sync(0xFFFFFFFFu, P.late)) wait();
+          // the lane's next four slots, which arrive behind the Philox blocks
+          int4 r[4], r2[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) load_slot((4 + i) * TL + tl, pre, r[i], r2[KQ == 2 ? i : 0]);
+          // Philox words of the replicas tl + TL k
+          uint32_t u[RPL];
+          {
+            const PhiloxCol col = philox_col(P.vo, kTagKsatSweep, B.k1);
+            constexpr int GPL = 8 / TL;  // groups this lane draws
+            uint4 own[GPL];
+#pragma unroll
+            for (int i = 0; i < GPL; ++i)
+              own[i] = philox4x32_meet(sh.rows.at(tl * GPL + i), col, B.k0, B.k1);
+#pragma unroll
+            for (int k = 0; k < RPL; ++k) {
+              // group (tl + TL k) / 4, word tl % 4 (TL is a multiple of 4)
+              const int src = TL == 8 ? 2 * k + (tl >> 2) : k >> 1;
+              const uint4 &o = own[TL == 8 ? 0 : k & 1];
+              const uint32_t a = __shfl_sync(0xFFFFFFFFu, o.x, src, TL),
+                             b = __shfl_sync(0xFFFFFFFFu, o.y, src, TL),
+                             d = __shfl_sync(0xFFFFFFFFu, o.z, src, TL),
+                             e = __shfl_sync(0xFFFFFFFFu, o.w, src, TL);
+              u[k] = (tl & 2) ? ((tl & 1) ? e : d) : ((tl & 1) ? b : a);
+            }
+          }
+          const uint32_t x = go ? xs[v] : 0u;
+          // the slots before `pre`, from -K on, summed over the team
+          uint32_t cnt[8];
+          {
+            const uint32_t k = tl == 0 && len > 0 ? 0u - marked_slots<KQ>(P.first) : 0u;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) cnt[j] = (uint32_t)((int)(k << (31 - j)) >> 31);
+            const int top = __reduce_max_sync(0xFFFFFFFFu, pre);
+            int4 q[4], q2[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if (KQ == 1) q[i] = P.q[i];
+              else load_slot(tl + i * TL, pre, q[i], q2[i]);
+            }
+#pragma unroll 1
+            for (int j = 0; j < top; j += 4 * TL) {
+              uint32_t z[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) z[i] = slot_mask<KQ>(xs, q[i], q2[KQ == 2 ? i : 0]);
+              csa4<8>(cnt, z[0], z[1], z[2], z[3]);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                q[i] = r[i];
+                if (KQ == 2) q2[i] = r2[i];
+              }
+              if (j + 8 * TL < top) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                  load_slot(j + (8 + i) * TL + tl, pre, r[i], r2[KQ == 2 ? i : 0]);
+              }
+            }
+            team_sum<TL, 8>(cnt);
+          }
+          int4 qp[POST], qp2[POST];
+#pragma unroll
+          for (int i = 0; i < POST; ++i) {
+            if (KQ == 1) qp[i] = P.qp[i];
+            else load_slot(pre + tl + i * TL, len, qp[i], qp2[i]);
+          }
+          const uint32_t bq = P.bq;
+          const bool free_ = go && bq != kFrozenQ16;  // a held variable takes no attempt
+          uint32_t beta[PT ? RPL : 1];
+          beta[0] = min(bq, (uint32_t)tab_len << 8);
+          if (PT) {
+#pragma unroll
+            for (int k = 0; k < RPL; ++k) beta[k] = pt_beta(pm[k], bq, tab_len);
+          }
+          wait();
+          // the remaining slots: at most POST per lane
+          {
+            uint32_t z[POST], p[8];
+#pragma unroll
+            for (int i = 0; i < POST; ++i) z[i] = slot_mask<KQ>(xs, qp[i], qp2[KQ == 2 ? i : 0]);
+            if constexpr (POST == 2) {
+              p[0] = z[0] ^ z[1];
+              p[1] = z[0] & z[1];
+              team_sum<TL, 2>(p);
             } else {
-              const uint32_t sa = (uint32_t)__cvta_generic_to_shared(xs + v);
+              const uint32_t s = z[0] ^ z[1] ^ z[2], m = maj3b(z[0], z[1], z[2]), g = s & z[3];
+              p[0] = s ^ z[3];
+              p[1] = m ^ g;
+              p[2] = m & g;
+              team_sum<TL, 3>(p);
+            }
+            uint32_t carry = 0u;  // at most 16 slots: 5 planes
 #pragma unroll
-              for (int r = 0; r < CS; ++r) st_rank(sa, r, xn);
+            for (int j = 0; j < 8; ++j) {
+              const uint32_t a = cnt[j], b = j < 5 ? p[j] : 0u;
+              cnt[j] = a ^ b ^ carry;
+              carry = maj3b(a, b, carry);
+            }
+          }
+          // dE planes, negated where x = 0; byte i of de[h]: replica tl + h TL + 8 i
+          uint32_t de[8 / TL] = {};
+          {
+            uint32_t carry = ~x;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const uint32_t y = cnt[j] ^ ~x, d = y ^ carry;
+              carry = y & carry;
+#pragma unroll
+              for (int h = 0; h < 8 / TL; ++h)
+                de[h] |= ((d >> (tl + h * TL)) << j) & (0x01010101u << j);
+            }
+          }
+          // every lookup before the first test: none depends on another, and none is skipped
+          uint32_t th[RPL];
+          int val[RPL];
+#pragma unroll
+          for (int k = 0; k < RPL; ++k) {
+            const uint32_t b8 = byte_of(de[TL == 8 ? 0 : k & 1], TL == 8 ? k : k >> 1);
+            val[k] = (int)(signed char)b8;
+            th[k] = tab_s[table_index(beta[PT ? k : 0], b8, tab_len)];
+          }
+          uint32_t flip = 0u;
+#pragma unroll
+          for (int k = 0; k < RPL; ++k) {
+            const bool ok = free_ & ((val[k] <= 0) | (u[k] < th[k]));
+            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, ok);
+            flip |= ((votes >> (team * TL)) & ((1u << TL) - 1u)) << (TL * k);
+            acc[k] += ok ? val[k] : 0;
+          }
+          if (flip) {
+            if (CS == 1) {
+              if (tl == 0) xs[v] = x ^ flip;
+            } else if (tl < CS) {
+              st_rank((uint32_t)__cvta_generic_to_shared(xs + v), tl, x ^ flip);
+              if (CS > TL) st_rank((uint32_t)__cvta_generic_to_shared(xs + v), tl + TL, x ^ flip);
             }
           }
         }
-        group_sync<CS>();
-        c0 = c1;
-        c1 = c2;
-        cg = cgn;
-      }
+        wait();
+        if (c + 1 == nc) {  // the sweep's energy changes, published with its last class
 #pragma unroll
-      for (int i = 0; i < 32 / TL; ++i)
-        if (acc[i] != 0) atomicAdd(&ep_s[4 * (tl * (8 / TL) + i / 4) + (i & 3)], acc[i]);
-      group_sync<CS>();
-      if (rank == 0 && warp == 0) {
-        int sum = e_s[lane];
+          for (int k = 0; k < RPL; ++k) {
+            int s = acc[k];
 #pragma unroll
-        for (int r = 0; r < CS; ++r) sum += rank_ptr<CS>(ep_s, r)[lane];
-        e_s[lane] = sum;
-        if (PT && B.stats && t >= B.stats_t0) {
-          s1 += sum;
-          s2 += (long long)sum * sum;
+            for (int o = TL; o < 32; o <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+            if (team == 0 && s != 0) atomicAdd(&sh.ep[t & 1][tl + TL * k], s);
+          }
         }
-        const bool better = sum < be_s[lane];
-        if (better) be_s[lane] = sum;
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, better);
-        if (lane == 0) imp_s = m;
-      }
-      group_sync<CS>();
-      const uint32_t m = *rank_ptr<CS>(&imp_s, 0);
-      if (threadIdx.x < 32) ep_s[threadIdx.x] = 0;
-      rows_s.fill(B, t + 1);
-      __syncthreads();
-      if (m) {  // the improved replicas' states, into this word's staging row (coalesced)
-        const int b0 = rank * share, b1 = min(n, b0 + share);
-        for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x)
-          best_t[v] = (best_t[v] & ~m) | (xs[v] & m);
-        m_item |= m;
-        group_sync<CS>();
-      }
-    }
-    {
-      const int b0 = rank * share, b1 = min(n, b0 + share);
-      for (int v = b0 + threadIdx.x; v < b1; v += blockDim.x) {
-        B.S[(size_t)(2 * v) * W + w] = xs[v];
-        B.S[(size_t)(2 * v + 1) * W + w] = ~xs[v];
-        if (m_item) {  // replicas improved during the item: their last best state from staging
-          const size_t bi = (size_t)v * W + w;
-          B.best[bi] = (B.best[bi] & ~m_item) | (best_t[v] & m_item);
+        __syncwarp();
+        class_arrive<CS>();
+        if (here) {
+          mine -= P.units;
+          while (mine < 0) mine += kWarps;
+          seek(c + 1, t);
         }
       }
+      class_wait();
+      end_sweep<CS, PT>(B, rank, t, xs, sh, track);
     }
-    if (rank == 0 && threadIdx.x < 32) {
-      B.energy[32 * w + threadIdx.x] = e_s[threadIdx.x];
-      B.best_energy[32 * w + threadIdx.x] = be_s[threadIdx.x];
-      if (PT && B.stats) {  // one item per word in a launch: plain read-modify-write
-        B.stats[32 * w + threadIdx.x] += s1;
-        B.stats[32 * (B.W + w) + threadIdx.x] += s2;
-      }
-    }
+    store_item<CS, PT>(B, rank, xs, track);
     group_sync<CS>();
   }
-  (void)team;
-  (void)small_teams;
 }
 
 // The launch shape of each kernel instance is queried once per (device, shared-memory size):
@@ -1073,7 +1252,14 @@ cudaError_t launch_batch(const BatchItem *items, int n_items, int *next_item,
                          const uint32_t *tab, int tab_len, int max_n, int device,
                          cudaStream_t st) {
   const int xs_words = max_n + 1;
-  const size_t smem = sizeof(uint32_t) * (((size_t)xs_words + 31) / 32 * 32 + (size_t)tab_len + 1);
+  size_t words = ((size_t)xs_words + 31) / 32 * 32 + (size_t)tab_len + 1;
+  int meta_words = 0;
+  if (TL > 1) {  // what room there is beside the vector and the table, up to kMetaWords
+    const long long room = (long long)batch_max_vars(tab_len, device) - max_n;
+    meta_words = (int)std::max(0LL, std::min((long long)kMetaWords, room));
+    words += meta_words;
+  }
+  const size_t smem = sizeof(uint32_t) * words;
   auto kern = TL == 1 ? ksat_batch_kernel<KQ, CS, PT> : ksat_team_kernel<KQ, CS, (TL > 1 ? TL : 4), PT>;
   constexpr int threads = sweep_threads<KQ, TL>();
   static std::mutex mu;
@@ -1152,7 +1338,8 @@ cudaError_t launch_batch(const BatchItem *items, int n_items, int *next_item,
   cfg.gridDim = dim3(clusters * CS);
   cudaError_t err = cudaMemsetAsync(next_item, 0, sizeof(int), st);
   if (err != cudaSuccess) return err;
-  return cudaLaunchKernelEx(&cfg, kern, items, n_items, next_item, tab, tab_len, xs_words, small_teams);
+  return cudaLaunchKernelEx(&cfg, kern, items, n_items, next_item, tab, tab_len, xs_words,
+                            TL > 1 ? meta_words : small_teams);
 }
 
 // Lanes per variable of the batched kernel: 1 (one thread per variable) or a team of 4 or 8.
