@@ -271,29 +271,30 @@ double ksat_sweep_us(int32_t n, int32_t n_colours) {
   const double per_class = std::max(1.0, n / nc);
   const double rounds = std::ceil(per_class / 512.0);
   const double last = per_class - 512.0 * (rounds - 1.0);  // variables in the last round
-  const double cycles = nc * (2200.0 + 16000.0 * (rounds - 1.0) + 27.0 * last);
+  const double cycles = nc * (2900.0 + 12000.0 * (rounds - 1.0) + 20.0 * last);
   return cycles / 2070.0;  // SM clock in MHz
+}
+
+// Teams of 8 lanes up to ~8 variables of a class on a CTA, of 4 up to ~64, single threads beyond
+// (us a sweep with 8, 4 and 1 lanes: 200 variables on one CTA 24.0, 25.4, 62.2; 10,007 on 8, 43 a
+// class, 84, 62.7, 85.7; the same on 4, 86 a class, 142, 104, 89.9; 20,001 on 4, 178 a class, 268,
+// 178, 104).
+int choose_lanes(int cs, int per_class) {
+  const int per_cta = per_class / cs;
+  return per_cta <= 8 ? 8 : (per_cta <= 64 ? 4 : 1);
 }
 
 double qap_step_us(int32_t n) { return 0.008 * static_cast<double>(n) * n + 1.0; }
 
-// CTAs per work item: few items are spread over the SMs (each cluster keeps its own copy of the
-// word vector), but a colour class is not split below about 32 variables per CTA, where a
-// cluster barrier per class costs more than the work it spreads (measured: 4-SAT N = 200 with 64
-// replicas, 43 us per sweep on one CTA per word against 78 on eight; N = 1,000 with 256, 82
-// against 105 on eight; N = 5,000 with 1,024 keeps four, 132 us).
-int choose_ctas(int sms, long long cnt, int per_class) {
-  int cs = 1;
-  while (cs < 8 && cnt * cs * 2 <= sms && per_class >= 64 * cs) cs *= 2;
-  return cs;
-}
-
-// Lanes per variable for about per_class / cs variables of a class on each CTA: teams of 8 up
-// to ~24, of 4 up to ~100, single threads beyond (the one-thread kernel still runs its smaller
-// classes with teams).
-int choose_lanes(int cs, int per_class) {
-  const int per_cta = per_class / cs;
-  return per_cta <= 24 ? 8 : (per_cta <= 100 ? 4 : 1);
+// CTAs per work item: the most whose clusters run all items at once (a second round of clusters
+// doubles the time: 20,001 variables with 16 words, 155 us a sweep on 2 CTAs a word, 104 on 4, 176 on
+// 8, of which 15 clusters fit) and that leave about four variables of a class to a CTA (1,000
+// variables, 8 words: 40.8, 39.9, 37.5, 33.5 us on 1, 2, 4, 8); with fewer variables a class the
+// cluster's barrier costs more than the split saves (200 variables, 2 words: 24.0, 32.0, 30.8, 30.9).
+int choose_ctas(int device, long long cnt, int per_class) {
+  for (int cs = 8; cs > 1; cs /= 2)
+    if (per_class >= 24 && per_class >= 4 * cs && cnt <= batch_clusters(cs, device)) return cs;
+  return 1;
 }
 
 int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t0,
@@ -351,11 +352,6 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
     }
     per_class[q] = std::max(per_class[q], class_size(*I));
   }
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(ctx, NMC_ECUDA, "query SMs");
-  }
   plan->items.clear();
   for (int q = 0; q < 2; ++q) {
     std::vector<size_t> idx(by_kq[q].size());
@@ -373,7 +369,7 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
       cs = tuned->second.first;
       lanes = tuned->second.second;
     } else {
-      cs = choose_ctas(sms, plan->cnt[q], per_class[q]);
+      cs = choose_ctas(ctx->device, plan->cnt[q], per_class[q]);
       lanes = choose_lanes(cs, per_class[q]);
     }
     if (cs != 1 && cs != 2 && cs != 4 && cs != 8) cs = 1;
@@ -484,12 +480,7 @@ void tuned_shape(nmc_ctx *ctx, const Instance &I, int cnt, int *cs, int *lanes) 
     *lanes = t->second.second;
     return;
   }
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
-    cudaGetLastError();
-    sms = 1;
-  }
-  int c = choose_ctas(sms, cnt, class_size(I));
+  int c = choose_ctas(ctx->device, cnt, class_size(I));
   if (const char *env = getenv("NMC_BATCH_CTAS")) c = atoi(env);
   if (c != 1 && c != 2 && c != 4 && c != 8) c = 1;
   *cs = c;

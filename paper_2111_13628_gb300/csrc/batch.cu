@@ -4,14 +4,13 @@
 // Work item = (replica set, word w of 32 replicas, sweep range). A cluster of CS CTAs takes
 // items from a device counter; each CTA loads the item's word vector x[0..n) into its shared
 // memory, runs the sweeps with the variables of one colour class spread over the cluster's
-// threads (one thread, or a team of 2, 4 or 8 lanes, per variable for the 32 replicas of the
-// word), stores every new word into all CS copies, and meets the cluster barrier between
-// classes; the next class's bounds are requested before that barrier. Words are independent
-// chains, so no grid-wide synchronisation is needed and uneven instances fill the GPU. The
-// dynamics are identical to the single-instance kernels. Occurrence lists are read in a
-// warp-interleaved layout (one coalesced load per occurrence for 32 variables); each thread
-// keeps its share of the sweep's energy change as 16 bit-sliced planes and converts them to
-// per-replica sums once per sweep.
+// threads (one thread per variable, or a team of 4 or 8 lanes where a class has few variables on a
+// CTA, for the 32 replicas of the word), stores every new word into all CS copies, and meets the
+// other CTAs between classes. Words are independent chains, so no grid-wide synchronisation is
+// needed and uneven instances fill the GPU. The dynamics are identical to the single-instance
+// kernels. Occurrence lists are read in a warp-interleaved layout (one coalesced load per
+// occurrence for 32 variables); a thread of the one-thread kernel keeps its share of the sweep's
+// energy change as 16 bit-sliced planes and converts them to per-replica sums once per sweep.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -182,18 +181,6 @@ __device__ __forceinline__ uint32_t others_or(const uint32_t *xs, const int4 &q,
          (xs_at(xs, q2.z) ^ sign_mask<2>(s6)) | (xs_at(xs, q2.w) ^ sign_mask<3>(s6));
   }
   return o;
-}
-
-// Adds the bit-sliced counter p into c (ripple carry).
-template <int NB>
-__device__ __forceinline__ void add_planes(uint32_t (&c)[NB], const uint32_t (&p)[NB]) {
-  uint32_t carry = 0u;
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    const uint32_t a = c[j], b = p[j];
-    c[j] = a ^ b ^ carry;
-    carry = maj3b(a, b, carry);
-  }
 }
 
 // The loads of one attempt that do not depend on the replicas' states: the variable's Q16
@@ -388,127 +375,6 @@ __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint3
   return x ^ flip;
 }
 
-// ---- small classes of the one-thread kernel: TL lanes per variable -------------------------------
-//
-// Same dynamics, shorter critical path: a team of TL consecutive lanes evaluates one variable.
-// Lane t of the team takes occurrences t, t+TL, ... of the variable's list, counts its break /
-// make masks in bit-sliced counters, and the team adds its TL partial counters with an xor
-// butterfly of shuffles, so every lane ends with the totals. Lane t then resolves the
-// acceptance of replica groups [t*8/TL, (t+1)*8/TL) (one Philox block per group of 4 replicas)
-// and the team ORs the flip bits. A colour class of a few hundred variables then costs the
-// latency of a TL-th of one attempt instead of a whole one.
-template <int KQ, int TL, bool PT>
-__device__ __forceinline__ uint32_t attempt_team(const BatchItem &B, const uint32_t *xs,
-                                                 const uint32_t *tab_s, int tab_len,
-                                                 const uint32_t *mult_s, const SweepRows &rows,
-                                                 int cg, int c0, int v, bool active, int t, int tl,
-                                                 int (&acc)[32 / TL]) {
-  constexpr int NB = 7;
-  const uint32_t x = active ? xs[v] : 0u;
-  const uint32_t bqv = active ? __ldg(B.bq + (size_t)t * B.n + v) : 0u;
-  // a held variable takes no attempt; the team still joins the shuffles below
-  const bool frozen = bqv == kFrozenQ16;
-  uint32_t bc[NB], mc[NB];
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    bc[j] = 0u;
-    mc[j] = 0u;
-  }
-  int len = 0;
-  const int4 *ent = nullptr;
-  if (active && !frozen) {
-    const int off = v - c0;
-    const int g = cg + (off >> 5), ln = off & 31;  // cg: the class's first group
-    const int gb = __ldg(B.grp_base + g);
-    len = (__ldg(B.grp_base + g + 1) - gb) / (32 * KQ);
-    ent = B.occ_t + gb + ln;
-  }
-  {
-    // each group's entries loaded where they are evaluated
-    for (int j0 = tl; j0 < len; j0 += 4 * TL) {
-      uint32_t bb[4], mm[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int j = j0 + i * TL;
-        bb[i] = 0u;
-        mm[i] = 0u;
-        if (j < len) {
-          const int4 q = __ldg(ent + (size_t)(j * KQ) * 32);
-          const int4 q2 = KQ == 2 ? __ldg(ent + (size_t)(j * KQ + 1) * 32) : q;
-          const uint32_t o = others_or<KQ>(xs, q, q2);
-          const uint32_t own = x ^ sign_mask<0>((uint32_t)q.x);
-          bb[i] = own & ~o;
-          mm[i] = ~(own | o);
-        }
-      }
-      csa4<NB>(bc, bb[0], bb[1], bb[2], bb[3]);
-      csa4<NB>(mc, mm[0], mm[1], mm[2], mm[3]);
-    }
-  }
-#pragma unroll
-  for (int sft = 1; sft < TL; sft <<= 1) {
-    uint32_t pb[NB], pm[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      pb[j] = __shfl_xor_sync(0xFFFFFFFFu, bc[j], sft);
-      pm[j] = __shfl_xor_sync(0xFFFFFFFFu, mc[j], sft);
-    }
-    add_planes<NB>(bc, pb);
-    add_planes<NB>(mc, pm);
-  }
-  uint32_t d[NB + 1];
-  {
-    uint32_t br = 0u;
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      d[j] = bc[j] ^ mc[j] ^ br;
-      br = maj3b(~bc[j], mc[j], br);
-    }
-    d[NB] = br;
-  }
-  const PhiloxCol col =
-      philox_col(active ? (uint32_t)__ldg(B.orig + v) : 0u, kTagKsatSweep, B.k1);
-  const uint32_t bqc = min(bqv, (uint32_t)tab_len << 8);
-  constexpr int GPL = 8 / TL;             // Philox groups (4 replicas) per lane
-  constexpr int NBK = GPL >= 2 ? GPL / 2 : 1;  // blocks of 8 replicas the lane's groups lie in
-  // one 8x8 transpose of the 8 planes of D per block gives the replicas' signed bytes
-  unsigned long long xmb[NBK];
-#pragma unroll
-  for (int b = 0; b < NBK; ++b) xmb[b] = transpose8(gather_bytes(d, ((tl * GPL) >> 1) + b));
-  uint32_t flip = 0u;
-  // the lane's Philox groups, drawn always (as in accept_batch)
-  int de[4 * GPL];
-  uint32_t th[4 * GPL];
-#pragma unroll
-  for (int gi = 0; gi < GPL; ++gi) {
-    const int g = tl * GPL + gi;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = 4 * g + j;
-      const int val = (int)(signed char)(unsigned char)(xmb[gi >> 1] >> (8 * (r & 7)));
-      de[4 * gi + j] = val;
-      const uint32_t b = PT ? pt_beta(mult_s[r], bqv, tab_len) : bqc;
-      th[4 * gi + j] = tab_s[table_index(b, (uint32_t)val & 255u, tab_len)];
-    }
-  }
-#pragma unroll
-  for (int gi = 0; gi < GPL; ++gi) {
-    const int g = tl * GPL + gi;
-    const uint4 u = philox4x32_meet(rows.at(g), col, B.k0, B.k1);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = 4 * gi + j;
-      const bool ok = de[i] <= 0 || uint4_word(u, j) < th[i];
-      flip |= (uint32_t)ok << (4 * g + j);
-      if (active) acc[i] += ok ? de[i] : 0;
-    }
-  }
-  if (frozen) flip = 0u;  // zero counters read as dE = 0: cancel those flips
-#pragma unroll
-  for (int sft = 1; sft < TL; sft <<= 1) flip |= __shfl_xor_sync(0xFFFFFFFFu, flip, sft);
-  return x ^ flip;
-}
-
 // A colour class [c0, c1) is shared out among the CS CTAs of a cluster by 32-variable groups,
 // round-robin: CTA `rank` takes groups rank, rank + CS, ... Variables are degree-descending
 // inside a class, so each CTA gets a like mix of long and short occurrence lists (contiguous
@@ -576,38 +442,6 @@ template <int CS, typename T>
 __device__ __forceinline__ T *rank_ptr(T *p, int r) {
   if (CS == 1) return p;
   return cg::this_cluster().map_shared_rank(p, r);
-}
-
-// A colour class whose share on this CTA is cnt <= blockDim / TT variables: team `team` (TT
-// consecutive lanes) updates local variable `team` (the same round-robin share as the one-thread
-// path) with attempt_team, stores its new word to every copy of the cluster, and adds its
-// replicas' energy changes to ep_s. Warps with no team in range skip the class.
-template <int KQ, int CS, int TT, bool PT>
-__device__ __forceinline__ void class_teams(const BatchItem &B, uint32_t *xs, const uint32_t *tab_s,
-                                            int tab_len, const uint32_t *mult_s,
-                                            const SweepRows &rows, int cg, int c0, int cnt, int rank, int t, int *ep_s) {
-  const int lane = threadIdx.x & 31;
-  if ((int)(threadIdx.x & ~31u) / TT >= cnt) return;  // the whole warp
-  const int team = threadIdx.x / TT, tl = lane % TT;
-  const bool active = team < cnt;
-  const int v = active ? share_var<CS>(c0, rank, team) : c0;
-  int tacc[32 / TT];
-#pragma unroll
-  for (int i = 0; i < 32 / TT; ++i) tacc[i] = 0;
-  const uint32_t xn = attempt_team<KQ, TT, PT>(B, xs, tab_s, tab_len, mult_s, rows, cg, c0, v,
-                                                  active, t, tl, tacc);
-  if (active && tl == 0) {
-    if (CS == 1) {
-      xs[v] = xn;
-    } else {
-      const uint32_t sa = (uint32_t)__cvta_generic_to_shared(xs + v);
-#pragma unroll
-      for (int r = 0; r < CS; ++r) st_rank(sa, r, xn);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 32 / TT; ++i)
-    if (tacc[i] != 0) atomicAdd(&ep_s[4 * (tl * (8 / TT) + i / 4) + (i & 3)], tacc[i]);
 }
 
 // ---- what both sweep kernels share --------------------------------------------------------------
@@ -732,7 +566,7 @@ __device__ __forceinline__ void store_item(const BatchItem &B, int rank, const u
 template <int KQ, int CS, bool PT>
 __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
     ksat_batch_kernel(const BatchItem *__restrict__ items, int n_items, int *next_item,
-                      const uint32_t *tab, int tab_len, int xs_words, int small_teams) {
+                      const uint32_t *tab, int tab_len, int xs_words, int) {
   extern __shared__ __align__(16) uint32_t smem[];
   uint32_t *xs = smem;                               // word vector first (byte offsets in lists)
   uint32_t *tab_s = smem + ((xs_words + 31) & ~31);  // then the acceptance table
@@ -753,13 +587,11 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
       // class bounds and first group: those of class c + 1 are requested during class c and
       // arrive behind its barrier
       int c0 = __ldg(B.col_ptr), c1 = __ldg(B.col_ptr + 1), cg = __ldg(B.cgrp);
-      // a share of a class with at most this many variables on the CTA runs with teams of lanes
       constexpr int kThreads = one_thread_threads<KQ>();
-      const int team_max = small_teams ? kThreads / 2 : -1;
       // the state-independent loads of this thread's first variable of each class: requested
       // for class c + 1 between the two halves of the barrier that ends class c
       // (every thread loads, those without a variable in the class for variable c0, so that
-      // P is written before every class and never live across the team path)
+      // P is written before every class)
       AttemptPrep<KQ> P;
       // the warp's group of the class's share (its first round): dealt on from class to class,
       // so that the warps left without a group, and those with the longest lists, change
@@ -767,7 +599,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
       int mygrp = warp;
       {
         const int cnt0 = share_count<CS>(c0, c1, rank);
-        const bool mine = cnt0 > team_max && (int)threadIdx.x < cnt0;
+        const bool mine = (int)threadIdx.x < cnt0;
         prep_attempt<KQ>(B, cg, c0, mine ? share_var<CS>(c0, rank, threadIdx.x) : c0, t, P);
       }
       for (int c = 0; c < B.n_colours; ++c) {
@@ -780,20 +612,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         // CTA's share of them to its warps
         const int cnt = share_count<CS>(c0, c1, rank);
         const int ngr = (cnt + 31) >> 5;
-        if (cnt <= team_max) {
-          if (c > 0) class_wait();
-          // a smaller share (the later colour classes): teams of 8, 4 or 2 lanes per variable
-          // shorten the class's critical path; their energy changes go to ep_s directly
-          if (cnt <= kThreads / 8)
-            class_teams<KQ, CS, 8, PT>(B, xs, tab_s, tab_len, sh.mult, sh.rows, cg, c0, cnt,
-                                         rank, t, sh.ep[t & 1]);
-          else if (cnt <= kThreads / 4)
-            class_teams<KQ, CS, 4, PT>(B, xs, tab_s, tab_len, sh.mult, sh.rows, cg, c0, cnt,
-                                         rank, t, sh.ep[t & 1]);
-          else
-            class_teams<KQ, CS, 2, PT>(B, xs, tab_s, tab_len, sh.mult, sh.rows, cg, c0, cnt,
-                                         rank, t, sh.ep[t & 1]);
-        } else {
+        {
           auto store = [&](int v, uint32_t xn) {
             if (CS == 1) {
               xs[v] = xn;
@@ -863,7 +682,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         if (c + 1 < B.n_colours) {
           const int cntn = share_count<CS>(c1, c2, rank), ln = 32 * mygrp + lane;
           prep_attempt<KQ>(B, cgn, c1,
-                           cntn > team_max && ln < cntn ? share_var<CS>(c1, rank, ln) : c1, t, P);
+                           ln < cntn ? share_var<CS>(c1, rank, ln) : c1, t, P);
         }
         c0 = c1;
         c1 = c2;
@@ -1264,7 +1083,6 @@ cudaError_t launch_batch(const BatchItem *items, int n_items, int *next_item,
   constexpr int threads = sweep_threads<KQ, TL>();
   static std::mutex mu;
   static std::map<std::pair<int, size_t>, int> shapes;  // (device, smem) -> resident clusters
-  static std::map<int, int> sm_count;                    // device -> SMs
   static std::map<int, size_t> smem_set;                // device -> largest smem attribute set
   int clusters = 0;
   {
@@ -1307,22 +1125,6 @@ cudaError_t launch_batch(const BatchItem *items, int n_items, int *next_item,
     }
   }
   if (clusters < 1) return cudaErrorInvalidConfiguration;
-  int sms = 0;
-  {
-    std::lock_guard<std::mutex> g(mu);
-    auto it = sm_count.find(device);
-    if (it == sm_count.end()) {
-      cudaError_t err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-      if (err != cudaSuccess) return err;
-      sm_count[device] = sms;
-    } else {
-      sms = it->second;
-    }
-  }
-  // Teams of lanes for the smaller colour classes shorten a class's critical path; they pay
-  // off when each SM runs one CTA of the launch (latency-bound), not when many items queue
-  // behind each other (measured on a 256-instance batch: 3% slower with them).
-  const int small_teams = (long long)n_items * CS <= sms ? 1 : 0;
   if (clusters > n_items) clusters = n_items;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(threads);
@@ -1339,26 +1141,22 @@ cudaError_t launch_batch(const BatchItem *items, int n_items, int *next_item,
   cudaError_t err = cudaMemsetAsync(next_item, 0, sizeof(int), st);
   if (err != cudaSuccess) return err;
   return cudaLaunchKernelEx(&cfg, kern, items, n_items, next_item, tab, tab_len, xs_words,
-                            TL > 1 ? meta_words : small_teams);
+                            meta_words);
 }
 
 // Lanes per variable of the batched kernel: 1 (one thread per variable) or a team of 4 or 8.
-// Few variables per CTA per colour class favour teams (latency), many favour single threads.
 int batch_lanes(int cs, int max_n, int want) {
   if (const char *env = getenv("NMC_BATCH_LANES")) {
     const int l = atoi(env);
     if (l == 1 || l == 4 || l == 8) return l;
   }
   if (want == 1 || want == 4 || want == 8) return want;  // a tuned shape
-  // variables of one colour class per CTA, taking ~32 classes. Measured on 4-SAT (alpha ~9.9,
-  // 640 threads): teams of 8 lanes win up to ~24 variables per CTA and class, teams of 4 up to
-  // ~100 (5,000 variables over 4-CTA clusters: 151 us per sweep vs 160 with 8 lanes and 227
-  // with 1), single threads beyond (20,000 variables over 4-CTA clusters: 253 vs 277 with 4).
-  const int per_cta = max_n / (32 * cs);
-  if (per_cta <= 24) return 8;
-  if (per_cta <= 100) return 4;
-  return 1;
+  return choose_lanes(cs, max_n / 32);  // taking ~32 classes
 }
+
+// Stands in for the sweep kernels when the number of resident clusters is asked for.
+template <int CS>
+__global__ void cluster_probe_kernel() {}
 
 template <int KQ, int CS>
 cudaError_t dispatch_lanes(const BatchItem *items, int n_items, int *next_item, const uint32_t *tab,
@@ -1390,6 +1188,42 @@ cudaError_t dispatch_batch(int cs, const BatchItem *items, int n_items, int *nex
 }
 
 }  // namespace
+
+// Clusters of cs CTAs that run at once, one CTA per SM: clusters do not span a GPC, so this is less
+// than SMs / cs (152 SMs: 76, 36 and 15 clusters of 2, 4 and 8).
+int batch_clusters(int cs, int device) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> known;
+  std::lock_guard<std::mutex> g(mu);
+  const auto it = known.find({cs, device});
+  if (it != known.end()) return it->second;
+  int n = 0;
+  const size_t smem = 128 * 1024;  // more than half of an SM's
+  cudaLaunchConfig_t q = {};
+  q.blockDim = dim3(kTeamThreads);
+  q.dynamicSmemBytes = smem;
+  q.gridDim = dim3(cs * 256);
+  cudaLaunchAttribute a[1];
+  a[0].id = cudaLaunchAttributeClusterDimension;
+  a[0].val.clusterDim.x = cs;
+  a[0].val.clusterDim.y = 1;
+  a[0].val.clusterDim.z = 1;
+  q.attrs = a;
+  q.numAttrs = 1;
+  const auto query = [&](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+               cudaSuccess &&
+           cudaOccupancyMaxActiveClusters(&n, kern, &q) == cudaSuccess;
+  };
+  const bool ok = cs == 2 ? query(cluster_probe_kernel<2>)
+                          : (cs == 4 ? query(cluster_probe_kernel<4>) : query(cluster_probe_kernel<8>));
+  if (!ok) {
+    cudaGetLastError();
+    n = 0;
+  }
+  known[{cs, device}] = n;
+  return n;
+}
 
 // ---- batched sweep without any allocation ----------------------------------------------------
 //

@@ -133,6 +133,10 @@ cudaError_t quantize_schedule(const float *beta, int32_t n_units, int32_t n_step
 // ---- batched k-SAT (batch.cu) -----------------------------------------------------------
 // Largest n whose word vector fits the batched kernel's shared memory on `device`.
 size_t batch_max_vars(int tab_len, int device);
+// Clusters of cs (2, 4, 8) CTAs that run at once on `device` with one CTA per SM.
+int batch_clusters(int cs, int device);
+// Lanes per variable for about per_class / cs variables of a colour class on each CTA.
+int choose_lanes(int cs, int per_class);
 // Runs n_items items (all of one occurrence width kq) in one launch with cs CTAs (1, 2, 4, 8)
 // per item; next_item is a device int. With pt, every item carries temperature multipliers
 // (mult) and may carry energy statistics. lanes: lanes per variable (1, 4, 8; 0 = the built-in
@@ -140,8 +144,8 @@ size_t batch_max_vars(int tab_len, int device);
 // Estimated GPU time, in microseconds, of one sweep of one 32-replica word of a k-SAT instance
 // with n variables in n_colours classes on one CTA (the shape of a launch with many items): per
 // class a latency floor plus the variables' share of a 512-thread round, rounds beyond 512
-// variables in full (from measured sweeps: ~2.4k cycles per class of a few variables, ~16k per
-// full round). Used to order work items and to size serving slices by time, not for results.
+// variables in full (from measured 4-SAT sweeps on one CTA: 89, 137 and 251 us at 5,000, 10,007 and
+// 20,001 variables). Used to order work items and to size serving slices by time, not for results.
 double ksat_sweep_us(int32_t n, int32_t n_colours);
 // The same for one swap step (n attempts) of one 32-replica block of a QAP instance.
 double qap_step_us(int32_t n);
