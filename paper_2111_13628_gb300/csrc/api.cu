@@ -42,6 +42,7 @@ struct ReplicaSet {
   uint64_t seed = 0;
   KsatReplicas ks{};
   QapReplicas qp{};
+  bool clusters = false;  // k-SAT: last launched with several CTAs per word
   // temperature ladder (k-SAT replica exchange); pt_L = 0 without one
   int32_t pt_L = 0;
   uint32_t *pt_lq = nullptr;    // pt_L Q16 inverse temperatures of the slots
@@ -196,6 +197,15 @@ ReplicaSet *find_set(nmc_ctx *ctx, int32_t id) {
 // Checks the sticky timeout word of a k-SAT replica set after its stream was synchronised.
 int check_timeout(nmc_ctx *ctx, ReplicaSet &S) {
   if (!S.ks.bar) return NMC_OK;
+  if (S.clusters) {
+    int32_t status = 0;
+    int32_t *at = S.ks.best_energy + 32 * S.ks.W;
+    NMC_CUDA(cudaMemcpy(&status, at, sizeof(int32_t), cudaMemcpyDeviceToHost), "read step status");
+    if (status == kStepTimeout) {
+      cudaMemset(at, 0, sizeof(int32_t));
+      return fail(ctx, NMC_ETIMEOUT, "a wait between the CTAs of a word expired; the sweep is void");
+    }
+  }
   int sticky = 0;
   NMC_CUDA(cudaMemcpy(&sticky, &S.ks.bar->sticky, sizeof(int), cudaMemcpyDeviceToHost),
            "read barrier status");
@@ -375,6 +385,10 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
     if (cs != 1 && cs != 2 && cs != 4 && cs != 8) cs = 1;
     plan->cs[q] = cs;
     plan->lanes[q] = lanes;
+    for (int32_t i = 0; i < n_sets; ++i) {
+      ReplicaSet *S = find_set(ctx, rs[i]);
+      if ((find_inst(ctx, S->inst)->ks.kq == 1 ? 0 : 1) == q) S->clusters = cs > 1;
+    }
   }
   plan->device = ctx->device;
   plan->stream = ctx->stream;
@@ -1575,7 +1589,8 @@ int nmc_replicas_create(nmc_ctx *ctx, int32_t inst, int32_t replicas, uint64_t s
     if ((e = dev_alloc(&S.ks.S, static_cast<size_t>(2 * n + 2) * W)) != cudaSuccess ||
         (e = dev_alloc(&S.ks.best, static_cast<size_t>(2 * n) * W)) != cudaSuccess ||
         (e = dev_alloc(&S.ks.energy, 32 * W)) != cudaSuccess ||
-        (e = dev_alloc(&S.ks.best_energy, 32 * W)) != cudaSuccess ||
+        (e = dev_alloc(&S.ks.best_energy, 32 * W + 1)) != cudaSuccess ||  // and the step status
+        (e = cudaMemset(S.ks.best_energy + 32 * W, 0, sizeof(int32_t))) != cudaSuccess ||
         (e = dev_alloc(&S.ks.imp, W)) != cudaSuccess ||
         (e = dev_alloc(&S.ks.bar, 1)) != cudaSuccess ||
         (e = cudaMemsetAsync(S.ks.imp, 0, sizeof(uint32_t) * W, ctx->stream)) != cudaSuccess ||
@@ -1915,6 +1930,7 @@ int nmc_replicas_run_pt(nmc_ctx *ctx, int32_t rs, int32_t t0, int32_t t1,
   const int kq = I->ks.kq;
   int cs = 1, lanes = 0;
   tuned_shape(ctx, *I, W, &cs, &lanes);
+  S->clusters = cs > 1;
   // segments end at t1 or after sweep t with (t+1) % per == 0, where an exchange round follows;
   // their work items are uploaded in chunks
   const int64_t max_chunk_items = std::max<int64_t>(W, 1 << 18);
@@ -2161,6 +2177,7 @@ int nmc_batch_autotune(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, int32_t 
   for (int32_t i = 0; i < n_sets; ++i) {
     ReplicaSet *S = find_set(ctx, rs[i]);
     Instance *I = find_inst(ctx, S->inst);
+    S->clusters = true;  // trials run every shape
     const size_t W = S->ks.W, n = I->ks.n;
     parts.push_back({S->ks.S, sizeof(uint32_t) * (2 * n + 2) * W});
     parts.push_back({S->ks.best, sizeof(uint32_t) * n * W});
@@ -2549,6 +2566,7 @@ int nmc_adaptive_ladder(nmc_ctx *ctx, int32_t inst, int32_t replicas, uint64_t s
     cnt[q] = W;
     max_n[q] = n;
     tuned_shape(ctx, *I, W, &cs[q], &lanes[q]);
+    S->clusters = cs[q] > 1;
     if ((e = fill_schedule(bq, static_cast<size_t>(n) * T, beta, ctx->flag, ctx->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(stats, 0, sizeof(long long) * 64 * W, ctx->stream)) != cudaSuccess) {
       rc = cuda_fail(ctx, e, "prepare ladder level");

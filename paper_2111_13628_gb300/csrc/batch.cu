@@ -415,27 +415,10 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// The barrier between colour classes in two halves, for one CTA as for several: a thread arrives
-// once its own words of the class are stored, and waits only before its first read of that class.
-// A release at cluster scope costs 300 - 400 cycles, whatever was stored; a CTA on its own needs its
-// stores ordered among its threads only (512 threads, one round of the barrier: 505 cycles with the
-// cluster release, 120 with the CTA fence, 85 for __syncthreads, which cannot be split).
-template <int CS>
-__device__ __forceinline__ void class_arrive() {
-  if (CS == 1) {
-    __threadfence_block();
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  } else {
-    cluster_arrive();
-  }
-}
-__device__ __forceinline__ void class_wait() { cluster_wait(); }
-
-// Stores v at the same shared-memory word of CTA `rank` of the cluster (32-bit addressing).
-__device__ __forceinline__ void st_rank(uint32_t saddr, int rank, uint32_t v) {
+__device__ __forceinline__ uint32_t shared_at(uint32_t saddr, int rank) {  // the same word of a CTA
   uint32_t ra;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(saddr), "r"(rank));
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(v) : "memory");
+  return ra;
 }
 
 template <int CS, typename T>
@@ -454,6 +437,7 @@ struct SweepShared {
   SweepRows rows;
   uint32_t improved;  // replicas that improved in the last sweep
   int next;           // index of the current item
+  unsigned long long full[2];  // CS > 1: barriers of the even and odd class steps (ClassBarrier)
 };
 
 // Energies of the word's replicas, kept by warp 0 of every CTA (its lane's replica), and the
@@ -462,6 +446,107 @@ struct EnergyTrack {
   int e, best;
   long long s1, s2;  // sums of E and E^2 of the sampled sweeps
   uint32_t m_item;
+};
+
+// The barrier between colour classes in two halves: a thread arrives once its own words of the class
+// are stored, and waits only before its first read of that class.
+//
+// One CTA: its stores need ordering among its threads only, so it fences at CTA scope and arrives
+// relaxed at the hardware barrier (512 threads, a round: 120 cycles; 505 with the cluster release,
+// 85 for __syncthreads, which cannot be split).
+//
+// Several CTAs: a release at cluster scope waits for all remote stores, 300 cycles at the least and
+// 1,000 - 1,700 in a sweep. Instead every new word is an asynchronous store that counts its bytes at
+// the receiving CTA's mbarrier (st.async), for the class step's parity. A step of a CTA completes
+// when all words of the class have arrived there, all its own warps have (none can miss a step), and
+// one warp of every CTA has (so that no CTA, also one without a variable in the class, is passed by
+// more than a step and a barrier never counts two steps at once). Words overwritten by a CTA that is
+// a step ahead are words nobody reads any more: every warp with a variable in the class has stored it,
+// hence finished reading, and warps counting ahead read neither their own class nor the one before.
+// The last class of a sweep meets at the hardware cluster barrier, which also publishes the CTAs'
+// energy changes. A wait gives up after about a second, marks the set (kStepTimeout at the end of
+// best_energy) and lets the rest of the launch run through without waiting.
+constexpr long long kStepLimitCycles = 1ll << 31;
+
+template <int CS, int WARPS>
+struct ClassBarrier {
+  uint32_t bar;                 // shared address of full[0]
+  uint32_t arrived, waited;     // steps at the mbarriers so far
+  bool dead;
+
+  // by all threads, before a barrier of the CTAs
+  __device__ __forceinline__ void init(SweepShared &sh) {
+    bar = (uint32_t)__cvta_generic_to_shared(&sh.full[0]);
+    arrived = waited = 0;
+    dead = false;
+    if (CS > 1 && threadIdx.x == 0) {
+      for (int i = 0; i < 2; ++i)
+        asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(bar + 8 * i), "r"(WARPS + CS) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+  }
+  // Stores v at word `saddr` of CTA `rank`, as part of the step being worked on.
+  __device__ __forceinline__ void store(uint32_t saddr, int rank, uint32_t v, bool last) const {
+    if (last)
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(shared_at(saddr, rank)), "r"(v) : "memory");
+    else
+      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(
+                       shared_at(saddr, rank)),
+                   "r"(v), "r"(shared_at(bar + 8 * (arrived & 1), rank))
+                   : "memory");
+  }
+  // The warp has stored its words of the class (n_words in all CTAs together).
+  __device__ __forceinline__ void arrive(int n_words, bool last) {
+    __syncwarp();
+    if (CS == 1) {
+      __threadfence_block();
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    } else if (last) {
+      cluster_arrive();
+    } else {
+      const int lane = threadIdx.x & 31;
+      const uint32_t b = bar + 8 * (arrived & 1);
+      if (threadIdx.x < CS)
+        asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                         shared_at(b, threadIdx.x))
+                     : "memory");
+      if (threadIdx.x == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(4 * n_words)
+                     : "memory");
+      else if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
+      ++arrived;
+    }
+  }
+  // Waits for the class before the one at hand (last: the sweep's last one).
+  __device__ __forceinline__ void wait(const BatchItem &B, bool last) {
+    __syncwarp();
+    if (CS == 1 || last) {
+      cluster_wait();
+      return;
+    }
+    const uint32_t b = bar + 8 * (waited & 1), parity = (waited >> 1) & 1;
+    ++waited;
+    if (dead) return;
+    uint32_t done = 0;
+    long long t0 = 0;
+    while (true) {
+      asm volatile(
+          "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+          "selp.u32 %0, 1, 0, p;\n}"
+          : "=r"(done)
+          : "r"(b), "r"(parity)
+          : "memory");
+      if (done) break;
+      if (t0 == 0) t0 = clock64();
+      if (clock64() - t0 > kStepLimitCycles) {
+        dead = true;
+        B.best_energy[32 * B.W] = kStepTimeout;
+        break;
+      }
+    }
+    dead = __any_sync(0xFFFFFFFFu, dead);
+  }
 };
 
 // Takes the next item from the counter into sh.item; false when there is none left.
@@ -574,6 +659,8 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
   const int rank = CS == 1 ? 0 : (int)cg::this_cluster().block_rank();
   for (int i = threadIdx.x; i <= tab_len; i += blockDim.x) tab_s[i] = i < tab_len ? tab[i] : 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  ClassBarrier<CS, one_thread_threads<KQ>() / 32> step;
+  step.init(sh);
   while (true) {
     if (!next_batch_item<CS>(items, n_items, next_item, rank, sh)) break;
     const BatchItem &B = sh.item;
@@ -612,6 +699,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         // CTA's share of them to its warps
         const int cnt = share_count<CS>(c0, c1, rank);
         const int ngr = (cnt + 31) >> 5;
+        const bool last_class = c + 1 == B.n_colours;
         {
           auto store = [&](int v, uint32_t xn) {
             if (CS == 1) {
@@ -619,7 +707,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
             } else {
               const uint32_t sa = (uint32_t)__cvta_generic_to_shared(xs + v);
 #pragma unroll
-              for (int r = 0; r < CS; ++r) st_rank(sa, r, xn);
+              for (int r = 0; r < CS; ++r) step.store(sa, r, xn, last_class);
             }
           };
           // first round: the slots before `pre` are counted before the wait for the previous
@@ -638,18 +726,17 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
 #pragma unroll 1
             for (int part = 0; part < 2; ++part) {
               const int pre = region_pre(P.regions);
-              if (part == 1 && first && c > 0) {
-                __syncwarp();
-                class_wait();
-              }
+              if (part == 1 && first && c > 0) step.wait(B, false);
               if (go) count_slots<KQ>(xs, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
             }
-            if (go) store(v, accept_batch<KQ, PT>(B, tab_s, tab_len, sh.mult, sh.rows, v, x,
-                                                    P.bq, C, acc));
+            uint32_t xn = x;
+            if (go) xn = accept_batch<KQ, PT>(B, tab_s, tab_len, sh.mult, sh.rows, v, x, P.bq, C, acc);
+            // every word counts at the receiving barriers, also one that did not change
+            if (CS > 1 ? li < cnt : go) store(v, xn);
             if (base + kThreads >= cnt) break;
           }
         }
-        if (c + 1 == B.n_colours) {
+        if (last_class) {
           // the sweep's energy changes, published with its last class: planes -> 16-bit values (one
           // byte transpose for each half of the planes), then a warp reduction per replica
           uint32_t lo[8], hi[8];
@@ -675,8 +762,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         }
         // this CTA's words of the class are published; the next class's loads are requested and
         // its slots before `pre` counted (none holds a literal of this class) before the wait
-        __syncwarp();
-        class_arrive<CS>();
+        step.arrive(c1 - c0, last_class);
         mygrp -= ngr;
         while (mygrp < 0) mygrp += kWarps;
         if (c + 1 < B.n_colours) {
@@ -688,7 +774,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
         c1 = c2;
         cg = cgn;
       }
-      class_wait();
+      step.wait(B, true);
       end_sweep<CS, PT>(B, rank, t, xs, sh, track);
     }
     store_item<CS, PT>(B, rank, xs, track);
@@ -787,6 +873,8 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
   for (int i = threadIdx.x; i <= tab_len; i += blockDim.x) tab_s[i] = i < tab_len ? tab[i] : 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tl = lane % TL, team = lane / TL;
+  ClassBarrier<CS, kWarps> step;
+  step.init(sh);
   while (true) {
     if (!next_batch_item<CS>(items, n_items, next_item, rank, sh)) break;
     const BatchItem &B = sh.item;
@@ -886,12 +974,11 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
 #pragma unroll
       for (int k = 0; k < RPL; ++k) acc[k] = 0;
       for (int c = 0; c < nc; ++c) {
+        const int c0 = col_ptr[c], c1 = col_ptr[c + 1];
+        const bool last_class = c + 1 == nc;
         bool waited = c == 0;  // a sweep starts with every word published
         auto wait = [&]() {
-          if (!waited) {
-            __syncwarp();
-            class_wait();
-          }
+          if (!waited) step.wait(B, false);
           waited = true;
         };
         if (P.c == c && P.t == t && !P.work) seek(c, t);
@@ -1029,17 +1116,17 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
             flip |= ((votes >> (team * TL)) & ((1u << TL) - 1u)) << (TL * k);
             acc[k] += ok ? val[k] : 0;
           }
-          if (flip) {
-            if (CS == 1) {
-              if (tl == 0) xs[v] = x ^ flip;
-            } else if (tl < CS) {
-              st_rank((uint32_t)__cvta_generic_to_shared(xs + v), tl, x ^ flip);
-              if (CS > TL) st_rank((uint32_t)__cvta_generic_to_shared(xs + v), tl + TL, x ^ flip);
-            }
+          if (CS == 1) {
+            if (flip && tl == 0) xs[v] = x ^ flip;
+          } else if (go && tl < CS) {
+            // every word counts at the receiving barriers, also one that did not change
+            const uint32_t sa = (uint32_t)__cvta_generic_to_shared(xs + v);
+            step.store(sa, tl, x ^ flip, last_class);
+            if (CS > TL) step.store(sa, tl + TL, x ^ flip, last_class);
           }
         }
         wait();
-        if (c + 1 == nc) {  // the sweep's energy changes, published with its last class
+        if (last_class) {  // the sweep's energy changes, published with its last class
 #pragma unroll
           for (int k = 0; k < RPL; ++k) {
             int s = acc[k];
@@ -1048,15 +1135,14 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
             if (team == 0 && s != 0) atomicAdd(&sh.ep[t & 1][tl + TL * k], s);
           }
         }
-        __syncwarp();
-        class_arrive<CS>();
+        step.arrive(c1 - c0, last_class);
         if (here) {
           mine -= P.units;
           while (mine < 0) mine += kWarps;
           seek(c + 1, t);
         }
       }
-      class_wait();
+      step.wait(B, true);
       end_sweep<CS, PT>(B, rank, t, xs, sh, track);
     }
     store_item<CS, PT>(B, rank, xs, track);

@@ -131,6 +131,8 @@ cudaError_t quantize_schedule(const float *beta, int32_t n_units, int32_t n_step
                               cudaStream_t st);
 
 // ---- batched k-SAT (batch.cu) -----------------------------------------------------------
+// Left in best_energy[32 W] of a set when a wait between the CTAs of its word gave up.
+constexpr int32_t kStepTimeout = 1;
 // Largest n whose word vector fits the batched kernel's shared memory on `device`.
 size_t batch_max_vars(int tab_len, int device);
 // Clusters of cs (2, 4, 8) CTAs that run at once on `device` with one CTA per SM.
