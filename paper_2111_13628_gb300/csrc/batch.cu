@@ -194,6 +194,7 @@ struct AttemptPrep {
   int len;
   int regions;  // slot regions of the variable's group (SlotRegions)
   uint32_t bq;
+  uint32_t vo;  // original id
 };
 
 // Slot regions of a group, in units of 4 slots: own-positive in every lane below ra, own-negated
@@ -209,6 +210,7 @@ template <int KQ>
 __device__ __forceinline__ void prep_attempt(const BatchItem &B, int cg, int c0, int v, int t,
                                              AttemptPrep<KQ> &p) {
   p.bq = __ldg(B.bq + (size_t)t * B.n + v);
+  p.vo = (uint32_t)__ldg(B.orig + v);
   const int off = v - c0;
   const int g = cg + (off >> 5), ln = off & 31;
   const int gb = __ldg(B.grp_base + g);
@@ -320,7 +322,7 @@ __device__ __forceinline__ void count_slots(const uint32_t *xs, AttemptPrep<KQ> 
   }
 }
 
-// Acceptance of variable v at the sweep of `rows` for the 32 replicas of the word, from the counters
+// Acceptance of the variable with original id vo at the sweep of `rows` for the 32 replicas of the word, from the counters
 // of its whole list; returns its new word. With the table index from one product, the eight-word
 // transpose and the Philox blocks from their third round on, 200 sweeps of the 50,000-variable
 // bench instance with 1,024 replicas take 41.90 ms (43.94 before), 24 uneven 3-/4-SAT sets 15.75
@@ -329,11 +331,12 @@ __device__ __forceinline__ void count_slots(const uint32_t *xs, AttemptPrep<KQ> 
 template <int KQ, bool PT>
 __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint32_t *tab_s,
                                                  int tab_len, const uint32_t *mult_s,
-                                                 const SweepRows &rows, int v, uint32_t x, uint32_t bqv, const Counts<KQ> &C,
+                                                 const SweepRows &rows, uint32_t vo, uint32_t x,
+                                                 uint32_t bqv, const Counts<KQ> &C,
                                                  uint32_t (&acc)[kAccPlanes]) {
   uint32_t s8[8];
   C.change(x, s8);
-  const PhiloxCol col = philox_col((uint32_t)__ldg(B.orig + v), kTagKsatSweep, B.k1);
+  const PhiloxCol col = philox_col(vo, kTagKsatSweep, B.k1);
   const uint32_t bqc = min(bqv, (uint32_t)tab_len << 8);
   // replicas whose dE <= 0 (sign plane set, or every plane zero) accept without a draw
   uint32_t flip = s8[7] | ~(s8[0] | s8[1] | s8[2] | s8[3] | s8[4] | s8[5] | s8[6]);
@@ -730,7 +733,8 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
               if (go) count_slots<KQ>(xs, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
             }
             uint32_t xn = x;
-            if (go) xn = accept_batch<KQ, PT>(B, tab_s, tab_len, sh.mult, sh.rows, v, x, P.bq, C, acc);
+            if (go)
+              xn = accept_batch<KQ, PT>(B, tab_s, tab_len, sh.mult, sh.rows, P.vo, x, P.bq, C, acc);
             // every word counts at the receiving barriers, also one that did not change
             if (CS > 1 ? li < cnt : go) store(v, xn);
             if (base + kThreads >= cnt) break;
