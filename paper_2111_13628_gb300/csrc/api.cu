@@ -401,6 +401,17 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
 
 namespace {
 
+// Touches every page of a result buffer that a device-to-host copy is about to fill. A copy into
+// pages that were never written (a caller's fresh array) is several times slower than one into pages
+// that exist (27 MB of LBP results: 23 ms more); done while the GPU still computes, it costs nothing.
+// The contents stay as they are.
+void prefault(void *p, size_t bytes) {
+  if (!p || bytes < (1u << 20)) return;
+  volatile char *c = static_cast<volatile char *>(p);
+  for (size_t i = 0; i < bytes; i += 4096) c[i] = c[i];
+  c[bytes - 1] = c[bytes - 1];
+}
+
 // Makes room for `total` work items in the context's device work list (waiting for earlier
 // launches that may still read it) and allocates the two work counters.
 int reserve_items(nmc_ctx *ctx, size_t total) {
@@ -1751,6 +1762,8 @@ static int read_impl(nmc_ctx *ctx, int32_t rs, const nmc_result *out, bool to_ho
     e = qap_unpack(I->qp, S->qp, static_cast<int16_t *>(st), static_cast<int16_t *>(bst), en, ben,
                    ctx->stream);
   if (e == cudaSuccess && to_host) {
+    prefault(out->states, state_bytes);  // the launches before it are still running
+    prefault(out->best_states, state_bytes);
     if (out->states && e == cudaSuccess)
       e = cudaMemcpyAsync(out->states, st, state_bytes, cudaMemcpyDeviceToHost, ctx->stream);
     if (out->best_states && e == cudaSuccess)
@@ -2353,7 +2366,12 @@ int nmc_cnf_lbp(nmc_ctx *ctx, int32_t inst, int32_t n_seeds, const uint8_t *x_st
   A.deltas = deltas;
   A.n_done = n_done;
   A.overlap = overlap;
+  std::thread touch([&] {  // beside the iterations, which keep this thread busy
+    prefault(marg_out, sizeof(double) * sn);
+    prefault(corr_out, sizeof(double) * S * static_cast<size_t>(m));
+  });
   const int err = lbp_run(A, ctx->stream);
+  touch.join();
   if (err != 0) return cuda_fail(ctx, static_cast<cudaError_t>(err), "LBP");
   NMC_CUDA(cudaMemcpyAsync(marg_out, marg, sizeof(double) * sn, cudaMemcpyDeviceToHost, ctx->stream), "read marginals");
   if (corr_out)
