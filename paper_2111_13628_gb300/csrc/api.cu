@@ -683,13 +683,9 @@ void parallel_ranges(int64_t count, F f, int64_t per_thread = 8192) {
 //
 // Occurrences that hold a literal of the previous colour class go to the last slots of every lane
 // (from slot `pre` on), so that the kernel can count all others while that class is still being
-// updated. Of the slots before `pre`, a lane's occurrences in which its own literal is positive
-// come first, those where it is negated last, so that the kernel can count each kind with one
-// bit-sliced counter outside the slots where lanes differ; which of a lane's occurrences fill up
-// the last slots is free, and is chosen to bring the lanes' sign boundaries together.
+// updated.
 struct BankOrder {
-  // per lane: own-positive / own-negative occurrences to place before `pre`, those to place after
-  std::vector<int32_t> pend[3][32];
+  std::vector<int32_t> pend[2][32];  // per lane: occurrences to place before `pre`, and after
   int32_t addr[3][32][32];           // per literal position and bank: distinct words this slot
   int32_t cnt[3][32];
 
@@ -706,9 +702,7 @@ struct BankOrder {
     addr[p][b][cnt[p][b]++] = w;
   }
   // Writes the group's len x 32 entries (int4 each: sign bytes, three word byte offsets); the
-  // previous colour class holds the new ids [prev0, prev1). Returns the slot regions (units of 4
-  // slots): own-positive in every lane below ra, own-negated in every lane from rb on, no literal
-  // of the previous class below pre, as ra | rb << 10 | pre << 20.
+  // previous colour class holds the new ids [prev0, prev1). Returns `pre`.
   int32_t build(int32_t g0, int32_t cend, int32_t len, int32_t n, int32_t prev0, int32_t prev1,
                 const HostVec &occ, const std::vector<int32_t> &occ_ptr,
                 const std::vector<int32_t> &orig, const std::vector<int32_t> &deg, int32_t *dst0) {
@@ -716,7 +710,8 @@ struct BankOrder {
     const int32_t lit0 = 2 * prev0, lit1 = 2 * prev1;  // literals of the previous class
     int32_t dep = 0;
     for (int32_t l = 0; l < 32; ++l) {
-      for (int i = 0; i < 3; ++i) pend[i][l].clear();
+      pend[0][l].clear();
+      pend[1][l].clear();
       const int32_t v = g0 + l;
       if (v >= cend) continue;
       for (int32_t j = 0; j < deg[orig[v]]; ++j) {
@@ -724,59 +719,28 @@ struct BankOrder {
         const int32_t *q = &occ[static_cast<size_t>(e) * 4];
         const bool d = (q[1] >= lit0 && q[1] < lit1) || (q[2] >= lit0 && q[2] < lit1) ||
                        (q[3] >= lit0 && q[3] < lit1);
-        pend[d ? 2 : (q[0] != 0 ? 1 : 0)][l].push_back(e);
+        pend[d ? 1 : 0][l].push_back(e);
       }
-      dep = std::max(dep, static_cast<int32_t>(pend[2][l].size()));
+      dep = std::max(dep, static_cast<int32_t>(pend[1][l].size()));
     }
     const int32_t pre = len - ((dep + 3) & ~3);
-    // a lane's sign boundary before `pre` can lie anywhere in [lo, hi]: with more occurrences than
-    // slots some move behind `pre`, with fewer there are inert entries between the two signs
-    int32_t lo[32], hi[32], top = 0, bot = pre;
-    for (int32_t l = 0; l < 32; ++l) {
-      const int32_t np = static_cast<int32_t>(pend[0][l].size()),
-                    nn = static_cast<int32_t>(pend[1][l].size());
-      lo[l] = np + nn > pre ? std::max(0, pre - nn) : np;
-      hi[l] = np + nn > pre ? std::min(np, pre) : pre - nn;
-      top = std::max(top, lo[l]);
-      bot = std::min(bot, hi[l]);
-    }
-    const int32_t aim = ((top + bot) / 2 + 2) & ~3;
-    int32_t bound[32], first_neg[32], ra = pre, rb = 0;
-    for (int32_t l = 0; l < 32; ++l) {
-      bound[l] = std::min(std::max(aim, lo[l]), hi[l]);
-      ra = std::min(ra, bound[l]);
-      rb = std::max(rb, bound[l]);
-      first_neg[l] = bound[l];
-      const int32_t np = static_cast<int32_t>(pend[0][l].size()),
-                    nn = static_cast<int32_t>(pend[1][l].size());
-      if (np + nn > pre) {  // the last of each sign move behind `pre`
-        for (int32_t k = bound[l]; k < np; ++k) pend[2][l].push_back(pend[0][l][k]);
-        for (int32_t k = pre - bound[l]; k < nn; ++k) pend[2][l].push_back(pend[1][l][k]);
-        pend[0][l].resize(bound[l]);
-        pend[1][l].resize(pre - bound[l]);
-      } else {
-        bound[l] = np;
-        first_neg[l] = pre - nn;
+    // what does not fit before `pre` goes behind it
+    for (int32_t l = 0; l < 32; ++l)
+      while (static_cast<int32_t>(pend[0][l].size()) > pre) {
+        pend[1][l].push_back(pend[0][l].back());
+        pend[0][l].pop_back();
       }
-    }
-    ra &= ~3;
-    rb = (rb + 3) & ~3;
-    // inert entries among the slots counted as negated in every lane are marked negated; a lane's
-    // number of marked entries goes into the low 7 bits of its first sign byte (the kernel's
-    // counter starts at minus that; lists it takes have at most 128 slots, and with all 128 none is
-    // counted as negated only, so that the counter stays below 128)
-    if (len >= 128) rb = len;
+    // a lane's number of own-negated occurrences goes into the low 7 bits of its first sign byte (the
+    // kernel's counter starts at minus that)
     int32_t marked[32] = {};
     for (int32_t j = 0; j < len; ++j) {
       for (int p = 0; p < 3; ++p)
         for (int b = 0; b < 32; ++b) cnt[p][b] = 0;
       for (int32_t l = 0; l < 32; ++l) {
         int32_t *dst = dst0 + (static_cast<size_t>(j) * 32 + l) * 4;
-        std::vector<int32_t> &pool = pend[j >= pre ? 2 : (j < bound[l] ? 0 : 1)][l];
-        if (pool.empty() || (j < pre && j >= bound[l] && j < first_neg[l])) {  // inert: own sign 0, one always-true literal (word n)
-          const bool neg = j >= rb && j < pre;
-          marked[l] += neg;
-          dst[0] = static_cast<int32_t>(1u << 15 | (neg ? 1u << 7 : 0u));
+        std::vector<int32_t> &pool = pend[j >= pre ? 1 : 0][l];
+        if (pool.empty()) {  // inert: own sign 0, one always-true literal (word n)
+          dst[0] = static_cast<int32_t>(1u << 15);
           dst[1] = dst[2] = dst[3] = n * 4;
           for (int p = 0; p < 3; ++p) add(p, n);
           continue;
@@ -812,7 +776,7 @@ struct BankOrder {
       }
     }
     for (int32_t l = 0; l < 32 && len > 0; ++l) dst0[4 * l] |= marked[l] & 0x7F;
-    return (ra / 4) | (rb / 4) << 10 | (pre / 4) << 20;
+    return pre;
   }
 };
 
@@ -1081,28 +1045,9 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
   for (int32_t v = 0; v < n; ++v) ++col_ptr[colour[v] + 1];
   for (int32_t c = 0; c < n_colours; ++c) col_ptr[c + 1] += col_ptr[c];
   std::vector<int32_t> orig(n), newid(n);
-  // own-positive occurrences of each variable (k <= 4 layout: a group's lanes keep those first)
-  std::vector<int32_t> npos(kq == 1 ? n : 0, 0);
-  if (kq == 1)
-    parallel_ranges(n, [&](int64_t v0, int64_t v1) {
-      for (int64_t v = v0; v < v1; ++v)
-        for (int32_t e = vptr[v]; e < vptr[v + 1]; ++e)
-          npos[v] += occ0[static_cast<size_t>(e) * slots] == 0 ? 1 : 0;
-    });
   {
     std::vector<int32_t> pos(col_ptr.begin(), col_ptr.end() - 1);
     for (int32_t r = 0; r < n; ++r) orig[pos[colour[ord[r]]]++] = ord[r];
-    if (kq == 1) {
-      // inside a class: degree down, then own-positive count down (a group's lanes then have
-      // similar splits between positive and negative occurrences), then id up
-      parallel_ranges(n_colours, [&](int64_t c0, int64_t c1) {
-        for (int64_t c = c0; c < c1; ++c)
-          std::stable_sort(orig.begin() + col_ptr[c], orig.begin() + col_ptr[c + 1],
-                           [&](int32_t a, int32_t b) {
-                             return deg[a] != deg[b] ? deg[a] > deg[b] : npos[a] > npos[b];
-                           });
-      }, 1);
-    }
     for (int32_t p = 0; p < n; ++p) newid[orig[p]] = p;
   }
   // -- occurrence lists in new ids, each padded to a multiple of 4 occurrences
@@ -1154,7 +1099,7 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
       grp_v0.push_back(g0);
     }
   }
-  // slot regions of every group, stored after the G + 1 offsets (BankOrder::build)
+  // `pre` of every group (BankOrder::build), stored after the G + 1 offsets
   const int32_t n_groups = static_cast<int32_t>(grp_v0.size());
   grp_base.resize(static_cast<size_t>(2) * n_groups + 1, 0);
   // of every group's class: its end, its first variable and the previous class's first variable
@@ -1197,7 +1142,7 @@ int prepare_ksat(int32_t n_vars, int32_t n_clauses, int32_t k_max, const int32_t
         dep = std::max(dep, static_cast<int32_t>(late[l].size()));
       }
       const int32_t pre = len - ((dep + 3) & ~3);
-      grp_base[n_groups + 1 + g] = (len / 4) << 10 | (pre / 4) << 20;  // no slot of one sign only
+      grp_base[n_groups + 1 + g] = pre | (K <= 6 ? 1 << 30 : 0);  // clauses of at most six literals
       for (int32_t l = 0; l < 32; ++l) {
         size_t at = 0, lat = 0;
         uint32_t marked = 0;  // own-negated occurrences: into free bits of the first sign word

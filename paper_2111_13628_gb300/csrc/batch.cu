@@ -167,20 +167,32 @@ struct SweepRows {
   }
 };
 
-// OR over the clause's other literals of their truth values (32 replicas), from an occurrence's
-// entry: q = {sign bits, byte offsets of literals 1..3}; for k > 4 also q2 = {byte offsets of
-// literals 4..7}, whose signs sit in bit 6 of bytes 0..3 of q.x (shifted up to bit 7 here).
-template <int KQ>
-__device__ __forceinline__ uint32_t others_or(const uint32_t *xs, const int4 &q, const int4 &q2) {
-  const uint32_t sg = (uint32_t)q.x;
-  uint32_t o = (xs_at(xs, q.y) ^ sign_mask<1>(sg)) | (xs_at(xs, q.z) ^ sign_mask<2>(sg)) |
-               (xs_at(xs, q.w) ^ sign_mask<3>(sg));
-  if (KQ == 2) {
-    const uint32_t s6 = sg << 1;
-    o |= (xs_at(xs, q2.x) ^ sign_mask<0>(s6)) | (xs_at(xs, q2.y) ^ sign_mask<1>(s6)) |
-         (xs_at(xs, q2.z) ^ sign_mask<2>(s6)) | (xs_at(xs, q2.w) ^ sign_mask<3>(s6));
+// ORs over the other literals of N slots' clauses of their truth values (32 replicas), from the slots'
+// entries: {sign bits, byte offsets of literals 1..3}; for k > 4 also {byte offsets of literals
+// 4..7}, whose signs sit in bit 6 of bytes 0..3 of the sign word (shifted up to bit 7 here). few: no
+// clause of the formula has more than six literals, so literals 6 and 7 are always false.
+template <int KQ, int N>
+__device__ __forceinline__ void others_or(const uint32_t *xs, const int4 (&q)[N * KQ], bool few,
+                                          uint32_t (&o)[N]) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const int4 &a = q[j * KQ];
+    const uint32_t sg = (uint32_t)a.x;
+    o[j] = (xs_at(xs, a.y) ^ sign_mask<1>(sg)) | (xs_at(xs, a.z) ^ sign_mask<2>(sg)) |
+           (xs_at(xs, a.w) ^ sign_mask<3>(sg));
+    if (KQ == 2) {
+      const int4 &b = q[j * KQ + KQ - 1];
+      o[j] |= (xs_at(xs, b.x) ^ sign_mask<0>(sg << 1)) | (xs_at(xs, b.y) ^ sign_mask<1>(sg << 1));
+    }
   }
-  return o;
+  if (KQ == 2 && !few) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int4 &b = q[j * KQ + KQ - 1];
+      const uint32_t s6 = (uint32_t)q[j * KQ].x << 1;
+      o[j] |= (xs_at(xs, b.z) ^ sign_mask<2>(s6)) | (xs_at(xs, b.w) ^ sign_mask<3>(s6));
+    }
+  }
 }
 
 // The loads of one attempt that do not depend on the replicas' states: the variable's Q16
@@ -192,17 +204,16 @@ struct AttemptPrep {
   int4 q[4 * KQ];
   const int4 *ent;
   int len;
-  int regions;  // slot regions of the variable's group (SlotRegions)
+  int regions;  // of the variable's group: region_pre, region_few
   uint32_t bq;
   uint32_t vo;  // original id
 };
 
-// Slot regions of a group, in units of 4 slots: own-positive in every lane below ra, own-negated
-// (or inert) in every lane from rb on (k <= 4), no literal of the previous colour class below pre
-// (ra and rb describe the slots below pre).
-__device__ __forceinline__ int region_ra(int r) { return (r & 0x3FF) * 4; }
-__device__ __forceinline__ int region_rb(int r) { return ((r >> 10) & 0x3FF) * 4; }
-__device__ __forceinline__ int region_pre(int r) { return ((r >> 20) & 0x3FF) * 4; }
+// What is kept of a group beside its list: slots from `pre` on may hold literals of the previous
+// colour class, those below do not.
+__device__ __forceinline__ int region_pre(int r) { return r & 0xFFFF; }
+// k > 4: no clause of the formula has more than six literals
+__device__ __forceinline__ bool region_few(int r) { return (r >> 30) & 1; }
 
 // v = c0 + off is a variable of colour class c (starting at new id c0; cg: the class's first
 // group of 32 variables), attempted at sweep t.
@@ -260,60 +271,43 @@ __device__ __forceinline__ void load_slots(const int4 *ent, int e, int4 (&q)[4 *
   for (int j = 0; j < 4 * KQ; ++j) q[j] = __ldg(ent + (size_t)(e * KQ + j) * 32);
 }
 
-// What 4 slots add to the counter: z where they count as positive in every lane, its complement
-// where as negated, and the one or the other by the own sign where lanes differ (k > 4: always).
-template <int KQ>
-__device__ __forceinline__ uint32_t count4(const uint32_t *xs, const int4 (&q)[4 * KQ], bool pos,
-                                           bool neg, uint32_t (&c)[8]) {
-  uint32_t z[4];
-  if constexpr (KQ == 2) {
+// What N slots add to the counter: z, complemented where the own literal is negated.
+template <int KQ, int N>
+__device__ __forceinline__ void slot_masks(const uint32_t *xs, const int4 (&q)[N * KQ], bool few,
+                                           uint32_t (&z)[N]) {
+  others_or<KQ, N>(xs, q, few, z);
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      z[j] = ~others_or<2>(xs, q[2 * j], q[2 * j + 1]) ^ sign_mask<0>((uint32_t)q[2 * j].x);
-  } else {
-    uint32_t o[4], m[4];  // z = ~(o | m)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t sg = (uint32_t)q[j].x;
-      o[j] = (xs_at(xs, q[j].y) ^ sign_mask<1>(sg)) | (xs_at(xs, q[j].z) ^ sign_mask<2>(sg));
-      m[j] = xs_at(xs, q[j].w) ^ sign_mask<3>(sg);
-    }
-    if (pos) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]);
-    } else if (neg) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) z[j] = o[j] | m[j];
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) z[j] = ~(o[j] | m[j]) ^ sign_mask<0>((uint32_t)q[j].x);
-    }
-  }
-  return csa4_low<8>(c, z[0], z[1], z[2], z[3]);
+  for (int j = 0; j < N; ++j) z[j] = ~z[j] ^ sign_mask<0>((uint32_t)q[j * KQ].x);
 }
 
 // Adds slots [e0, e1) (multiples of 4) of the variable's list to the counters; P.q holds the
 // entries of slot e0's group on entry and those of slot e1's on return (while there are any).
-// Two groups of 4 a trip: each group's weight-4 carry is kept aside and the pair's carries enter
-// the planes from weight 4 up together, and the entries of a group are requested into the other of
-// two buffers while the group before it is evaluated, so the L2 latency of the list overlaps the
-// shared-memory gathers and counting and no entry is copied. With one counter instead of two and
-// no copies an attempt of 32 variables takes 2,025 warp instructions instead of 2,370 (4-SAT, 50,000
-// variables, 1,024 replicas, 200 sweeps: 41.90 -> 40.56 ms; 24 uneven 3-/4-SAT sets: 15.75 -> 12.91).
+// Two groups of 4 a trip, without a branch between them: each group's weight-4 carry is kept aside and
+// the pair's carries enter the planes from weight 4 up together, and the entries of a group are
+// requested into the other of two buffers while the group before it is evaluated, so the L2 latency of
+// the list overlaps the shared-memory gathers and counting and no entry is copied. (Counting slots
+// whose own signs agree in all lanes without the sign mask saves one instruction in such a slot, and
+// its three-way branch per group costs more: 36.4 -> 35.9 ms without it, 4-SAT, 50,000 variables, 1,024
+// replicas, 200 sweeps; 24 uneven 3-/4-SAT sets 12.1 -> 11.8.)
 template <int KQ>
 __device__ __forceinline__ void count_slots(const uint32_t *xs, AttemptPrep<KQ> &P, int e0, int e1,
-                                            bool mixed, Counts<KQ> &C) {
+                                            Counts<KQ> &C) {
   const int len = P.len;
   const int4 *ent = P.ent;
   int4 qb[4 * KQ];
-  const int ra = mixed ? 0 : region_ra(P.regions), rb = mixed ? len : region_rb(P.regions);
+  const bool few = region_few(P.regions);
+  const auto count4 = [&](const int4 (&q)[4 * KQ]) {
+    uint32_t z[4];
+    slot_masks<KQ, 4>(xs, q, few, z);
+    return csa4_low<8>(C.c, z[0], z[1], z[2], z[3]);
+  };
 #pragma unroll 1
   for (int e = e0; e < e1; e += 8) {
     if (e + 4 < len) load_slots<KQ>(ent, e + 4, qb);
-    const uint32_t f = count4<KQ>(xs, P.q, e + 4 <= ra, e >= rb, C.c);
+    const uint32_t f = count4(P.q);
     if (e + 4 < e1) {
       if (e + 8 < len) load_slots<KQ>(ent, e + 8, P.q);
-      add_carry_pair<8>(C.c, f, count4<KQ>(xs, qb, e + 8 <= ra, e + 4 >= rb, C.c));
+      add_carry_pair<8>(C.c, f, count4(qb));
     } else {
       add_carry<8>(C.c, f);
 #pragma unroll
@@ -730,7 +724,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
             for (int part = 0; part < 2; ++part) {
               const int pre = region_pre(P.regions);
               if (part == 1 && first && c > 0) step.wait(B, false);
-              if (go) count_slots<KQ>(xs, P, part ? pre : 0, part ? P.len : pre, part == 1, C);
+              if (go) count_slots<KQ>(xs, P, part ? pre : 0, part ? P.len : pre, C);
             }
             uint32_t xn = x;
             if (go)
@@ -832,12 +826,6 @@ struct TeamPrep {
   // k <= 4: the lane's first slots before and behind `pre` (two entries per slot would not fit)
   int4 q[KQ == 1 ? 4 : 1], qp[KQ == 1 ? post_slots<TL>() : 1];
 };
-
-// What one slot adds to the counter: z, complemented where the own literal is negated.
-template <int KQ>
-__device__ __forceinline__ uint32_t slot_mask(const uint32_t *xs, const int4 &q, const int4 &q2) {
-  return ~others_or<KQ>(xs, q, q2) ^ sign_mask<0>((uint32_t)q.x);
-}
 
 // Adds the other lanes' counters of the team (A planes) in a butterfly: one plane more per stage,
 // at most 8 (two's complement).
@@ -994,9 +982,10 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
           const int len = P.len, pre = P.pre;
           if (__any_sync(0xFFFFFFFFu, P.late)) wait();
           // the lane's next four slots, which arrive behind the Philox blocks
-          int4 r[4], r2[4];
+          const bool few = region_few(P.regions);
+          int4 r[4 * KQ];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) load_slot((4 + i) * TL + tl, pre, r[i], r2[KQ == 2 ? i : 0]);
+          for (int i = 0; i < 4; ++i) load_slot((4 + i) * TL + tl, pre, r[i * KQ], r[i * KQ + KQ - 1]);
           // Philox words of the replicas tl + TL k
           uint32_t u[RPL];
           {
@@ -1026,36 +1015,32 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
 #pragma unroll
             for (int j = 0; j < 8; ++j) cnt[j] = (uint32_t)((int)(k << (31 - j)) >> 31);
             const int top = __reduce_max_sync(0xFFFFFFFFu, pre);
-            int4 q[4], q2[4];
+            int4 q[4 * KQ];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               if (KQ == 1) q[i] = P.q[i];
-              else load_slot(tl + i * TL, pre, q[i], q2[i]);
+              else load_slot(tl + i * TL, pre, q[i * KQ], q[i * KQ + KQ - 1]);
             }
 #pragma unroll 1
             for (int j = 0; j < top; j += 4 * TL) {
               uint32_t z[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) z[i] = slot_mask<KQ>(xs, q[i], q2[KQ == 2 ? i : 0]);
+              slot_masks<KQ, 4>(xs, q, few, z);
               csa4<8>(cnt, z[0], z[1], z[2], z[3]);
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                q[i] = r[i];
-                if (KQ == 2) q2[i] = r2[i];
-              }
+              for (int i = 0; i < 4 * KQ; ++i) q[i] = r[i];
               if (j + 8 * TL < top) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                  load_slot(j + (8 + i) * TL + tl, pre, r[i], r2[KQ == 2 ? i : 0]);
+                  load_slot(j + (8 + i) * TL + tl, pre, r[i * KQ], r[i * KQ + KQ - 1]);
               }
             }
             team_sum<TL, 8>(cnt);
           }
-          int4 qp[POST], qp2[POST];
+          int4 qp[POST * KQ];
 #pragma unroll
           for (int i = 0; i < POST; ++i) {
             if (KQ == 1) qp[i] = P.qp[i];
-            else load_slot(pre + tl + i * TL, len, qp[i], qp2[i]);
+            else load_slot(pre + tl + i * TL, len, qp[i * KQ], qp[i * KQ + KQ - 1]);
           }
           const uint32_t bq = P.bq;
           const bool free_ = go && bq != kFrozenQ16;  // a held variable takes no attempt
@@ -1069,8 +1054,7 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
           // the remaining slots: at most POST per lane
           {
             uint32_t z[POST], p[8];
-#pragma unroll
-            for (int i = 0; i < POST; ++i) z[i] = slot_mask<KQ>(xs, qp[i], qp2[KQ == 2 ? i : 0]);
+            slot_masks<KQ, POST>(xs, qp, few, z);
             if constexpr (POST == 2) {
               p[0] = z[0] ^ z[1];
               p[1] = z[0] & z[1];

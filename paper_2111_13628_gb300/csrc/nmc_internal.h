@@ -103,7 +103,7 @@ struct BatchItem {
   const uint32_t *mult;  // 32W Q16 temperature multipliers of the replicas, or null
   long long *stats;      // 64W: per-replica sums of E (first 32W) and E^2 (next 32W), or null
   int32_t stats_t0;      // sweeps t >= stats_t0 add their end-of-sweep energies to stats
-  int32_t n_groups;      // groups of 32 variables; grp_base[n_groups + 1 + g]: g's sign regions
+  int32_t n_groups;      // groups of 32 variables; grp_base[n_groups + 1 + g]: g's `pre`
 };
 
 // ---- k-SAT launchers (ksat.cu); all asynchronous on `st` -------------------------------
