@@ -20,6 +20,7 @@
 // busy with, half the packing and a quarter of the dp4a. Then the sums over the lanes. The Philox blocks of LPR consecutive attempts of each replica are drawn
 // in parallel, one per lane, and broadcast in turn.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "nmc_internal.h"
@@ -162,6 +163,20 @@ __device__ __forceinline__ uint32_t shared_byte(uint32_t addr) {
   return *static_cast<const uint8_t *>(__cvta_shared_to_generic(addr));
 }
 
+// Largest uphill change an attempt with draw u accepts at inverse temperature b (Q16). The table does
+// not increase, so with c entries above u the test u < tab[(b d) >> 8] is (b d) >> 8 < c, that is
+// d <= (256 c - 1) / b. Found once by the lane that draws the attempt: the attempt itself, which all
+// lanes of a replica go through one after the other, is left with one comparison. c comes from the
+// logarithm the table was built from and is then set right by the table itself.
+__device__ __forceinline__ int largest_uphill(const uint32_t *tab_s, int tab_len, uint32_t u,
+                                              uint32_t b) {
+  int c = min(max((int)(256.0f * (22.18071f - __logf((float)u))), 0), tab_len);
+  while (c < tab_len && tab_s[c] > u) ++c;
+  while (c > 0 && tab_s[c - 1] <= u) --c;
+  if (c == 0) return 0;
+  return b == 0u ? INT_MAX : (int)min(((uint32_t)c * 256u - 1u) / b, (uint32_t)INT_MAX);
+}
+
 // A CTA runs the a.rpb (at most 32) replicas of one block: lane group h = lane / LPR of warp w runs
 // replica rpb block + RPW w + h, its lane l = lane % LPR owning facilities NPL l + i.
 template <int NPL, int LPR, bool NARROW>
@@ -234,17 +249,21 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
         // lane l of each replica draws its attempt a0 + l
         const int at = a0 + hl;
         int fr = 0, fs = 0, frs = 0, frz = live ? 0 : 1;  // no replica: every attempt rejected
-        uint32_t u2 = 0u, bqs = 0u;
+        int dm = INT_MIN;  // the largest change the attempt accepts
         if (at < n && live) {
           const uint4 u =
               philox4x32_10(make_uint4((uint32_t)at, (uint32_t)t, (uint32_t)r, kTagQapStep), a.k0, a.k1);
           fr = (int)(((unsigned long long)u.x * (unsigned)n) >> 32);
           fs = (int)(((unsigned long long)u.y * (unsigned)nm1) >> 32);
           fs += fs >= fr;
-          u2 = u.z;
           const uint32_t br = __ldg(bqt + fr), bs = __ldg(bqt + fs);
           frz = (br == kFrozenQ16 || bs == kFrozenQ16) ? 1 : 0;  // a held facility: reject
-          bqs = (uint32_t)(((unsigned long long)br + bs) >> 1);
+          uint32_t bj = (uint32_t)(((unsigned long long)br + bs) >> 1);
+          if (a.mult) {  // min(2^32 - 1, (mult * bq) >> 16)
+            const unsigned long long be2 = (mr * bj) >> 16;
+            bj = be2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)be2;
+          }
+          if (!frz) dm = largest_uphill(tab_s, a.tab_len, u.z, bj);
           frs = Fs[FLayout<NPL, LPR>::at(fr, fs)];
         }
         const int cnt = (n - a0) < LPR ? (n - a0) : LPR;
@@ -252,10 +271,14 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
         // broadcast per attempt within each replica's lanes
         const int packed = fr | (fs << 8) | (frs << 16) | (frz << 24);
         const bool any_held = __any_sync(0xFFFFFFFFu, frz);
+        // the next attempt's broadcasts are under way while the current one is evaluated
+        int pnext = __shfl_sync(0xFFFFFFFFu, packed, 0, LPR), dnext = __shfl_sync(0xFFFFFFFFu, dm, 0, LPR);
         for (int j = 0; j < cnt; ++j) {
-          const int pj = __shfl_sync(0xFFFFFFFFu, packed, j, LPR);
-          const bool held = (pj >> 24) != 0;
-          if (any_held && __all_sync(0xFFFFFFFFu, held)) continue;  // every replica of the warp held
+          const int pj = pnext, dj = dnext;
+          pnext = __shfl_sync(0xFFFFFFFFu, packed, j + 1, LPR);
+          dnext = __shfl_sync(0xFFFFFFFFu, dm, j + 1, LPR);
+          // every replica of the warp held
+          if (any_held && __all_sync(0xFFFFFFFFu, (pj >> 24) != 0)) continue;
           const int rr = pj & 255, ss = (pj >> 8) & 255;
           const int pr = pw[rr], ps = pw[ss];
           const uint8_t *Dr = Ds + pr * ldd, *Dsr = Ds + ps * ldd;
@@ -320,27 +343,7 @@ __device__ __forceinline__ void qap_body(const QapArgs &a, int block) {
           }
           acc += 2 * ((pj >> 16) & 255) * (int)Dr[ps];
           const int d = 2 * acc;  // |acc| < 2^25
-          // the draw and pair temperature of the attempt: with two replicas per warp fetched
-          // always (the uphill test below may diverge between them)
-          uint32_t bj = 0u, uj = 0u;
-          if (LPR < 32) {
-            bj = __shfl_sync(0xFFFFFFFFu, bqs, j, LPR);
-            uj = __shfl_sync(0xFFFFFFFFu, u2, j, LPR);
-          }
-          bool ok = !held && d <= 0;
-          if (!held && d > 0) {
-            if (LPR == 32) {  // one replica per warp: a warp-uniform branch
-              bj = __shfl_sync(0xFFFFFFFFu, bqs, j);
-              uj = __shfl_sync(0xFFFFFFFFu, u2, j);
-            }
-            if (a.mult) {  // min(2^32 - 1, (mult * bq) >> 16)
-              const unsigned long long be2 = (mr * bj) >> 16;
-              bj = be2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)be2;
-            }
-            const unsigned long long idx = ((unsigned long long)bj * (uint32_t)d) >> 8;
-            ok = idx < (unsigned long long)a.tab_len && uj < tab_s[idx];
-          }
-          if (ok) {
+          if (d <= dj) {
             if (hl == rr / NPL) put<NPL>(p, rr % NPL, off + ps);
             if (hl == ss / NPL) put<NPL>(p, ss % NPL, off + pr);
             if (hl == 0) {

@@ -27,3 +27,28 @@ def test_narrow_and_wide_entries(n, f_max, d_max):
     for a, b in (("states", "perms"), ("energies", "energies"),
                  ("best_energies", "best_energies"), ("best_states", "best_perms")):
         assert np.array_equal(got[a], want[b]), a
+
+
+@pytest.mark.parametrize("n", [2, 5, 33, 64, 130, 256])
+@pytest.mark.parametrize("temps", ["zero", "largest", "mixed"])
+def test_largest_uphill_change(n, temps):
+    """Acceptance by the largest change a draw allows: inverse temperatures 0 (every change), the
+    largest (none uphill), and per facility from 0 over the steps of the table to held."""
+    import paper_2111_13628_gb300 as nmc
+    F, D = W.random_qap(n, 81 + n)
+    T, R = 5, 70
+    if temps == "mixed":
+        u = W.Stream(82).unit(n * T).reshape(n, T)
+        beta = (10.0 ** (-6.0 + 8.0 * u)).astype(np.float32)
+        beta[::5] = 0.0
+        beta[3::7, ::2] = np.inf
+    else:
+        beta = W.beta_constant(n, T, 0.0 if temps == "zero" else 65535.0)
+    want = O.qap_anneal(F, D, beta, 0, T, seed=83, replicas=R)
+    with nmc.Context(0) as ctx:
+        inst = ctx.load_qap(F, D)
+        ctx.set_schedule(inst, beta)
+        got = ctx.anneal(inst, R, 0, T, seed=83)
+    for a, b in (("states", "perms"), ("energies", "energies"),
+                 ("best_energies", "best_energies"), ("best_states", "best_perms")):
+        assert np.array_equal(got[a], want[b]), a
