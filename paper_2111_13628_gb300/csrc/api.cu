@@ -72,6 +72,9 @@ int32_t build_table(uint32_t *out, int32_t cap) {
 
 }  // namespace
 
+// Most launches of one batch: occurrence widths x CTAs a word x lanes a variable.
+constexpr int kBatchGroups = 2 * 4 * 3;
+
 struct nmc_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -85,7 +88,7 @@ struct nmc_ctx {
   int32_t *flag = nullptr;  // device scratch flag for schedule validation
   BatchItem *items = nullptr;  // batched-kernel work list (grown on demand)
   size_t items_cap = 0;
-  int32_t *next_item = nullptr;  // two work counters (one per occurrence width)
+  int32_t *next_item = nullptr;  // work counters, one per launch of a batch
   QapArgs *qitems = nullptr;     // batched QAP work list (grown on demand)
   size_t qitems_cap = 0;
   // auxiliary streams of the batched QAP launches (one per launch shape, created on first use):
@@ -93,11 +96,11 @@ struct nmc_ctx {
   cudaStream_t qaux[kQapShapes] = {};
   cudaEvent_t qfork = nullptr;
   cudaEvent_t qjoin[kQapShapes] = {};
-  // auxiliary stream of the batched k-SAT launch of the second occurrence width (created on first
-  // use): forked after the work-list upload and joined back, so that the two widths' persistent
-  // launches share the SMs (the second fills those the first's tail leaves idle)
-  cudaStream_t kaux = nullptr;
-  cudaEvent_t kfork = nullptr, kjoin = nullptr;
+  // auxiliary streams of the batched k-SAT launches but the first (created on first use): forked
+  // after the work-list upload and joined back, so that the launches of a batch share the SMs (a
+  // later one fills those an earlier one's tail leaves idle)
+  cudaStream_t kaux[kBatchGroups - 1] = {};
+  cudaEvent_t kfork[kBatchGroups - 1] = {}, kjoin[kBatchGroups - 1] = {};
   // LBP: pinned read-back of the running seeds and its events (created on first use)
   int32_t *lbp_seen = nullptr;
   cudaEvent_t lbp_ev[2] = {};
@@ -307,8 +310,71 @@ int choose_ctas(int device, long long cnt, int per_class) {
   return 1;
 }
 
+// Estimated microseconds of one sweep of one word on cs CTAs, for choosing between shapes: a floor
+// per colour class and the CTA's variables of it, for the lanes choose_lanes gives; occurrence words
+// per variable set both. Within a tenth or two of 3-, 4- and 6-SAT sweeps of 500 to 20,001 variables
+// on 1 to 8 CTAs (20,001 variables: 3-SAT 172, 101, 63, 41 us, 4-SAT 250, 149, 103, 90, 6-SAT 683,
+// 429, 345, 274).
+double shape_sweep_us(const Instance &I, int cs) {
+  const double words = static_cast<double>(I.ks.kq) * I.ks.m * I.ks.kmax / std::max(1, I.ks.n);
+  const double v = static_cast<double>(class_size(I)) / cs;
+  const double per = choose_lanes(cs, class_size(I)) > 1
+                         ? 1.2 + (0.012 + 0.00037 * words) * v
+                         : 1.6 + 0.016 * words + (0.0063 + 0.00012 * words) * std::max(0.0, v - 64.0);
+  return I.ks.n_colours * (per + (cs > 1 ? 0.3 : 0.0));
+}
+
+// Words of one replica set that a batch runs, with the CTAs each gets.
+struct SetShape {
+  const Instance *I;
+  int words, sweeps;
+  int cs;
+};
+
+// Shapes of the words of a batch that is waited for by itself. One shape for all leaves SMs idle while
+// the longest word runs: with one CTA each, 96 words of 1,128 to 19,706 variables take as long as the
+// 17,502-variable 4-SAT words, 25 ms for 100 sweeps, while on 56 SMs there is none at all. Here a word
+// gets the fewest CTAs (by the rule of choose_ctas 1, 2, 4 or 8) that bring it under a common time,
+// the shortest for which everything fits side by side: 14 ms. A cluster of 8 takes the place of two
+// of 4, one of 4 that of two of 2; words of one CTA and less than half of the time share CTAs, with a
+// fifth to spare. False if no time does, with one CTA each (then lengths even out over the queue).
+//
+// More CTAs a word cost more SM time in all (17,502 variables: 2.25 ms on one CTA, 2 x 1.35 on two),
+// so where other work fills the SMs that one shape leaves idle, one shape is the better: the same 96
+// words 11.8 ms against 12.4 with several contexts' batches in flight.
+bool mixed_shapes(int device, std::vector<SetShape> &sets) {
+  const int fit2 = batch_clusters(2, device), fit4 = batch_clusters(4, device), fit8 = batch_clusters(8, device);
+  const auto shape = [&](double t, bool assign) {
+    long long c[9] = {0}, own = 0;
+    double shared = 0.0;
+    for (SetShape &s : sets) {
+      const int size = class_size(*s.I);
+      int cs = 1;
+      while (s.sweeps * shape_sweep_us(*s.I, cs) > t) {
+        cs *= 2;
+        if (cs > 8 || size < 24 || size < 4 * cs) return false;
+      }
+      c[cs] += s.words;
+      if (cs == 1) {
+        const double part = s.sweeps * shape_sweep_us(*s.I, 1) / t;
+        own += part > 0.5 ? s.words : 0;
+        shared += 1.2 * s.words * part;
+      }
+      if (assign) s.cs = cs;
+    }
+    c[1] = std::max(own, static_cast<long long>(std::ceil(shared)));
+    return c[8] <= fit8 && 2 * c[8] + c[4] <= fit4 && 4 * c[8] + 2 * c[4] + c[2] <= fit2 &&
+           8 * c[8] + 4 * c[4] + 2 * c[2] + c[1] <= 2ll * fit2;
+  };
+  double lo = 0.0, hi = 0.0;
+  for (const SetShape &s : sets) hi = std::max(hi, s.sweeps * shape_sweep_us(*s.I, 1));
+  if (!shape(hi, false)) return false;
+  for (int i = 0; i < 12; ++i) (shape(0.5 * (lo + hi), false) ? hi : lo) = 0.5 * (lo + hi);
+  return shape(hi, true);
+}
+
 int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t0,
-               const int32_t *t1, BatchPlan *plan) {
+               const int32_t *t1, BatchPlan *plan, bool mixed) {
   if (!ctx || !plan) return NMC_EINVAL;
   if (n_sets < 0 || (n_sets > 0 && (!rs || !t0 || !t1)))
     return fail(ctx, NMC_EINVAL, "bad batch arrays");
@@ -318,6 +384,9 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
   std::map<int32_t, int> seen;
   plan->max_n[0] = plan->max_n[1] = 0;
   int per_class[2] = {0, 0};  // largest mean colour-class size among the items
+  std::vector<SetShape> shapes;
+  std::vector<ReplicaSet *> shaped;
+  std::vector<int> owner[2];  // an item's index in shapes
   for (int32_t i = 0; i < n_sets; ++i) {
     ReplicaSet *S = find_set(ctx, rs[i]);
     if (!S) return fail(ctx, NMC_EINVAL, "unknown replica set in batch");
@@ -332,6 +401,9 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
       return fail(ctx, NMC_EINVAL, "instance too large for the batched kernel");
     if (t1[i] == t0[i]) continue;
     const int q = I->ks.kq == 1 ? 0 : 1;
+    shapes.push_back({I, S->ks.W, t1[i] - t0[i], 1});
+    shaped.push_back(S);
+    owner[q].insert(owner[q].end(), S->ks.W, static_cast<int>(shapes.size()) - 1);
     for (int32_t w = 0; w < S->ks.W; ++w) {
       BatchItem B{};
       B.occ_t = I->ks.occ_t;
@@ -363,13 +435,34 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
     per_class[q] = std::max(per_class[q], class_size(*I));
   }
   plan->items.clear();
+  plan->groups.clear();
+  mixed = mixed && shapes.size() > 1 && !getenv("NMC_BATCH_CTAS");
+  for (int q = 0; q < 2; ++q)
+    mixed = mixed && !ctx->tune.count(std::make_tuple(q + 1, plan->max_n[q], static_cast<int>(by_kq[q].size())));
+  mixed = mixed && mixed_shapes(ctx->device, shapes);
   for (int q = 0; q < 2; ++q) {
     std::vector<size_t> idx(by_kq[q].size());
     for (size_t k = 0; k < idx.size(); ++k) idx[k] = k;
-    std::stable_sort(idx.begin(), idx.end(), [&](size_t a, size_t b) { return cost[q][a] > cost[q][b]; });
+    const auto group = [&](size_t k) {  // largest clusters first
+      const SetShape &s = shapes[owner[q][k]];
+      return std::make_pair(-s.cs, choose_lanes(s.cs, class_size(*s.I)));
+    };
+    std::stable_sort(idx.begin(), idx.end(), [&](size_t a, size_t b) {
+      if (mixed && group(a) != group(b)) return group(a) < group(b);
+      return cost[q][a] > cost[q][b];
+    });
     plan->off[q] = plan->items.size();
     plan->cnt[q] = static_cast<int>(idx.size());
-    for (size_t k : idx) plan->items.push_back(by_kq[q][k]);
+    for (size_t k : idx) {
+      if (mixed) {
+        const int cs = -group(k).first, lanes = group(k).second;
+        if (plan->groups.empty() || plan->groups.back().kq != q + 1 || plan->groups.back().cs != cs ||
+            plan->groups.back().lanes != lanes)
+          plan->groups.push_back({q + 1, cs, lanes, plan->items.size(), 0});
+        ++plan->groups.back().cnt;
+      }
+      plan->items.push_back(by_kq[q][k]);
+    }
     // CTAs per item: spread few items over the SMs (word vectors replicated per cluster)
     int cs = 1, lanes = 0;
     const auto tuned = ctx->tune.find(std::make_tuple(q + 1, plan->max_n[q], plan->cnt[q]));
@@ -385,11 +478,15 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
     if (cs != 1 && cs != 2 && cs != 4 && cs != 8) cs = 1;
     plan->cs[q] = cs;
     plan->lanes[q] = lanes;
-    for (int32_t i = 0; i < n_sets; ++i) {
-      ReplicaSet *S = find_set(ctx, rs[i]);
-      if ((find_inst(ctx, S->inst)->ks.kq == 1 ? 0 : 1) == q) S->clusters = cs > 1;
-    }
+    if (!mixed && plan->cnt[q]) plan->groups.push_back({q + 1, cs, lanes, plan->off[q], plan->cnt[q]});
+    for (size_t i = 0; i < shapes.size(); ++i)
+      if ((shapes[i].I->ks.kq == 1 ? 0 : 1) == q) shaped[i]->clusters = (mixed ? shapes[i].cs : cs) > 1;
   }
+  // launch order: the largest clusters while the GPU is empty; without them the two-entry items
+  // (k > 4) first
+  std::stable_sort(plan->groups.begin(), plan->groups.end(), [&](const BatchGroup &a, const BatchGroup &b) {
+    return mixed && a.cs != b.cs ? a.cs > b.cs : a.kq > b.kq;
+  });
   plan->device = ctx->device;
   plan->stream = ctx->stream;
   plan->tab = ctx->tab;
@@ -422,15 +519,18 @@ int reserve_items(nmc_ctx *ctx, size_t total) {
     NMC_CUDA(dev_alloc(&ctx->items, total), "allocate batch work list");
     ctx->items_cap = total;
   }
-  if (!ctx->next_item) NMC_CUDA(dev_alloc(&ctx->next_item, 2), "allocate batch counters");
+  if (!ctx->next_item) NMC_CUDA(dev_alloc(&ctx->next_item, kBatchGroups), "allocate batch counters");
   return NMC_OK;
 }
 
-// Uploads a work list and launches it: items [off[q], off[q] + cnt[q]) have occurrence width
-// q + 1. pt selects the kernels with temperature multipliers and energy statistics.
-int launch_items(nmc_ctx *ctx, const std::vector<BatchItem> &items, const size_t off[2],
-                 const int cnt[2], const int max_n[2], const int cs[2], bool pt,
-                 const int lanes[2]) {
+// Uploads a work list and launches its groups side by side, the first on the context's stream, the
+// others on auxiliary streams that it then waits for. pt selects the kernels with temperature
+// multipliers and energy statistics. Each group's stream is let go by the one before it, right before
+// that one's kernel, and the counters are cleared for all beforehand: the launches reach the GPU in
+// the order of the list, a microsecond or two apart. Let go together, single CTAs were placed first,
+// one to a pair of SMs, and clusters that the plan had room for would wait for them.
+int launch_items(nmc_ctx *ctx, const std::vector<BatchItem> &items, const std::vector<BatchGroup> &groups,
+                 const int max_n[2], bool pt) {
   if (items.empty()) return NMC_OK;
   const int rc = reserve_items(ctx, items.size());
   if (rc != NMC_OK) return rc;
@@ -438,35 +538,39 @@ int launch_items(nmc_ctx *ctx, const std::vector<BatchItem> &items, const size_t
   NMC_CUDA(cudaMemcpyAsync(ctx->items, items.data(), sizeof(BatchItem) * items.size(),
                            cudaMemcpyHostToDevice, ctx->stream),
            "upload batch work list");
-  if (!cnt[0] || !cnt[1]) {
-    const int q = cnt[0] ? 0 : 1;
-    NMC_CUDA(ksat_batch(ctx->items + off[q], cnt[q], q + 1, cs[q], max_n[q], ctx->next_item + q,
-                        ctx->tab, ctx->tab_len, ctx->device, ctx->stream, pt, lanes[q]),
-             "launch batched sweep");
-    return NMC_OK;
+  const int n_groups = static_cast<int>(groups.size());
+  for (int i = 0; i < n_groups - 1; ++i) {
+    if (!ctx->kaux[i])
+      NMC_CUDA(cudaStreamCreateWithFlags(&ctx->kaux[i], cudaStreamNonBlocking), "create batch stream");
+    for (cudaEvent_t *ev : {&ctx->kfork[i], &ctx->kjoin[i]})
+      if (!*ev) NMC_CUDA(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "create batch event");
   }
-  // both widths: the two-entry items (k > 4) on the auxiliary stream, launched first, the
-  // one-entry items on the context's stream, which then waits for the auxiliary one
-  if (!ctx->kaux) {
-    NMC_CUDA(cudaStreamCreateWithFlags(&ctx->kaux, cudaStreamNonBlocking), "create batch stream");
-    NMC_CUDA(cudaEventCreateWithFlags(&ctx->kfork, cudaEventDisableTiming), "create batch event");
-    NMC_CUDA(cudaEventCreateWithFlags(&ctx->kjoin, cudaEventDisableTiming), "create batch event");
+  NMC_CUDA(cudaMemsetAsync(ctx->next_item, 0, sizeof(int32_t) * n_groups, ctx->stream), "clear work counters");
+  cudaError_t err = cudaSuccess;
+  int forked = 0;
+  for (int i = 0; i < n_groups && err == cudaSuccess; ++i) {
+    const BatchGroup &g = groups[i];
+    cudaStream_t st = i ? ctx->kaux[i - 1] : ctx->stream;
+    if (i) {
+      if ((err = cudaStreamWaitEvent(st, ctx->kfork[i - 1], 0)) != cudaSuccess) break;
+      forked = i;
+    }
+    if (i < n_groups - 1 && (err = cudaEventRecord(ctx->kfork[i], st)) != cudaSuccess) break;
+    err = ksat_batch(ctx->items + g.off, g.cnt, g.kq, g.cs, max_n[g.kq - 1], ctx->next_item + i, ctx->tab,
+                     ctx->tab_len, ctx->device, st, pt, g.lanes, true);
   }
-  NMC_CUDA(cudaEventRecord(ctx->kfork, ctx->stream), "fork batch stream");
-  NMC_CUDA(cudaStreamWaitEvent(ctx->kaux, ctx->kfork, 0), "fork batch stream");
-  const cudaError_t e1 = ksat_batch(ctx->items + off[1], cnt[1], 2, cs[1], max_n[1],
-                                    ctx->next_item + 1, ctx->tab, ctx->tab_len, ctx->device,
-                                    ctx->kaux, pt, lanes[1]);
-  // joined whether or not the launch succeeded, so that nothing is left unjoined
-  const cudaError_t ej = cudaEventRecord(ctx->kjoin, ctx->kaux);
-  const cudaError_t e0 = ksat_batch(ctx->items + off[0], cnt[0], 1, cs[0], max_n[0],
-                                    ctx->next_item, ctx->tab, ctx->tab_len, ctx->device,
-                                    ctx->stream, pt, lanes[0]);
-  cudaError_t ew = ej == cudaSuccess ? cudaStreamWaitEvent(ctx->stream, ctx->kjoin, 0) : ej;
-  if (ew != cudaSuccess) cudaStreamSynchronize(ctx->kaux);  // no join: wait on the host instead
-  if (e1 != cudaSuccess) return cuda_fail(ctx, e1, "launch batched sweep");
-  if (e0 != cudaSuccess) return cuda_fail(ctx, e0, "launch batched sweep");
-  if (ew != cudaSuccess) return cuda_fail(ctx, ew, "join batch stream");
+  // joined whether or not the launches succeeded, so that nothing is left unjoined
+  cudaError_t join = cudaSuccess;
+  for (int i = 0; i < forked; ++i) {
+    cudaError_t e = cudaEventRecord(ctx->kjoin[i], ctx->kaux[i]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->kjoin[i], 0);
+    if (e != cudaSuccess) {
+      cudaStreamSynchronize(ctx->kaux[i]);  // no join: wait on the host instead
+      join = e;
+    }
+  }
+  if (err != cudaSuccess) return cuda_fail(ctx, err, "launch batched sweep");
+  if (join != cudaSuccess) return cuda_fail(ctx, join, "join batch stream");
   return NMC_OK;
 }
 
@@ -570,12 +674,14 @@ void nmc_destroy(nmc_ctx *ctx) {
   if (!ctx) return;
   DeviceGuard g(ctx->device);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  if (ctx->kaux) {
-    cudaStreamSynchronize(ctx->kaux);
-    cudaStreamDestroy(ctx->kaux);
+  for (int i = 0; i < kBatchGroups - 1; ++i) {
+    if (ctx->kaux[i]) {
+      cudaStreamSynchronize(ctx->kaux[i]);
+      cudaStreamDestroy(ctx->kaux[i]);
+    }
+    if (ctx->kfork[i]) cudaEventDestroy(ctx->kfork[i]);
+    if (ctx->kjoin[i]) cudaEventDestroy(ctx->kjoin[i]);
   }
-  if (ctx->kfork) cudaEventDestroy(ctx->kfork);
-  if (ctx->kjoin) cudaEventDestroy(ctx->kjoin);
   if (ctx->lbp_seen) cudaFreeHost(ctx->lbp_seen);
   for (cudaEvent_t ev : ctx->lbp_ev)
     if (ev) cudaEventDestroy(ev);
@@ -1752,12 +1858,7 @@ int32_t nmc_batch_max_vars(nmc_ctx *ctx) {
 
 int nmc_batch_run(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t0,
                   const int32_t *t1) {
-  if (!ctx) return NMC_EINVAL;
-  DeviceGuard g(ctx->device);
-  BatchPlan plan;
-  const int rc = batch_plan(ctx, n_sets, rs, t0, t1, &plan);
-  if (rc != NMC_OK) return rc;
-  return launch_items(ctx, plan.items, plan.off, plan.cnt, plan.max_n, plan.cs, false, plan.lanes);
+  return nmc::batch_run(ctx, n_sets, rs, t0, t1, false);
 }
 
 int nmc_replicas_set_ladder(nmc_ctx *ctx, int32_t rs, int32_t n_temps, const float *ladder,
@@ -2116,6 +2217,20 @@ int qap_ladder(nmc_ctx *ctx, const Instance &I, ReplicaSet &S, double beta0, dou
 }
 
 }  // namespace
+
+namespace nmc {
+
+int batch_run(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t0, const int32_t *t1,
+              bool mixed) {
+  if (!ctx) return NMC_EINVAL;
+  DeviceGuard g(ctx->device);
+  BatchPlan plan;
+  const int rc = batch_plan(ctx, n_sets, rs, t0, t1, &plan, mixed);
+  if (rc != NMC_OK) return rc;
+  return launch_items(ctx, plan.items, plan.groups, plan.max_n, false);
+}
+
+}  // namespace nmc
 
 extern "C" {
 
@@ -2524,18 +2639,16 @@ int nmc_adaptive_ladder(nmc_ctx *ctx, int32_t inst, int32_t replicas, uint64_t s
       items.push_back(B);
     }
     const int q = I->ks.kq == 1 ? 0 : 1;
-    size_t off[2] = {0, 0};
-    int cnt[2] = {0, 0}, max_n[2] = {0, 0}, cs[2] = {1, 1}, lanes[2] = {0, 0};
-    cnt[q] = W;
+    int max_n[2] = {0, 0}, cs = 1, lanes = 0;
     max_n[q] = n;
-    tuned_shape(ctx, *I, W, &cs[q], &lanes[q]);
-    S->clusters = cs[q] > 1;
+    tuned_shape(ctx, *I, W, &cs, &lanes);
+    S->clusters = cs > 1;
     if ((e = fill_schedule(bq, static_cast<size_t>(n) * T, beta, ctx->flag, ctx->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(stats, 0, sizeof(long long) * 64 * W, ctx->stream)) != cudaSuccess) {
       rc = cuda_fail(ctx, e, "prepare ladder level");
       break;
     }
-    rc = launch_items(ctx, items, off, cnt, max_n, cs, true, lanes);
+    rc = launch_items(ctx, items, {{q + 1, cs, lanes, 0, W}}, max_n, true);
     if (rc != NMC_OK) break;
     double out[2] = {0.0, 0.0};
     if ((e = ladder_step(stats, S->R, W, static_cast<long long>(S->R) * sweeps_meas, beta, alpha,

@@ -1212,8 +1212,6 @@ cudaError_t launch_batch(const BatchItem *items, int n_items, int *next_item,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(clusters * CS);
-  cudaError_t err = cudaMemsetAsync(next_item, 0, sizeof(int), st);
-  if (err != cudaSuccess) return err;
   return cudaLaunchKernelEx(&cfg, kern, items, n_items, next_item, tab, tab_len, xs_words,
                             meta_words);
 }
@@ -1394,8 +1392,12 @@ size_t batch_max_vars(int tab_len, int device) {
 
 cudaError_t ksat_batch(const BatchItem *items_dev, int n_items, int kq, int cs, int max_n,
                        int *next_item, const uint32_t *tab, int tab_len, int device,
-                       cudaStream_t st, bool pt, int lanes) {
+                       cudaStream_t st, bool pt, int lanes, bool cleared) {
   if (n_items <= 0) return cudaSuccess;
+  if (!cleared) {
+    const cudaError_t err = cudaMemsetAsync(next_item, 0, sizeof(int), st);
+    if (err != cudaSuccess) return err;
+  }
   if (kq == 1) return dispatch_batch<1>(cs, items_dev, n_items, next_item, tab, tab_len, max_n, device, st, pt, lanes);
   return dispatch_batch<2>(cs, items_dev, n_items, next_item, tab, tab_len, max_n, device, st, pt, lanes);
 }

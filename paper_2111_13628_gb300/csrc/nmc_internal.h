@@ -142,7 +142,7 @@ int choose_lanes(int cs, int per_class);
 // Runs n_items items (all of one occurrence width kq) in one launch with cs CTAs (1, 2, 4, 8)
 // per item; next_item is a device int. With pt, every item carries temperature multipliers
 // (mult) and may carry energy statistics. lanes: lanes per variable (1, 4, 8; 0 = the built-in
-// choice from cs and max_n).
+// choice from cs and max_n). cleared: the caller has set next_item to zero.
 // Estimated GPU time, in microseconds, of one sweep of one 32-replica word of a k-SAT instance
 // with n variables in n_colours classes on one CTA (the shape of a launch with many items): per
 // class a latency floor plus the variables' share of a 512-thread round, rounds beyond 512
@@ -154,13 +154,20 @@ double qap_step_us(int32_t n);
 
 cudaError_t ksat_batch(const BatchItem *items_dev, int n_items, int kq, int cs, int max_n,
                        int *next_item, const uint32_t *tab, int tab_len, int device,
-                       cudaStream_t st, bool pt = false, int lanes = 0);
+                       cudaStream_t st, bool pt = false, int lanes = 0, bool cleared = false);
 
 // A validated batched launch, ready to be placed into device memory: the work items in launch
 // order (occurrence width 1 first, then 2), with their counts, shapes and the context's
 // stream, table and device. Filled by batch_plan (api.cu).
+// One launch of a batch: items [off, off + cnt) with cs CTAs a word and `lanes` lanes a variable.
+struct BatchGroup {
+  int kq, cs, lanes;
+  size_t off;
+  int cnt;
+};
 struct BatchPlan {
   std::vector<BatchItem> items;
+  std::vector<BatchGroup> groups;  // one per occurrence width, or the mixed shapes
   size_t off[2];
   int cnt[2];
   int max_n[2];
@@ -173,8 +180,12 @@ struct BatchPlan {
 };
 // Validates a batch as nmc_batch_run does and fills `plan`; returns NMC_OK or an error code
 // (recorded on the context).
+// With `mixed` (launches that run side by side) the words of a batch may get different shapes.
 int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t0,
-               const int32_t *t1, BatchPlan *plan);
+               const int32_t *t1, BatchPlan *plan, bool mixed = false);
+// nmc_batch_run; with `mixed` for a caller that waits for the batch before it starts other work.
+int batch_run(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t0, const int32_t *t1,
+              bool mixed);
 // Records an error message on the context; returns `code`.
 int set_ctx_error(nmc_ctx *ctx, int code, const char *msg);
 
