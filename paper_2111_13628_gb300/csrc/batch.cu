@@ -31,9 +31,8 @@ namespace {
 
 // One-thread kernel for k <= 4: 16 warps, up to 128 registers (no spills; a DSatur colour class
 // of the 50,000-variable bench instance puts at most ~490 variables on each CTA of a 4-CTA
-// cluster, one round of 512 threads: measured 296 us per sweep against 295 with 640 threads and
-// 96 registers, and 293 with the next class's loads requested at the barrier, which 640 threads
-// cannot hold without spilling). For k <= 8 (two int4 list entries per occurrence, twice the
+// cluster, one round of 512 threads; 640 threads with 96 registers spill 200 bytes: 44.5 ms per 200
+// sweeps against 36.4). For k <= 8 (two int4 list entries per occurrence, twice the
 // prefetched registers) 12 warps with up to 168 registers, so that nothing spills.
 template <int KQ>
 __host__ __device__ constexpr int one_thread_threads() {
@@ -316,11 +315,11 @@ __device__ __forceinline__ void count_slots(const uint32_t *xs, AttemptPrep<KQ> 
   }
 }
 
-// Acceptance of the variable with original id vo at the sweep of `rows` for the 32 replicas of the word, from the counters
-// of its whole list; returns its new word. With the table index from one product, the eight-word
-// transpose and the Philox blocks from their third round on, 200 sweeps of the 50,000-variable
-// bench instance with 1,024 replicas take 41.90 ms (43.94 before), 24 uneven 3-/4-SAT sets 15.75
-// ms per 100 sweeps (16.96). With PT, replica j of the word moves at min(2^32-1,
+// Acceptance of the variable with original id vo at the sweep of `rows` for the 32 replicas of the
+// word, from the counters of its whole list; returns its new word. The table index from one product,
+// the eight-word transpose and the Philox blocks from their third round on took 200 sweeps of the
+// 50,000-variable bench instance with 1,024 replicas from 43.94 to 41.90 ms, 24 uneven 3-/4-SAT sets
+// from 16.96 to 15.75 per 100 (37.9 and 12.0 with all later steps). With PT, replica j of the word moves at min(2^32-1,
 // (mult_s[j] * bq) >> 16) instead of bq.
 template <int KQ, bool PT>
 __device__ __forceinline__ uint32_t accept_batch(const BatchItem &B, const uint32_t *tab_s,
