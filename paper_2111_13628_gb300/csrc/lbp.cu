@@ -13,13 +13,18 @@
 // negated). h_{i->a} = sigma_ai (lambda eps_i s*_i + sum_{b != a} sigma_bi u_{b->i});
 // u_{a->i} = -1/2 ln[1 - (1 - e^{-2 beta}) prod_{j != i} (1 - tanh h_{j->a}) / 2].
 //
-// Two forms of the same iteration. The product form keeps w = e^{-2u} and E = e^{2h} instead of u
-// and h: sums of u become products of w, (1 - tanh h) / 2 is 1 / (1 + E), and an iteration needs
-// neither exponentials nor logarithms (9 double-precision instructions per message instead of 82;
-// the log form was bound by them, 85% of the pipe). It is used whenever no e^{2 field} can leave
-// the range of a double and the tolerance is above the resolution of w; the log form runs otherwise.
-// 4-SAT, 5,000 variables, 64 seeds: clause pass 1,924 -> 140 us, a call with its backbones 120 -> 34
-// ms; 500 variables, 5 seeds: 5.9 -> 2.8 ms.
+// Two forms of the same iteration. The product form keeps m = 1 - e^{-2u} and E = e^{2h} instead of
+// u and h: sums of u become products of 1 - m, (1 - tanh h) / 2 is 1 / (1 + E), and an iteration
+// needs neither exponentials nor logarithms (13 double-precision instructions per message instead of
+// 82; the log form was bound by them, 85% of the pipe). It is used whenever no e^{2 field} can leave
+// the range of a double and the tolerance is above the resolution of m; the log form runs otherwise.
+//
+// Its error stays that of the log form: a small u has a small m, E near 1 is kept as E - 1, and the
+// products are carried with the sum of their rounding errors (ProductSum, clause_messages). Largest
+// error of a converged call against 80 bits, product form over log form, mean of 84 4-SAT inputs of 300
+// to 5,000 variables at beta = 1: 0.90 marginals, 0.99 correlations (root mean square 0.84, 0.86); 36
+// sparser inputs at beta = 4: 0.85, 0.97; without a bias at beta = 1e-3: 0.46, 0.92. With 1 - m, E and
+// plain products kept instead: 1.08, 1.11 at beta = 1 and 440 without a bias at beta = 1e-3.
 #include <math.h>
 
 #include "nmc_internal.h"
@@ -122,59 +127,99 @@ __global__ void lbp_var_kernel(const int32_t *__restrict__ vptr, const int32_t *
 
 // ---- product form -----------------------------------------------------------------------------
 
+// E of an edge as one double v: E - 1 where the variable's e^{+-2 field} is at least a half, so that
+// fields near zero keep their relative precision, else -2^1000 E, at most -2^19 as long as |field| <
+// 340. E - 1 is above -1, so the two do not meet.
+constexpr double kEdgeScale = 0x1p1000;
+__device__ __forceinline__ bool edge_scaled(double v) {  // v <= -1
+  return (unsigned)__double2hiint(v) >= 0xBFF00000u;
+}
+__device__ __forceinline__ double edge_plus_one(double v) {  // 1 + E
+  const bool sc = edge_scaled(v);
+  return fma(v, sc ? -1.0 / kEdgeScale : 1.0, sc ? 1.0 : 2.0);
+}
+
 // Largest 1 + E a clause product takes: with it the K factors of a clause stay below 2^1000. A
-// larger one (a literal false with probability below 2^-125) changes no w.
+// larger one (a literal false with probability below 2^-125) leaves every other m below 2^-125.
 template <int K>
 __device__ __forceinline__ double cut_factor(double d) {
   constexpr int kHi = (1023 + 1000 / K) << 20;  // high word of 2^(1000 / K)
   return __double2hiint(d) >= kHi ? __hiloint2double(kHi, 0) : d;
 }
 
-// |x| to 20 bits as a float, for |x| < 2^128 (0 below 2^-126), with integer operations only.
+// |x| and x cut off to 24 bits as a float, for |x| < 2^128 (0 below 2^-126), with integer operations
+// only (a conversion takes the double-precision pipe).
 __device__ __forceinline__ float approx_abs(double x) {
   const int h = (__double2hiint(x) & 0x7FFFFFFF) - (896 << 20);
-  return h <= 0 ? 0.0f : __int_as_float(h << 3);
+  return h <= 0 ? 0.0f : __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)h, 3));
+}
+__device__ __forceinline__ float approx(double x) {
+  return __int_as_float(__float_as_int(approx_abs(x)) | (__double2hiint(x) & (int)0x80000000));
 }
 
-// E of every edge at the first lambda (G = e^{2 lambda eps s*} per variable and seed).
+// g[v][s] = expm1(2 |lambda eps_v|) with the sign of the bias lambda eps_v s*_{v,s}.
+__global__ void lbp_gain_kernel(const double *__restrict__ eps, const uint8_t *__restrict__ xs,
+                                int32_t n, int32_t S, double lambda, double *g) {
+  const long long total = (long long)n * S;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const double b = 2.0 * lambda * eps[i / S] * (2.0 * (double)xs[i] - 1.0);
+    g[i] = copysign(expm1(fabs(b)), b);
+  }
+}
+
+// Edges at the first lambda: E = e^{+-2 bias}.
 __global__ void lbp_init_prod_kernel(const int32_t *__restrict__ clits, long long n_edges, int32_t n,
-                                     int32_t S, const double *__restrict__ G, double *E) {
+                                     int32_t S, const double *__restrict__ g, double *E) {
   const long long total = n_edges * S;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const int l = clits[i / S];
     if (l >= 2 * n) continue;
-    const double g = G[(size_t)(l >> 1) * S + i % S];
-    E[i] = (l & 1) ? 1.0 / g : g;
+    const double b = g[(size_t)(l >> 1) * S + i % S], a = fabs(b);
+    if ((b < 0.0) == ((l & 1) != 0)) E[i] = a;  // the literal is the bias's: e^{|2 bias|}
+    else E[i] = a <= 1.0 ? -a / (1.0 + a) : -kEdgeScale / (1.0 + a);
   }
 }
 
-// G[v][s] = e^{2 lambda eps_v s*_{v,s}}.
-__global__ void lbp_gain_kernel(const double *__restrict__ eps, const uint8_t *__restrict__ xs,
-                                int32_t n, int32_t S, double lambda, double *G) {
-  const long long total = (long long)n * S;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x)
-    G[i] = exp(2.0 * lambda * eps[i / S] * (2.0 * (double)xs[i] - 1.0));
+// |ln(w / w_old)| of w = 1 - m, from the change of m and the smaller of the two w: the series where
+// it is short enough, else log1p.
+__device__ __forceinline__ double log_change(double chg, double m_max) {
+  const double r = fabs(chg) / (1.0 - m_max);
+  if (r < 1e-4) return r * fma(r, fma(r, fma(r, -0.25, 1.0 / 3.0), -0.5), 1.0);
+  return log1p(r);
 }
 
-// |ln(w / old)| with chg = w - old: the series where it is short enough, else log1p.
-__device__ __forceinline__ double log_change(double chg, double old) {
-  const double r = chg / old;
-  if (fabs(r) < 1e-4) return fabs(r * fma(r, fma(r, fma(r, -0.25, 1.0 / 3.0), -0.5), 1.0));
-  return fabs(log1p(r));
+// m = c prod_{j != i} 1 / (1 + E_j) of the K literals of a clause from their d = 1 + E: one
+// reciprocal of the product of all, by two Newton steps r (2 - x r) from the hardware's approximation,
+// with the rounding errors of that product in the second (first order: err is what the exact product
+// is above `all`). Without them the roundings of the product, larger than those of a product of
+// 1 / (1 + E) < 1, are amplified by e^{2 beta} in u. 1 <= all <= 2^1000, so nothing leaves the range.
+template <int K>
+__device__ __forceinline__ void clause_messages(const double (&d)[K], double c, double (&m)[K]) {
+  double all = d[0], err = 0.0;
+#pragma unroll
+  for (int q = 1; q < K; ++q) {
+    const double p = all * d[q];
+    const double e = fma(all, d[q], -p);
+    err = q > 1 ? fma(err, d[q], e) : e;
+    all = p;
+  }
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(all));
+  r = fma(r, fma(-all, r, 1.0), r);
+  r = c * fma(r, fma(-err, r, fma(-all, r, 1.0)), r);
+#pragma unroll
+  for (int q = 0; q < K; ++q) m[q] = __dmul_rn(d[q], r);  // not one operation with m - m_old
 }
 
-// Clause pass: w = 1 - c prod_{j != i} 1 / (1 + E_j) of every literal, from one division by the
-// product of all K factors. The largest change of u per seed, |ln(w / w_old)| / 2, is found in two steps:
-// single precision picks the edges that can hold the maximum (relative error below 2e-5, margin
-// twice that), and only those are evaluated in double precision, usually one per thread. The
-// recorded maximum does not depend on which thread comes first: an edge is passed over only when
-// a larger value is already recorded.
-// Bound by the double-precision pipe (2 lanes per cycle and SM): 27 instructions a clause and seed.
+// Clause pass. The largest change of u per seed, |ln(w / w_old)| / 2, is found in two steps: single
+// precision picks the edges that can hold the maximum, and only those are evaluated in double
+// precision, usually one per thread.
+// Bound by the double-precision pipe (2 lanes per cycle and SM).
 template <int K>
 __global__ void lbp_clause_prod_kernel(const int32_t *__restrict__ clits, int32_t m, int32_t n,
-                                       int32_t S, const double *__restrict__ E, double *w, double c,
+                                       int32_t S, const double *__restrict__ E, double *msg, double c,
                                        const int32_t *__restrict__ status, unsigned long long *dmax,
                                        int track) {
   const long long total = (long long)m * S;
@@ -184,40 +229,36 @@ __global__ void lbp_clause_prod_kernel(const int32_t *__restrict__ clits, int32_
     const int s = (int)(i - a * S);
     if (status && status[s] != kRunning) continue;
     const size_t e0 = (size_t)(a * K) * S + s;
-    double d[K], old[K];
+    double d[K], old[K], now[K];
     bool used[K];
-    double all = 1.0;
 #pragma unroll
     for (int q = 0; q < K; ++q) {
       used[q] = clits[a * K + q] < 2 * n;
-      d[q] = used[q] ? cut_factor<K>(1.0 + E[e0 + (size_t)q * S]) : 1.0;
-      old[q] = used[q] && track ? w[e0 + (size_t)q * S] : 1.0;
+      d[q] = used[q] ? cut_factor<K>(edge_plus_one(E[e0 + (size_t)q * S])) : 1.0;
+      old[q] = used[q] && track ? msg[e0 + (size_t)q * S] : 0.0;
     }
-#pragma unroll
-    for (int q = 0; q < K; ++q) all *= d[q];
-    const double r = 1.0 / all;
-    double chg[K], chg_top = 0.0, old_top = 1.0;
+    clause_messages<K>(d, c, now);
+    double chg[K], big[K], chg_top = 0.0, big_top = 0.0;
     float est[K], top = 0.0f;
 #pragma unroll
     for (int q = 0; q < K; ++q) {
-      const double wn = fma(-c, d[q] * r, 1.0);
-      if (used[q]) w[e0 + (size_t)q * S] = wn;
-      chg[q] = used[q] ? wn - old[q] : 0.0;
+      if (used[q]) msg[e0 + (size_t)q * S] = now[q];
+      chg[q] = used[q] ? now[q] - old[q] : 0.0;
+      big[q] = __double2hiint(chg[q]) < 0 ? old[q] : now[q];
       est[q] = 0.0f;
       if (track) {
-        const float x = __fdividef(approx_abs(chg[q]), approx_abs(old[q]));
-        est[q] = fabsf(log1pf(__double2hiint(chg[q]) < 0 ? -x : x));
+        est[q] = log1pf(__fdividef(approx_abs(chg[q]), 1.0f - approx_abs(big[q])));
         if (est[q] > top) {
           top = est[q];
           chg_top = chg[q];
-          old_top = old[q];
+          big_top = big[q];
         }
       }
     }
     if (!track || top == 0.0f) continue;
     const float seen = approx_abs(__longlong_as_double((long long)*(volatile unsigned long long *)&dmax[s]));
     if (0.5f * top * (1.0f + 4e-5f) < seen) continue;
-    double dm = log_change(chg_top, old_top);
+    double dm = log_change(chg_top, big_top);
     const float tie = top * (1.0f - 4e-5f);
     int ties = 0;
 #pragma unroll
@@ -225,35 +266,87 @@ __global__ void lbp_clause_prod_kernel(const int32_t *__restrict__ clits, int32_
     if (ties > 1) {  // another edge may hold the larger change
 #pragma unroll
       for (int q = 0; q < K; ++q)
-        if (est[q] >= tie) dm = fmax(dm, log_change(chg[q], old[q]));
+        if (est[q] >= tie) dm = fmax(dm, log_change(chg[q], big[q]));
     }
     if (dm > 0.0) atomicMax(&dmax[s], (unsigned long long)__double_as_longlong(0.5 * dm));
   }
 }
 
-// Products of w over the positive and the negated edges p0, p0 + step, ... of a variable for seed s.
+// A product of factors 1 - m as p + r, r the sum of p's rounding errors (first order; single precision
+// holds it well enough, and off the double-precision pipe. It counts errors as zero once p is below
+// 2^-73, a sum of u beyond 25).
+struct ProductSum {
+  double p;
+  float r;
+  __device__ __forceinline__ void factor(double m) {
+    const double q = fma(-p, m, p);
+    // the error of q: p - q is exact up to m = 1/2, beyond it as good as m itself
+    const double e = fma(-p, m, p - q);
+    r = fmaf(-r, approx_abs(m), r + approx(e));
+    p = q;
+  }
+};
+__device__ __forceinline__ ProductSum times(const ProductSum &a, const ProductSum &b) {
+  const double q = a.p * b.p;
+  return ProductSum{q, fmaf(approx_abs(a.p), b.r, fmaf(a.r, approx_abs(b.p), approx(fma(a.p, b.p, -q))))};
+}
+
+// e^{2 field} = top / den of a variable, with num = top - den.
+struct FieldRatio {
+  double num, top, den;
+};
+// From the products of 1 - m over the positive and the negated edges and the bias's g. The bias
+// multiplies the side that it makes larger, so nothing is taken from 1.
+__device__ __forceinline__ FieldRatio field_ratio(const ProductSum &pos, const ProductSum &neg, double g) {
+  const bool up = !(g < 0.0);
+  const double a = fabs(g);
+  const double ps = up ? neg.p : pos.p, pw = up ? pos.p : neg.p;
+  const double rs = (double)(up ? neg.r : pos.r), rw = (double)(up ? pos.r : neg.r);
+  const double num = fma(a, ps, ps - pw) + fma(a, rs, rs - rw);
+  const double big = fma(a, ps, ps) + fma(a, rs, rs), other = pw + rw;
+  return up ? FieldRatio{num, big, other} : FieldRatio{-num, other, big};
+}
+
+// Products over the positive and the negated edges of variable v for seed s: over every LANES-th edge
+// in each of LANES consecutive lanes, then over the lanes (all get the result).
+template <int LANES>
 __device__ __forceinline__ void edge_products(const int32_t *vedge, const int32_t *clits, int p0,
-                                              int p1, int step, int S, int s, const double *w,
-                                              double &pp, double &pn) {
-  pp = pn = 1.0;
+                                              int p1, int S, int s, const double *msg,
+                                              ProductSum &pos, ProductSum &neg) {
+  const int sub = LANES == 1 ? 0 : (int)threadIdx.x % LANES;
+  pos = neg = ProductSum{1.0, 0.0f};
 #pragma unroll 4
-  for (int p = p0; p < p1; p += step) {
+  for (int p = p0 + sub; p < p1; p += LANES) {
     const long long e = vedge[p];
-    const double x = w[e * S + s];
-    if (clits[e] & 1) pn *= x;
-    else pp *= x;
+    const double m = msg[e * S + s];
+    const bool sign = clits[e] & 1;
+    ProductSum x = sign ? neg : pos;
+    x.factor(m);
+    pos = sign ? pos : x;
+    neg = sign ? x : neg;
+  }
+  if constexpr (LANES > 1) {
+    const unsigned team = ((1u << LANES) - 1u) << ((threadIdx.x & 31) - sub);
+    const auto over_lanes = [&](ProductSum &f) {
+#pragma unroll
+      for (int o = LANES / 2; o > 0; o >>= 1) {
+        const ProductSum other{__shfl_xor_sync(team, f.p, o), __shfl_xor_sync(team, f.r, o)};
+        f = sub & o ? times(other, f) : times(f, other);
+      }
+    };
+    over_lanes(pos);
+    over_lanes(neg);
   }
 }
 
-// Variable pass: e^{2 field} = G prod_neg w / prod_pos w, and E = e^{+-2 field} w of each edge
-// (the cavity takes the edge's own message out again). LANES consecutive lanes share a variable
-// and seed and split its edges: one where there are enough of them to fill the GPU (coalesced over
-// seeds), eight where a single lane's chain of loads and products would be the time (5 seeds of a
-// 500-variable formula).
+// Variable pass: the field of v for seed s, and E = e^{+-2 field} (1 - m) of each edge (the cavity
+// takes the edge's own message out again). LANES = 1 where there are enough variables and seeds to
+// fill the GPU (coalesced over seeds), 8 where a single lane's chain of loads and products would be
+// the time (5 seeds of a 500-variable formula).
 template <int LANES>
 __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int32_t *__restrict__ vedge,
                                     const int32_t *__restrict__ clits, int32_t n, int32_t S,
-                                    const double *__restrict__ G, const double *__restrict__ w,
+                                    const double *__restrict__ g, const double *__restrict__ msg,
                                     double *E, const int32_t *__restrict__ status) {
   const long long total = (long long)n * S;
   const int sub = threadIdx.x % LANES;
@@ -263,44 +356,48 @@ __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int3
     const int v = (int)(i / S), s = (int)(i - (long long)v * S);
     if (status[s] != kRunning) continue;
     const int p0 = vptr[v], p1 = vptr[v + 1];
-    double pp, pn;
-    edge_products(vedge, clits, p0 + sub, p1, LANES, S, s, w, pp, pn);
-    if (LANES > 1) {
-      const unsigned team = ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) - sub);
-#pragma unroll
-      for (int o = LANES / 2; o > 0; o >>= 1) {
-        pp *= __shfl_xor_sync(team, pp, o);
-        pn *= __shfl_xor_sync(team, pn, o);
-      }
-    }
-    pn *= G[i];
-    const double x = pn / pp, xi = pp / pn;
+    ProductSum pos, neg;
+    edge_products<LANES>(vedge, clits, p0, p1, S, s, msg, pos, neg);
+    const FieldRatio f = field_ratio(pos, neg, g[i]);
+    // an edge's v as a m + b, for each sign (see edge_scaled)
+    const auto line = [](double top, double den, double num, double &a, double &b) {
+      const double y = num / den;
+      b = y < -0.5 ? -kEdgeScale * (top / den) : y;
+      a = y < -0.5 ? -b : -(1.0 + y);
+    };
+    double ap, bp, an, bn;
+    line(f.top, f.den, f.num, ap, bp);
+    line(f.den, f.top, -f.num, an, bn);
 #pragma unroll 4
     for (int p = p0 + sub; p < p1; p += LANES) {
       const long long e = vedge[p];
-      E[e * S + s] = ((clits[e] & 1) ? xi : x) * w[e * S + s];
+      const bool sign = clits[e] & 1;
+      E[e * S + s] = fma(sign ? an : ap, msg[e * S + s], sign ? bn : bp);
     }
   }
 }
 
-// Marginals <r_v> = tanh field = (a - b) / (a + b), a / b = e^{2 field}, each seed at its own
-// lambda. Written as 1 - 2 b / (a + b) or its mirror image, whichever term is the small one.
+// Marginals <r_v> = tanh field = num / (top + den), each seed at its own lambda; away from zero as
+// 1 - 2 den / (top + den) or its mirror image, whichever term is the small one.
 __global__ void lbp_marg_prod_kernel(const int32_t *__restrict__ vptr, const int32_t *__restrict__ vedge,
                                      const int32_t *__restrict__ clits,
                                      const int32_t *__restrict__ orig, int32_t n, int32_t S,
                                      const double *__restrict__ eps, const uint8_t *__restrict__ xs,
                                      const double *__restrict__ lambdas,
                                      const int32_t *__restrict__ lam_idx,
-                                     const double *__restrict__ w, double *marg) {
+                                     const double *__restrict__ msg, double *marg) {
   const long long total = (long long)n * S;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const int v = (int)(i / S), s = (int)(i - (long long)v * S);
-    double pp, pn;
-    edge_products(vedge, clits, vptr[v], vptr[v + 1], 1, S, s, w, pp, pn);
-    pn *= exp(2.0 * lambdas[lam_idx[s]] * eps[v] * (2.0 * (double)xs[i] - 1.0));
-    marg[(size_t)s * n + orig[v]] =
-        pn >= pp ? fma(-2.0, pp / (pn + pp), 1.0) : fma(2.0, pn / (pn + pp), -1.0);
+    ProductSum pos, neg;
+    edge_products<1>(vedge, clits, vptr[v], vptr[v + 1], S, s, msg, pos, neg);
+    const double b = 2.0 * lambdas[lam_idx[s]] * eps[v] * (2.0 * (double)xs[i] - 1.0);
+    const FieldRatio f = field_ratio(pos, neg, copysign(expm1(fabs(b)), b));
+    const double sum = f.top + f.den;
+    marg[(size_t)s * n + orig[v]] = 4.0 * fabs(f.num) < sum ? f.num / sum
+                                    : f.num > 0.0           ? fma(-2.0, f.den / sum, 1.0)
+                                                            : fma(2.0, f.top / sum, -1.0);
   }
 }
 
@@ -332,8 +429,8 @@ __global__ void lbp_overlap_kernel(const int32_t *__restrict__ orig, int32_t n, 
   }
 }
 
-// Clause correlations as lbp_corr_kernel, from f = 1 / (1 + E) = (1 - t) / 2; t = 1 - 2 f or
-// 2 E f - 1, whichever has the small product.
+// Clause correlations as lbp_corr_kernel, from f = 1 / (1 + E) = (1 - t) / 2 and t = tanh h, each from
+// whichever of E - 1, E and 1 / E is the small one.
 __global__ void lbp_corr_prod_kernel(const int32_t *__restrict__ clits, int32_t m, int32_t kmax,
                                      int32_t n, int32_t S, const double *__restrict__ E, double c,
                                      double *corr) {
@@ -348,22 +445,33 @@ __global__ void lbp_corr_prod_kernel(const int32_t *__restrict__ clits, int32_t 
       const long long e = a * kmax + q;
       const int l = clits[e];
       if (l >= 2 * n) continue;
-      const double sg = lit_sigma(l), x = E[e * S + s], f = 1.0 / (1.0 + x);
-      free_prod *= sg * (x >= 1.0 ? fma(-2.0, f, 1.0) : fma(2.0 * x, f, -1.0));
+      const double sg = lit_sigma(l), v = E[e * S + s];
+      double f = 1.0 / edge_plus_one(v), t;
+      if (v >= 1.0) {  // E >= 2
+        t = fma(-2.0, f, 1.0);
+      } else if (v > -0.5) {
+        t = v * f;
+        f = fma(-0.5, t, 0.5);
+      } else {
+        const double x = edge_scaled(v) ? v * (-1.0 / kEdgeScale) : 1.0 + v;
+        t = fma(2.0 * x, f, -1.0);
+        f = fma(-x, f, 1.0);
+      }
+      free_prod *= sg * t;
       viol_prod *= f;
       sign *= -sg;
       ++k;
     }
-    const double z = 1.0 - c * viol_prod;
-    corr[(size_t)s * m + a] = k > 0 ? (free_prod - c * sign * viol_prod) / z : 0.0;
+    corr[(size_t)s * m + a] = k > 0 ? fma(-c * sign, viol_prod, free_prod) / fma(-c, viol_prod, 1.0) : 0.0;
   }
 }
 
 template <int K>
-void clause_prod(const int32_t *clits, int32_t m, int32_t n, int32_t S, const double *E, double *w,
+void clause_prod(const int32_t *clits, int32_t m, int32_t n, int32_t S, const double *E, double *msg,
                  double c, const int32_t *status, unsigned long long *dmax, int track,
                  unsigned grid, cudaStream_t st) {
-  lbp_clause_prod_kernel<K><<<grid, kLbpBlock, 0, st>>>(clits, m, n, S, E, w, c, status, dmax, track);
+  lbp_clause_prod_kernel<K><<<grid, kLbpBlock, 0, st>>>(clits, m, n, S, E, msg, c, status, dmax,
+                                                      track);
 }
 
 // Per seed after an iteration at lambda index k: count, convergence, failure, bookkeeping.
@@ -558,10 +666,10 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
   const unsigned gS = (unsigned)((S + kLbpBlock - 1) / kLbpBlock);
   const unsigned gVS = blocks_for((long long)n * S), gMS = blocks_for((long long)m * S),
                  gES = blocks_for(E * S);
-  // the product form needs every product of w and every e^{2 field} inside the range of a double:
-  // u lies in [0, beta], so |field| <= beta deg + |lambda eps|. w is resolved to about 1e-16, a
-  // change of u to 1e-16 e^{2 beta} / 2: smaller tolerances take the log form, whose resolution is
-  // the same for large u but finer for small ones
+  // the product form needs every product of 1 - m and every e^{2 field} inside the range of a double:
+  // u lies in [0, beta], so |field| <= beta deg + |lambda eps|. m near c is resolved to about 1e-16, a
+  // change of u to 1e-16 e^{2 beta} / 2: smaller tolerances take the log form, which has settled as
+  // far as it can there
   const bool prod = A.beta <= 4.0 && A.beta * A.max_deg + A.max_bias < 340.0 &&
                     A.tol >= 2e-15 * exp(2.0 * A.beta);
   const bool split = (long long)n * S < 152 * 256;  // fewer than eight warps an SM otherwise
