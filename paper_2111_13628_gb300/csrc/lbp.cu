@@ -215,13 +215,17 @@ __device__ __forceinline__ void clause_messages(const double (&d)[K], double c, 
 
 // Clause pass. The largest change of u per seed, |ln(w / w_old)| / 2, is found in two steps: single
 // precision picks the edges that can hold the maximum, and only those are evaluated in double
-// precision, usually one per thread.
+// precision, usually one per thread. The single-precision value is log1p(|m - m_old| / w), w the
+// smaller of the two 1 - m, whose relative error e^{2 beta} 2^-23 (m cut off to 24 bits, w >= e^{-2
+// beta}) outweighs all others; `slack` is four times its bound, so an edge is passed over only when
+// a larger value is already recorded, and the recorded maximum does not depend on which thread comes
+// first.
 // Bound by the double-precision pipe (2 lanes per cycle and SM).
 template <int K>
 __global__ void lbp_clause_prod_kernel(const int32_t *__restrict__ clits, int32_t m, int32_t n,
                                        int32_t S, const double *__restrict__ E, double *msg, double c,
                                        const int32_t *__restrict__ status, unsigned long long *dmax,
-                                       int track) {
+                                       int track, float slack) {
   const long long total = (long long)m * S;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -257,9 +261,9 @@ __global__ void lbp_clause_prod_kernel(const int32_t *__restrict__ clits, int32_
     }
     if (!track || top == 0.0f) continue;
     const float seen = approx_abs(__longlong_as_double((long long)*(volatile unsigned long long *)&dmax[s]));
-    if (0.5f * top * (1.0f + 4e-5f) < seen) continue;
+    if (0.5f * top * (1.0f + slack) < seen) continue;
     double dm = log_change(chg_top, big_top);
-    const float tie = top * (1.0f - 4e-5f);
+    const float tie = top * (1.0f - slack);
     int ties = 0;
 #pragma unroll
     for (int q = 0; q < K; ++q) ties += est[q] >= tie;
@@ -468,10 +472,10 @@ __global__ void lbp_corr_prod_kernel(const int32_t *__restrict__ clits, int32_t 
 
 template <int K>
 void clause_prod(const int32_t *clits, int32_t m, int32_t n, int32_t S, const double *E, double *msg,
-                 double c, const int32_t *status, unsigned long long *dmax, int track,
+                 double c, const int32_t *status, unsigned long long *dmax, int track, float slack,
                  unsigned grid, cudaStream_t st) {
-  lbp_clause_prod_kernel<K><<<grid, kLbpBlock, 0, st>>>(clits, m, n, S, E, msg, c, status, dmax,
-                                                      track);
+  lbp_clause_prod_kernel<K><<<grid, kLbpBlock, 0, st>>>(clits, m, n, S, E, msg, c, status, dmax, track,
+                                                      slack);
 }
 
 // Per seed after an iteration at lambda index k: count, convergence, failure, bookkeeping.
@@ -673,6 +677,7 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
   const bool prod = A.beta <= 4.0 && A.beta * A.max_deg + A.max_bias < 340.0 &&
                     A.tol >= 2e-15 * exp(2.0 * A.beta);
   const bool split = (long long)n * S < 152 * 256;  // fewer than eight warps an SM otherwise
+  const float slack = (float)((exp(2.0 * A.beta) + 8.0) * 0x1p-21);
   const auto clause = [&](const int32_t *seeds, int track) {
     if (!prod) {
       lbp_clause_kernel<<<gMS, kLbpBlock, 0, st>>>(A.clits, m, kmax, n, S, h, u, c, seeds, dmax, track);
@@ -680,7 +685,7 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
     }
     switch (kmax) {
 #define LBP_CASE(k) \
-  case k: clause_prod<k>(A.clits, m, n, S, h, u, c, seeds, dmax, track, gMS, st); break;
+  case k: clause_prod<k>(A.clits, m, n, S, h, u, c, seeds, dmax, track, slack, gMS, st); break;
       LBP_CASE(1) LBP_CASE(2) LBP_CASE(3) LBP_CASE(4)
       LBP_CASE(5) LBP_CASE(6) LBP_CASE(7) LBP_CASE(8)
 #undef LBP_CASE
