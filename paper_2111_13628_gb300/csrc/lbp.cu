@@ -311,41 +311,61 @@ __device__ __forceinline__ FieldRatio field_ratio(const ProductSum &pos, const P
   return up ? FieldRatio{num, big, other} : FieldRatio{-num, other, big};
 }
 
-// Products over the positive and the negated edges of variable v for seed s: over every LANES-th edge
-// in each of LANES consecutive lanes, then over the lanes (all get the result).
+// Products over the positive and the negated edges of variable v for seed s, always in the same
+// order, whatever the launch: four of each, over every fourth edge, then (0 2)(1 3). LANES = 4: one of
+// the four in each of four consecutive lanes (all get the result); LANES = 1: all in one.
 template <int LANES>
 __device__ __forceinline__ void edge_products(const int32_t *vedge, const int32_t *clits, int p0,
                                               int p1, int S, int s, const double *msg,
                                               ProductSum &pos, ProductSum &neg) {
+  constexpr int PER = 4 / LANES;
   const int sub = LANES == 1 ? 0 : (int)threadIdx.x % LANES;
-  pos = neg = ProductSum{1.0, 0.0f};
-#pragma unroll 4
-  for (int p = p0 + sub; p < p1; p += LANES) {
-    const long long e = vedge[p];
-    const double m = msg[e * S + s];
-    const bool sign = clits[e] & 1;
-    ProductSum x = sign ? neg : pos;
-    x.factor(m);
-    pos = sign ? pos : x;
-    neg = sign ? x : neg;
-  }
-  if constexpr (LANES > 1) {
-    const unsigned team = ((1u << LANES) - 1u) << ((threadIdx.x & 31) - sub);
-    const auto over_lanes = [&](ProductSum &f) {
+  ProductSum f[2][PER];
 #pragma unroll
-      for (int o = LANES / 2; o > 0; o >>= 1) {
-        const ProductSum other{__shfl_xor_sync(team, f.p, o), __shfl_xor_sync(team, f.r, o)};
-        f = sub & o ? times(other, f) : times(f, other);
+  for (int j = 0; j < PER; ++j) f[0][j] = f[1][j] = ProductSum{1.0, 0.0f};
+#pragma unroll (LANES == 1 ? 2 : 8)
+  for (int p = p0 + sub; p < p1; p += 4) {
+    double m[PER];
+    int sign[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      m[j] = 0.0;
+      sign[j] = 0;
+      if (p + j < p1) {
+        const long long e = vedge[p + j];
+        m[j] = msg[e * S + s];
+        sign[j] = clits[e] & 1;
       }
-    };
-    over_lanes(pos);
-    over_lanes(neg);
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {  // a factor of m = 0 changes nothing
+      ProductSum x = sign[j] ? f[1][j] : f[0][j];
+      x.factor(m[j]);
+      f[0][j] = sign[j] ? f[0][j] : x;
+      f[1][j] = sign[j] ? x : f[1][j];
+    }
+  }
+  if constexpr (LANES == 1) {
+    pos = times(times(f[0][0], f[0][2]), times(f[0][1], f[0][3]));
+    neg = times(times(f[1][0], f[1][2]), times(f[1][1], f[1][3]));
+  } else {
+    const unsigned team = 0xFu << ((threadIdx.x & 31) - sub);
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+#pragma unroll
+      for (int o = 2; o > 0; o >>= 1) {
+        const ProductSum &mine = f[z][0];
+        const ProductSum other{__shfl_xor_sync(team, mine.p, o), __shfl_xor_sync(team, mine.r, o)};
+        f[z][0] = sub & o ? times(other, mine) : times(mine, other);
+      }
+    pos = f[0][0];
+    neg = f[1][0];
   }
 }
 
 // Variable pass: the field of v for seed s, and E = e^{+-2 field} (1 - m) of each edge (the cavity
 // takes the edge's own message out again). LANES = 1 where there are enough variables and seeds to
-// fill the GPU (coalesced over seeds), 8 where a single lane's chain of loads and products would be
+// fill the GPU (coalesced over seeds), 4 where a single lane's chain of loads and products would be
 // the time (5 seeds of a 500-variable formula).
 template <int LANES>
 __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int32_t *__restrict__ vedge,
@@ -372,7 +392,7 @@ __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int3
     double ap, bp, an, bn;
     line(f.top, f.den, f.num, ap, bp);
     line(f.den, f.top, -f.num, an, bn);
-#pragma unroll 4
+#pragma unroll (LANES == 1 ? 4 : 8)
     for (int p = p0 + sub; p < p1; p += LANES) {
       const long long e = vedge[p];
       const bool sign = clits[e] & 1;
@@ -711,7 +731,7 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
     // alone), and the GPU does not wait for the host in between.
     for (int32_t it = 0; it < A.max_iter; ++it) {
       if (prod && split)
-        lbp_var_prod_kernel<8><<<blocks_for(8LL * n * S), kLbpBlock, 0, st>>>(
+        lbp_var_prod_kernel<4><<<blocks_for(4LL * n * S), kLbpBlock, 0, st>>>(
             A.vptr, A.vedge, A.clits, n, S, bias, u, h, status);
       else if (prod)
         lbp_var_prod_kernel<1><<<gVS, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, n, S, bias, u, h,
