@@ -432,11 +432,13 @@ int nmc_server_stats(nmc_server *srv, int64_t *ticks, int64_t *attempts, double 
 /* Message of the last failed nmc_server_result. */
 const char *nmc_server_last_error(nmc_server *srv);
 
-/* Self-test of the bounded device wait: launches one CTA that waits at the grid barrier the
+/* Self-test of the bounded device waits: launches one CTA that waits at the grid barrier the
  * sweep kernel uses, for a second arrival that never comes, with the given limit in
- * milliseconds (1..10000). Returns NMC_ETIMEOUT when the wait expired and was reported as
- * the sweep would report it, NMC_OK if it did not expire (a defect), or an error code. The
- * context stays usable afterwards. */
+ * milliseconds (1..10000), then a cluster of two CTAs of which one waits at the batched
+ * kernel's class barrier for the other, for about as long, over three work items. Returns
+ * NMC_ETIMEOUT when both waits expired and were reported as the sweeps would report them (the
+ * second for every item), NMC_OK if not (a defect), or an error code. The context stays
+ * usable afterwards. */
 int nmc_selftest_wait_timeout(nmc_ctx *ctx, int32_t timeout_ms);
 
 /* The library's acceptance-threshold table: writes min(cap, L) entries

@@ -731,8 +731,29 @@ int nmc_selftest_wait_timeout(nmc_ctx *ctx, int32_t timeout_ms) {
   if (e == cudaSuccess) e = cudaMemcpy(&host, gb, sizeof(GridBarrier), cudaMemcpyDeviceToHost);
   cudaFree(gb);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "wait self-test");
-  if (host.sticky && host.error) return fail(ctx, NMC_ETIMEOUT, "bounded wait expired as designed");
-  return NMC_OK;
+  if (!host.sticky || !host.error) return NMC_OK;
+  // the class barrier of the batched kernel: three items, all of which must be marked, and only they
+  constexpr int kItems = 3;
+  int32_t *best = nullptr, got[kItems][33];
+  BatchItem *items = nullptr, its[kItems] = {};
+  e = dev_alloc(&best, kItems * 33);
+  if (e == cudaSuccess) e = dev_alloc(&items, kItems);
+  if (e == cudaSuccess) e = cudaMemset(best, 0, sizeof(got));
+  for (int i = 0; i < kItems; ++i) {
+    its[i].W = 1;
+    its[i].best_energy = best + 33 * i;
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(items, its, sizeof(its), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = step_selftest(items, kItems, 2000000ll * timeout_ms, ctx->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  if (e == cudaSuccess) e = cudaMemcpy(got, best, sizeof(got), cudaMemcpyDeviceToHost);
+  dev_free(items);
+  dev_free(best);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "wait self-test");
+  for (int i = 0; i < kItems; ++i)
+    for (int j = 0; j < 33; ++j)
+      if (got[i][j] != (j == 32 ? kStepTimeout : 0)) return NMC_OK;
+  return fail(ctx, NMC_ETIMEOUT, "bounded waits expired as designed");
 }
 
 int32_t nmc_threshold_table(uint32_t *out, int32_t cap) {

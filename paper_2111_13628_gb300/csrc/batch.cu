@@ -460,30 +460,52 @@ struct EnergyTrack {
 // a step ahead are words nobody reads any more: every warp with a variable in the class has stored it,
 // hence finished reading, and warps counting ahead read neither their own class nor the one before.
 // The last class of a sweep meets at the hardware cluster barrier, which also publishes the CTAs'
-// energy changes. A wait gives up after about a second, marks the set (kStepTimeout at the end of
-// best_energy) and lets the rest of the launch run through without waiting.
+// energy changes.
+//
+// A wait gives up after about a second. Its warp is `dead` from then on: it marks the set at hand and
+// that of every later item of the launch (kStepTimeout at the end of best_energy), runs through
+// without waiting, and leaves the mbarriers alone, whose phases it no longer follows: its words are
+// plain stores, and the warps that wait for it give up as well.
 constexpr long long kStepLimitCycles = 1ll << 31;
+constexpr long long kDrainCycles = 1ll << 21;  // a millisecond: hundreds of times what a store takes
 
 template <int CS, int WARPS>
 struct ClassBarrier {
   uint32_t bar;                 // shared address of full[0]
   uint32_t arrived, waited;     // steps at the mbarriers so far
-  bool dead;
+  bool dead;                    // of the warp: a wait has given up
+  long long limit;
 
   // by all threads, before a barrier of the CTAs
-  __device__ __forceinline__ void init(SweepShared &sh) {
+  __device__ __forceinline__ void init(SweepShared &sh, long long limit_cycles = kStepLimitCycles) {
     bar = (uint32_t)__cvta_generic_to_shared(&sh.full[0]);
     arrived = waited = 0;
     dead = false;
+    limit = limit_cycles;
     if (CS > 1 && threadIdx.x == 0) {
       for (int i = 0; i < 2; ++i)
         asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(bar + 8 * i), "r"(WARPS + CS) : "memory");
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
   }
+  __device__ __forceinline__ static void mark(const BatchItem &B) { B.best_energy[32 * B.W] = kStepTimeout; }
+  // Before the first class of an item.
+  __device__ __forceinline__ void begin(const BatchItem &B) const {
+    if (CS > 1 && dead) mark(B);
+  }
+  // After the barrier of the CTAs that ends an item; the CTAs meet again before any of them exits.
+  // A dead warp holds them until the cluster's asynchronous stores, which nobody waits for any more,
+  // have arrived in shared memory that is still there.
+  __device__ __forceinline__ void drain() const {
+    if (CS > 1 && dead) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < kDrainCycles) {
+      }
+    }
+  }
   // Stores v at word `saddr` of CTA `rank`, as part of the step being worked on.
   __device__ __forceinline__ void store(uint32_t saddr, int rank, uint32_t v, bool last) const {
-    if (last)
+    if (last || dead)
       asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(shared_at(saddr, rank)), "r"(v) : "memory");
     else
       asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(
@@ -502,6 +524,8 @@ struct ClassBarrier {
     } else {
       const int lane = threadIdx.x & 31;
       const uint32_t b = bar + 8 * (arrived & 1);
+      ++arrived;
+      if (dead) return;
       if (threadIdx.x < CS)
         asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(
                          shared_at(b, threadIdx.x))
@@ -511,7 +535,6 @@ struct ClassBarrier {
                      : "memory");
       else if (lane == 0)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
-      ++arrived;
     }
   }
   // Waits for the class before the one at hand (last: the sweep's last one).
@@ -535,9 +558,9 @@ struct ClassBarrier {
           : "memory");
       if (done) break;
       if (t0 == 0) t0 = clock64();
-      if (clock64() - t0 > kStepLimitCycles) {
+      if (clock64() - t0 > limit) {
         dead = true;
-        B.best_energy[32 * B.W] = kStepTimeout;
+        mark(B);
         break;
       }
     }
@@ -662,6 +685,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
     const BatchItem &B = sh.item;
     EnergyTrack track;
     load_item<CS, PT>(B, rank, xs, sh, track);
+    step.begin(B);
     group_sync<CS>();
     for (int t = B.t0; t < B.t1; ++t) {
       uint32_t acc[kAccPlanes];
@@ -776,6 +800,7 @@ __global__ void __launch_bounds__(one_thread_threads<KQ>(), 1)
     }
     store_item<CS, PT>(B, rank, xs, track);
     group_sync<CS>();
+    step.drain();
   }
 }
 
@@ -873,6 +898,7 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
     const int32_t inert_off = n * 4;
     EnergyTrack track;
     load_item<CS, PT>(B, rank, xs, sh, track);
+    step.begin(B);
     uint32_t pm[PT ? RPL : 1];  // the lane's replicas' temperature multipliers
     if (PT) {
 #pragma unroll
@@ -1134,7 +1160,32 @@ __global__ void __launch_bounds__(sweep_threads<KQ, TL>(), 1)
     }
     store_item<CS, PT>(B, rank, xs, track);
     group_sync<CS>();
+    step.drain();
   }
+}
+
+// The class barrier between two CTAs of which one never arrives at the first step, over n items of two
+// classes each (items[i].W == 1): the other's wait runs out at the first item, and every item has to
+// be marked. Both keep meeting at the cluster barrier.
+constexpr int kSelftestThreads = 64;
+__global__ void __cluster_dims__(2, 1, 1) step_selftest_kernel(const BatchItem *items, int n, long long limit) {
+  __shared__ SweepShared sh;
+  const bool absent = cg::this_cluster().block_rank() == 1;
+  ClassBarrier<2, kSelftestThreads / 32> step;
+  step.init(sh, limit);
+  group_sync<2>();
+  for (int i = 0; i < n; ++i) {
+    const BatchItem &B = items[i];
+    step.begin(B);
+    if (!absent) {
+      step.arrive(0, false);
+      step.wait(B, false);
+    }
+    step.arrive(0, true);
+    step.wait(B, true);
+    step.drain();
+  }
+  group_sync<2>();
 }
 
 // The launch shape of each kernel instance is queried once per (device, shared-memory size):
@@ -1387,6 +1438,11 @@ size_t batch_max_vars(int tab_len, int device) {
   // dynamic shared memory: table + n+1 words; the static part is under 192 words
   const long long words = (long long)optin / 4 - tab_len - 1 - 32 - 1 - 192;
   return words > 0 ? (size_t)words : 0;
+}
+
+cudaError_t step_selftest(const BatchItem *items_dev, int n, long long limit_cycles, cudaStream_t st) {
+  step_selftest_kernel<<<2, kSelftestThreads, 0, st>>>(items_dev, n, limit_cycles);
+  return cudaGetLastError();
 }
 
 cudaError_t ksat_batch(const BatchItem *items_dev, int n_items, int kq, int cs, int max_n,

@@ -131,8 +131,12 @@ cudaError_t quantize_schedule(const float *beta, int32_t n_units, int32_t n_step
                               cudaStream_t st);
 
 // ---- batched k-SAT (batch.cu) -----------------------------------------------------------
-// Left in best_energy[32 W] of a set when a wait between the CTAs of its word gave up.
+// Left in best_energy[32 W] of a set when a wait between the CTAs of its word gave up, or one of an
+// earlier item of the same cluster had.
 constexpr int32_t kStepTimeout = 1;
+// Runs the class barrier of n items (W = 1, best_energy 33 ints each) into a wait of limit_cycles that
+// nothing ends; all of them are marked afterwards.
+cudaError_t step_selftest(const BatchItem *items_dev, int n, long long limit_cycles, cudaStream_t st);
 // Largest n whose word vector fits the batched kernel's shared memory on `device`.
 size_t batch_max_vars(int tab_len, int device);
 // Clusters of cs (2, 4, 8) CTAs that run at once on `device` with one CTA per SM.
