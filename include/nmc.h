@@ -435,10 +435,11 @@ const char *nmc_server_last_error(nmc_server *srv);
 /* Self-test of the bounded device waits: launches one CTA that waits at the grid barrier the
  * sweep kernel uses, for a second arrival that never comes, with the given limit in
  * milliseconds (1..10000), then a cluster of two CTAs of which one waits at the batched
- * kernel's class barrier for the other, for about as long, over three work items. Returns
- * NMC_ETIMEOUT when both waits expired and were reported as the sweeps would report them (the
- * second for every item), NMC_OK if not (a defect), or an error code. The context stays
- * usable afterwards. */
+ * kernel's class barrier for the other, for about as long, over three work items, and the
+ * same twice for a small replica set. Returns NMC_ETIMEOUT when the waits expired and were
+ * reported as the sweeps would report them (every item; the set also after a later valid
+ * launch, once, and not after a reset), NMC_OK if not (a defect), or an error code. The
+ * context stays usable afterwards. */
 int nmc_selftest_wait_timeout(nmc_ctx *ctx, int32_t timeout_ms);
 
 /* The library's acceptance-threshold table: writes min(cap, L) entries

@@ -42,7 +42,6 @@ struct ReplicaSet {
   uint64_t seed = 0;
   KsatReplicas ks{};
   QapReplicas qp{};
-  bool clusters = false;  // k-SAT: last launched with several CTAs per word
   // temperature ladder (k-SAT replica exchange); pt_L = 0 without one
   int32_t pt_L = 0;
   uint32_t *pt_lq = nullptr;    // pt_L Q16 inverse temperatures of the slots
@@ -174,8 +173,8 @@ void free_set(ReplicaSet &S) {
   dev_free(S.ks.best);
   dev_free(S.ks.energy);
   dev_free(S.ks.best_energy);
+  S.ks.bar = nullptr;
   dev_free(S.ks.imp);
-  dev_free(S.ks.bar);
   dev_free(S.qp.perm);
   dev_free(S.qp.best_perm);
   dev_free(S.qp.energy);
@@ -200,24 +199,22 @@ ReplicaSet *find_set(nmc_ctx *ctx, int32_t id) {
 // Checks the sticky timeout word of a k-SAT replica set after its stream was synchronised.
 int check_timeout(nmc_ctx *ctx, ReplicaSet &S) {
   if (!S.ks.bar) return NMC_OK;
-  if (S.clusters) {
-    int32_t status = 0;
-    int32_t *at = S.ks.best_energy + 32 * S.ks.W;
-    NMC_CUDA(cudaMemcpy(&status, at, sizeof(int32_t), cudaMemcpyDeviceToHost), "read step status");
-    if (status == kStepTimeout) {
-      cudaMemset(at, 0, sizeof(int32_t));
-      return fail(ctx, NMC_ETIMEOUT, "a wait between the CTAs of a word expired; the sweep is void");
-    }
-  }
   int sticky = 0;
   NMC_CUDA(cudaMemcpy(&sticky, &S.ks.bar->sticky, sizeof(int), cudaMemcpyDeviceToHost),
            "read barrier status");
   if (sticky) {
     const int zero = 0;
     cudaMemcpy(&S.ks.bar->sticky, &zero, sizeof(int), cudaMemcpyHostToDevice);
-    return fail(ctx, NMC_ETIMEOUT, "a grid barrier wait expired; the sweep stopped early");
+    return fail(ctx, NMC_ETIMEOUT, sticky == kStepTimeout
+                                       ? "a wait between the CTAs of a word expired; the sweep is void"
+                                       : "a grid barrier wait expired; the sweep stopped early");
   }
   return NMC_OK;
+}
+
+// What an expired wait left behind goes with the states it spoiled, when those are replaced.
+cudaError_t clear_timeout(nmc_ctx *ctx, ReplicaSet &S) {
+  return S.ks.bar ? cudaMemsetAsync(&S.ks.bar->sticky, 0, sizeof(int), ctx->stream) : cudaSuccess;
 }
 
 // Host-side check of caller-given initial states.
@@ -385,7 +382,6 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
   plan->max_n[0] = plan->max_n[1] = 0;
   int per_class[2] = {0, 0};  // largest mean colour-class size among the items
   std::vector<SetShape> shapes;
-  std::vector<ReplicaSet *> shaped;
   std::vector<int> owner[2];  // an item's index in shapes
   for (int32_t i = 0; i < n_sets; ++i) {
     ReplicaSet *S = find_set(ctx, rs[i]);
@@ -402,7 +398,6 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
     if (t1[i] == t0[i]) continue;
     const int q = I->ks.kq == 1 ? 0 : 1;
     shapes.push_back({I, S->ks.W, t1[i] - t0[i], 1});
-    shaped.push_back(S);
     owner[q].insert(owner[q].end(), S->ks.W, static_cast<int>(shapes.size()) - 1);
     for (int32_t w = 0; w < S->ks.W; ++w) {
       BatchItem B{};
@@ -479,8 +474,6 @@ int batch_plan(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, const int32_t *t
     plan->cs[q] = cs;
     plan->lanes[q] = lanes;
     if (!mixed && plan->cnt[q]) plan->groups.push_back({q + 1, cs, lanes, plan->off[q], plan->cnt[q]});
-    for (size_t i = 0; i < shapes.size(); ++i)
-      if ((shapes[i].I->ks.kq == 1 ? 0 : 1) == q) shaped[i]->clusters = (mixed ? shapes[i].cs : cs) > 1;
   }
   // launch order: the largest clusters while the GPU is empty; without them the two-entry items
   // (k > 4) first
@@ -732,7 +725,9 @@ int nmc_selftest_wait_timeout(nmc_ctx *ctx, int32_t timeout_ms) {
   cudaFree(gb);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "wait self-test");
   if (!host.sticky || !host.error) return NMC_OK;
-  // the class barrier of the batched kernel: three items, all of which must be marked, and only they
+  // the class barrier of the batched kernel: items of their own, all of which must be marked, and
+  // only they, and then one of a replica set, which must be reported once, also after a launch on one
+  // CTA a word, and no longer after a reset
   constexpr int kItems = 3;
   int32_t *best = nullptr, got[kItems][33];
   BatchItem *items = nullptr, its[kItems] = {};
@@ -753,6 +748,42 @@ int nmc_selftest_wait_timeout(nmc_ctx *ctx, int32_t timeout_ms) {
   for (int i = 0; i < kItems; ++i)
     for (int j = 0; j < 33; ++j)
       if (got[i][j] != (j == 32 ? kStepTimeout : 0)) return NMC_OK;
+  const int32_t lits[2] = {1, -2};
+  const float beta[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+  const int32_t t0 = 0, t1 = 2;
+  int32_t inst = 0, rs = 0;
+  int rc = nmc_load_ksat(ctx, 2, 1, 2, lits, &inst);
+  if (rc != NMC_OK) return rc;
+  bool reported = false;
+  if ((rc = nmc_set_schedule(ctx, inst, 2, beta)) == NMC_OK &&
+      (rc = nmc_replicas_create(ctx, inst, 32, 1, nullptr, &rs)) == NMC_OK) {
+    ReplicaSet &S = *find_set(ctx, rs);
+    const auto give_up = [&] {
+      BatchItem it{};
+      it.W = 1;
+      it.best_energy = S.ks.best_energy;
+      BatchItem *dev = nullptr;
+      cudaError_t x = dev_alloc(&dev, 1);
+      if (x == cudaSuccess) x = cudaMemcpy(dev, &it, sizeof(it), cudaMemcpyHostToDevice);
+      if (x == cudaSuccess) x = step_selftest(dev, 1, 2000000ll * timeout_ms, ctx->stream);
+      if (x == cudaSuccess) x = cudaStreamSynchronize(ctx->stream);
+      dev_free(dev);
+      return x;
+    };
+    const auto outcome = [&] {
+      cudaStreamSynchronize(ctx->stream);
+      return check_timeout(ctx, S);
+    };
+    if ((e = give_up()) == cudaSuccess && (rc = nmc_batch_run(ctx, 1, &rs, &t0, &t1)) == NMC_OK) {
+      reported = outcome() == NMC_ETIMEOUT && outcome() == NMC_OK;
+      if ((e = give_up()) == cudaSuccess && (rc = nmc_replicas_reset(ctx, rs, 1, nullptr)) == NMC_OK)
+        reported = reported && outcome() == NMC_OK;
+    }
+    nmc_replicas_destroy(ctx, rs);
+  }
+  nmc_unload(ctx, inst);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "wait self-test");
+  if (rc != NMC_OK || !reported) return rc;
   return fail(ctx, NMC_ETIMEOUT, "bounded waits expired as designed");
 }
 
@@ -1672,10 +1703,9 @@ int nmc_replicas_create(nmc_ctx *ctx, int32_t inst, int32_t replicas, uint64_t s
     if ((e = dev_alloc(&S.ks.S, static_cast<size_t>(2 * n + 2) * W)) != cudaSuccess ||
         (e = dev_alloc(&S.ks.best, static_cast<size_t>(2 * n) * W)) != cudaSuccess ||
         (e = dev_alloc(&S.ks.energy, 32 * W)) != cudaSuccess ||
-        (e = dev_alloc(&S.ks.best_energy, 32 * W + 1)) != cudaSuccess ||  // and the step status
-        (e = cudaMemset(S.ks.best_energy + 32 * W, 0, sizeof(int32_t))) != cudaSuccess ||
+        (e = dev_alloc(&S.ks.best_energy, 32 * W + sizeof(GridBarrier) / sizeof(int32_t))) != cudaSuccess ||
+        (S.ks.bar = reinterpret_cast<GridBarrier *>(S.ks.best_energy + 32 * W), false) ||
         (e = dev_alloc(&S.ks.imp, W)) != cudaSuccess ||
-        (e = dev_alloc(&S.ks.bar, 1)) != cudaSuccess ||
         (e = cudaMemsetAsync(S.ks.imp, 0, sizeof(uint32_t) * W, ctx->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(S.ks.bar, 0, sizeof(GridBarrier), ctx->stream)) != cudaSuccess) {
       free_set(S);
@@ -1720,6 +1750,7 @@ int nmc_replicas_reset(nmc_ctx *ctx, int32_t rs, uint64_t seed, const void *init
   if (rc != NMC_OK) return rc;
   DeviceGuard g(ctx->device);
   S->seed = seed;
+  NMC_CUDA(clear_timeout(ctx, *S), "clear wait status");
   return init_replicas(ctx, *I, *S, init_states);
 }
 
@@ -1739,7 +1770,9 @@ int nmc_replicas_restore(nmc_ctx *ctx, int32_t rs, const nmc_result *in) {
   void *dev = nullptr;
   NMC_CUDA(cudaMallocAsync(&dev, 2 * bytes, ctx->stream), "allocate restore staging");
   char *bdev = static_cast<char *>(dev), *sdev = bdev + bytes;
-  cudaError_t e = cudaMemcpyAsync(bdev, in->best_states, bytes, cudaMemcpyHostToDevice, ctx->stream);
+  cudaError_t e = clear_timeout(ctx, *S);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(bdev, in->best_states, bytes, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(sdev, in->states, bytes, cudaMemcpyHostToDevice, ctx->stream);
   // the best states first (their energies become the best energies), then the current states
@@ -2010,7 +2043,6 @@ int nmc_replicas_run_pt(nmc_ctx *ctx, int32_t rs, int32_t t0, int32_t t1,
   const int kq = I->ks.kq;
   int cs = 1, lanes = 0;
   tuned_shape(ctx, *I, W, &cs, &lanes);
-  S->clusters = cs > 1;
   // segments end at t1 or after sweep t with (t+1) % per == 0, where an exchange round follows;
   // their work items are uploaded in chunks
   const int64_t max_chunk_items = std::max<int64_t>(W, 1 << 18);
@@ -2271,7 +2303,6 @@ int nmc_batch_autotune(nmc_ctx *ctx, int32_t n_sets, const int32_t *rs, int32_t 
   for (int32_t i = 0; i < n_sets; ++i) {
     ReplicaSet *S = find_set(ctx, rs[i]);
     Instance *I = find_inst(ctx, S->inst);
-    S->clusters = true;  // trials run every shape
     const size_t W = S->ks.W, n = I->ks.n;
     parts.push_back({S->ks.S, sizeof(uint32_t) * (2 * n + 2) * W});
     parts.push_back({S->ks.best, sizeof(uint32_t) * n * W});
@@ -2663,7 +2694,6 @@ int nmc_adaptive_ladder(nmc_ctx *ctx, int32_t inst, int32_t replicas, uint64_t s
     int max_n[2] = {0, 0}, cs = 1, lanes = 0;
     max_n[q] = n;
     tuned_shape(ctx, *I, W, &cs, &lanes);
-    S->clusters = cs > 1;
     if ((e = fill_schedule(bq, static_cast<size_t>(n) * T, beta, ctx->flag, ctx->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(stats, 0, sizeof(long long) * 64 * W, ctx->stream)) != cudaSuccess) {
       rc = cuda_fail(ctx, e, "prepare ladder level");

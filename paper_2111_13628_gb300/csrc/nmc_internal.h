@@ -34,7 +34,7 @@ constexpr int kMaxQapN = 256;
 // barriers it has passed in its own flag and waits until all flags reach it.
 constexpr int kMaxGridCtas = 1024;
 struct GridBarrier {
-  int sticky;  // set when a wait expired; kept across launches until the host reads it
+  int sticky;  // set when a wait expired (1, kStepTimeout); kept across launches until the host reads it
   int error;   // set when a wait expired; the launch stops early (cleared every launch)
   unsigned int flags[kMaxGridCtas];
 };
@@ -66,9 +66,9 @@ struct KsatReplicas {
   uint32_t *S;        // (2n+2) * W: row 2v = x_v bits, row 2v+1 = not x_v, rows 2n/2n+1 dummy
   uint32_t *best;     // n * W ([var][word]), then n * W of word-major staging for the batched kernel
   int32_t *energy;    // 32W
-  int32_t *best_energy;
+  int32_t *best_energy;  // 32W, then *bar
   uint32_t *imp;      // W: replicas whose best improved at the last sweep end (pending copy)
-  GridBarrier *bar;
+  GridBarrier *bar;   // not an allocation of its own
 };
 
 struct QapDevice {
@@ -131,9 +131,9 @@ cudaError_t quantize_schedule(const float *beta, int32_t n_units, int32_t n_step
                               cudaStream_t st);
 
 // ---- batched k-SAT (batch.cu) -----------------------------------------------------------
-// Left in best_energy[32 W] of a set when a wait between the CTAs of its word gave up, or one of an
-// earlier item of the same cluster had.
-constexpr int32_t kStepTimeout = 1;
+// Left in best_energy[32 W] of a set, which is its bar->sticky, when a wait between the CTAs of its
+// word gave up, or one of an earlier item of the same cluster had.
+constexpr int32_t kStepTimeout = 2;
 // Runs the class barrier of n items (W = 1, best_energy 33 ints each) into a wait of limit_cycles that
 // nothing ends; all of them are marked afterwards.
 cudaError_t step_selftest(const BatchItem *items_dev, int n, long long limit_cycles, cudaStream_t st);
