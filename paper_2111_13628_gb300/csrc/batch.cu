@@ -1313,13 +1313,19 @@ cudaError_t dispatch_batch(int cs, const BatchItem *items, int n_items, int *nex
 
 // Clusters of cs CTAs that run at once, one CTA per SM: clusters do not span a GPC, so this is less
 // than SMs / cs (152 SMs: 76, 36 and 15 clusters of 2, 4 and 8).
+// Asked of `device`, whichever is current; an answer is kept, a failed query (0: no clusters) is not.
 int batch_clusters(int cs, int device) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, int> known;
   std::lock_guard<std::mutex> g(mu);
   const auto it = known.find({cs, device});
   if (it != known.end()) return it->second;
-  int n = 0;
+  int n = 0, prev = -1;
+  if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
+  if (prev != device && cudaSetDevice(device) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   const size_t smem = 128 * 1024;  // more than half of an SM's
   cudaLaunchConfig_t q = {};
   q.blockDim = dim3(kTeamThreads);
@@ -1339,10 +1345,9 @@ int batch_clusters(int cs, int device) {
   };
   const bool ok = cs == 2 ? query(cluster_probe_kernel<2>)
                           : (cs == 4 ? query(cluster_probe_kernel<4>) : query(cluster_probe_kernel<8>));
-  if (!ok) {
-    cudaGetLastError();
-    n = 0;
-  }
+  if (!ok) cudaGetLastError();
+  if (prev >= 0 && prev != device) cudaSetDevice(prev);
+  if (!ok) return 0;
   known[{cs, device}] = n;
   return n;
 }
