@@ -10,6 +10,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <tuple>
 #include <unordered_map>
@@ -494,9 +495,10 @@ namespace {
 // Touches every page of a result buffer that a device-to-host copy is about to fill. A copy into
 // pages that were never written (a caller's fresh array) is several times slower than one into pages
 // that exist (27 MB of LBP results: 23 ms more); done while the GPU still computes, it costs nothing.
-// The contents stay as they are.
+// The contents stay as they are. Small buffers are left alone.
+bool worth_prefault(const void *p, size_t bytes) { return p && bytes >= (1u << 20); }
 void prefault(void *p, size_t bytes) {
-  if (!p || bytes < (1u << 20)) return;
+  if (!worth_prefault(p, bytes)) return;
   volatile char *c = static_cast<volatile char *>(p);
   for (size_t i = 0; i < bytes; i += 4096) c[i] = c[i];
   c[bytes - 1] = c[bytes - 1];
@@ -2478,12 +2480,19 @@ int nmc_cnf_lbp(nmc_ctx *ctx, int32_t inst, int32_t n_seeds, const uint8_t *x_st
   A.deltas = deltas;
   A.n_done = n_done;
   A.overlap = overlap;
-  std::thread touch([&] {  // beside the iterations, which keep this thread busy
-    prefault(marg_out, sizeof(double) * sn);
-    prefault(corr_out, sizeof(double) * S * static_cast<size_t>(m));
-  });
+  const size_t marg_bytes = sizeof(double) * sn, corr_bytes = sizeof(double) * S * static_cast<size_t>(m);
+  std::thread touch;  // beside the iterations, which keep this thread busy
+  if (worth_prefault(marg_out, marg_bytes) || worth_prefault(corr_out, corr_bytes)) {
+    try {
+      touch = std::thread([=] {
+        prefault(marg_out, marg_bytes);
+        prefault(corr_out, corr_bytes);
+      });
+    } catch (const std::system_error &) {  // no thread to be had: the copies touch the pages
+    }
+  }
   const int err = lbp_run(A, ctx->stream);
-  touch.join();
+  if (touch.joinable()) touch.join();
   if (err != 0) return cuda_fail(ctx, static_cast<cudaError_t>(err), "LBP");
   NMC_CUDA(cudaMemcpyAsync(marg_out, marg, sizeof(double) * sn, cudaMemcpyDeviceToHost, ctx->stream), "read marginals");
   if (corr_out)
