@@ -311,6 +311,8 @@ __device__ __forceinline__ FieldRatio field_ratio(const ProductSum &pos, const P
   return up ? FieldRatio{num, big, other} : FieldRatio{-num, other, big};
 }
 
+constexpr int kBatch = 8;  // edges a lane of the variable pass requests together
+
 // Products over the positive and the negated edges of variable v for seed s, always in the same
 // order, whatever the launch: four of each, over every fourth edge, then (0 2)(1 3). LANES = 4: one of
 // the four in each of four consecutive lanes (all get the result); LANES = 1: all in one.
@@ -323,26 +325,26 @@ __device__ __forceinline__ void edge_products(const int32_t *vedge, const int32_
   ProductSum f[2][PER];
 #pragma unroll
   for (int j = 0; j < PER; ++j) f[0][j] = f[1][j] = ProductSum{1.0, 0.0f};
-#pragma unroll (LANES == 1 ? 2 : 8)
-  for (int p = p0 + sub; p < p1; p += 4) {
-    double m[PER];
-    int sign[PER];
+#pragma unroll 1
+  for (int p = p0 + sub; p < p1; p += kBatch * LANES) {
+    double m[kBatch];
+    int sign[kBatch];
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
+    for (int j = 0; j < kBatch; ++j) {
       m[j] = 0.0;
       sign[j] = 0;
-      if (p + j < p1) {
-        const long long e = vedge[p + j];
+      if (p + j * LANES < p1) {
+        const long long e = vedge[p + j * LANES];
         m[j] = msg[e * S + s];
         sign[j] = clits[e] & 1;
       }
     }
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {  // a factor of m = 0 changes nothing
-      ProductSum x = sign[j] ? f[1][j] : f[0][j];
+    for (int j = 0; j < kBatch; ++j) {  // a factor of m = 0 changes nothing
+      ProductSum x = sign[j] ? f[1][j % PER] : f[0][j % PER];
       x.factor(m[j]);
-      f[0][j] = sign[j] ? f[0][j] : x;
-      f[1][j] = sign[j] ? x : f[1][j];
+      f[0][j % PER] = sign[j] ? f[0][j % PER] : x;
+      f[1][j % PER] = sign[j] ? x : f[1][j % PER];
     }
   }
   if constexpr (LANES == 1) {
@@ -392,11 +394,26 @@ __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int3
     double ap, bp, an, bn;
     line(f.top, f.den, f.num, ap, bp);
     line(f.den, f.top, -f.num, an, bn);
-#pragma unroll (LANES == 1 ? 4 : 8)
-    for (int p = p0 + sub; p < p1; p += LANES) {
-      const long long e = vedge[p];
-      const bool sign = clits[e] & 1;
-      E[e * S + s] = fma(sign ? an : ap, msg[e * S + s], sign ? bn : bp);
+#pragma unroll 1
+    for (int p = p0 + sub; p < p1; p += kBatch * LANES) {
+      long long at[kBatch];
+      double m[kBatch];
+      bool sign[kBatch];
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        at[j] = -1;
+        m[j] = 0.0;
+        sign[j] = false;
+        if (p + j * LANES < p1) {
+          const long long e = vedge[p + j * LANES];
+          sign[j] = clits[e] & 1;
+          at[j] = e * S + s;
+          m[j] = msg[at[j]];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j)
+        if (at[j] >= 0) E[at[j]] = fma(sign[j] ? an : ap, m[j], sign[j] ? bn : bp);
     }
   }
 }
@@ -696,7 +713,11 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
   // far as it can there
   const bool prod = A.beta <= 4.0 && A.beta * A.max_deg + A.max_bias < 340.0 &&
                     A.tol >= 2e-15 * exp(2.0 * A.beta);
-  const bool split = (long long)n * S < 152 * 256;  // fewer than eight warps an SM otherwise
+  // four lanes a variable where there would be fewer than eight warps an SM otherwise, in blocks small
+  // enough to reach every SM (5 seeds of 500 variables: 40 blocks of 256 threads, 157 of 64)
+  constexpr int kSplitBlock = 64;
+  const bool split = (long long)n * S < 152 * 256;
+  const unsigned gSplit = (unsigned)((4LL * n * S + kSplitBlock - 1) / kSplitBlock);
   const float slack = (float)((exp(2.0 * A.beta) + 8.0) * 0x1p-21);
   const auto clause = [&](const int32_t *seeds, int track) {
     if (!prod) {
@@ -731,8 +752,8 @@ int lbp_run(const LbpArgs &A, cudaStream_t st) {
     // alone), and the GPU does not wait for the host in between.
     for (int32_t it = 0; it < A.max_iter; ++it) {
       if (prod && split)
-        lbp_var_prod_kernel<4><<<blocks_for(4LL * n * S), kLbpBlock, 0, st>>>(
-            A.vptr, A.vedge, A.clits, n, S, bias, u, h, status);
+        lbp_var_prod_kernel<4><<<gSplit, kSplitBlock, 0, st>>>(A.vptr, A.vedge, A.clits, n, S, bias, u, h,
+                                                             status);
       else if (prod)
         lbp_var_prod_kernel<1><<<gVS, kLbpBlock, 0, st>>>(A.vptr, A.vedge, A.clits, n, S, bias, u, h,
                                                           status);
