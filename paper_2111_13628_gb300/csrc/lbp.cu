@@ -25,6 +25,9 @@
 // to 5,000 variables at beta = 1: 0.90 marginals, 0.99 correlations (root mean square 0.84, 0.86); 36
 // sparser inputs at beta = 4: 0.85, 0.97; without a bias at beta = 1e-3: 0.46, 0.92. With 1 - m, E and
 // plain products kept instead: 1.08, 1.11 at beta = 1 and 440 without a bias at beta = 1e-3.
+//
+// 4-SAT, 5,000 variables, 64 seeds: clause pass 1,920 -> 149 us, variable pass 120 -> 141, a call with
+// its backbones 122 -> 26.4 ms (22.8 with the plain products); 500 variables, 5 seeds: 5.6 -> 2.8 ms.
 #include <math.h>
 
 #include "nmc_internal.h"
@@ -311,7 +314,9 @@ __device__ __forceinline__ FieldRatio field_ratio(const ProductSum &pos, const P
   return up ? FieldRatio{num, big, other} : FieldRatio{-num, other, big};
 }
 
-constexpr int kBatch = 8;  // edges a lane of the variable pass requests together
+// Edges a lane of the variable pass requests together (with one lane a variable other warps hide the
+// latency: eight at a time 143 us a pass instead of 141, 64 seeds of 5,000 variables).
+__host__ __device__ constexpr int edge_batch(int lanes) { return lanes == 1 ? 4 : 8; }
 
 // Products over the positive and the negated edges of variable v for seed s, always in the same
 // order, whatever the launch: four of each, over every fourth edge, then (0 2)(1 3). LANES = 4: one of
@@ -320,17 +325,17 @@ template <int LANES>
 __device__ __forceinline__ void edge_products(const int32_t *vedge, const int32_t *clits, int p0,
                                               int p1, int S, int s, const double *msg,
                                               ProductSum &pos, ProductSum &neg) {
-  constexpr int PER = 4 / LANES;
+  constexpr int PER = 4 / LANES, BATCH = edge_batch(LANES);
   const int sub = LANES == 1 ? 0 : (int)threadIdx.x % LANES;
   ProductSum f[2][PER];
 #pragma unroll
   for (int j = 0; j < PER; ++j) f[0][j] = f[1][j] = ProductSum{1.0, 0.0f};
-#pragma unroll 1
-  for (int p = p0 + sub; p < p1; p += kBatch * LANES) {
-    double m[kBatch];
-    int sign[kBatch];
+#pragma unroll (LANES == 1 ? 2 : 1)
+  for (int p = p0 + sub; p < p1; p += BATCH * LANES) {
+    double m[BATCH];
+    int sign[BATCH];
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) {
+    for (int j = 0; j < BATCH; ++j) {
       m[j] = 0.0;
       sign[j] = 0;
       if (p + j * LANES < p1) {
@@ -340,7 +345,7 @@ __device__ __forceinline__ void edge_products(const int32_t *vedge, const int32_
       }
     }
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) {  // a factor of m = 0 changes nothing
+    for (int j = 0; j < BATCH; ++j) {  // a factor of m = 0 changes nothing
       ProductSum x = sign[j] ? f[1][j % PER] : f[0][j % PER];
       x.factor(m[j]);
       f[0][j % PER] = sign[j] ? f[0][j % PER] : x;
@@ -394,13 +399,14 @@ __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int3
     double ap, bp, an, bn;
     line(f.top, f.den, f.num, ap, bp);
     line(f.den, f.top, -f.num, an, bn);
+    constexpr int BATCH = edge_batch(LANES);
 #pragma unroll 1
-    for (int p = p0 + sub; p < p1; p += kBatch * LANES) {
-      long long at[kBatch];
-      double m[kBatch];
-      bool sign[kBatch];
+    for (int p = p0 + sub; p < p1; p += BATCH * LANES) {
+      long long at[BATCH];
+      double m[BATCH];
+      bool sign[BATCH];
 #pragma unroll
-      for (int j = 0; j < kBatch; ++j) {
+      for (int j = 0; j < BATCH; ++j) {
         at[j] = -1;
         m[j] = 0.0;
         sign[j] = false;
@@ -412,7 +418,7 @@ __global__ void lbp_var_prod_kernel(const int32_t *__restrict__ vptr, const int3
         }
       }
 #pragma unroll
-      for (int j = 0; j < kBatch; ++j)
+      for (int j = 0; j < BATCH; ++j)
         if (at[j] >= 0) E[at[j]] = fma(sign[j] ? an : ap, m[j], sign[j] ? bn : bp);
     }
   }

@@ -78,3 +78,18 @@ def test_converged_near_the_limit(k, alpha, beta):
     x = (W.splitmix64(92, 3 * n) & np.uint64(1)).astype(np.uint8).reshape(3, n)
     want = _run(lits, n, x, beta, [0.4, 0.2], 1e-8, 60, np.full(n, 0.5))
     assert all(w["n_done"] == 2 for w in want)
+
+
+@pytest.mark.parametrize("k,alpha", [(2, 1.2), (3, 3.0), (4, 4.0)])
+@pytest.mark.parametrize("beta,bias", [(0.5, 320.0), (1.0, 300.0), (4.0, 150.0), (2.0, 18.0)])
+def test_fields_near_the_end_of_the_range(k, alpha, beta, bias):
+    """|field| up to just below 340, where e^{+-2 field} and products of 1 - m reach the ends of what the
+    product form holds; every third variable without a bias."""
+    n = 150
+    lits = W.random_ksat(n, alpha, k, 97)
+    assert beta * np.bincount(np.abs(lits).reshape(-1) - 1).max() + bias < 340.0
+    x = (W.splitmix64(98, 3 * n) & np.uint64(1)).astype(np.uint8).reshape(3, n)
+    eps = np.full(n, bias)
+    eps[::3] = 0.0
+    eps[1::3] *= np.linspace(-1.0, 1.0, len(eps[1::3]))
+    _run(lits, n, x, beta, [1.0, 0.5], 1e-8, 4, eps)
